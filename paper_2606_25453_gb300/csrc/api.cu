@@ -558,13 +558,15 @@ emu_status_t run_scheme_I(emu_handle_s* h, const View& v, int64_t k, int p, doub
   auto* hatB = reinterpret_cast<int8_t*>(ws + pl.off_hatB);
   const T* A = static_cast<const T*>(v.A);
   const T* B = static_cast<const T*>(v.B);
-  trace_begin(h, PH_SCAN, st);
-  launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, 1, maxA, h->status, st);
-  launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
-  trace_end(h, PH_SCAN, st, 2);
+  if (!v.maxA) {
+    trace_begin(h, PH_SCAN, st);
+    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, 1, maxA, h->status, st);
+    launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+    trace_end(h, PH_SCAN, st, 2);
+  }
   trace_begin(h, PH_SPLIT, st);
-  launch_split_I<T>(A, v.ldA, v.a_kcontig, v.M, k, p, maxA, hatA, EA, st, f8);
-  launch_split_I<T>(B, v.ldB, v.b_kcontig, v.N, k, p, maxB, hatB, FB, st, f8);
+  launch_split_I<T>(A, v.ldA, v.a_kcontig, v.M, k, p, v.maxA ? v.maxA : maxA, hatA, EA, st, f8);
+  launch_split_I<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, hatB, FB, st, f8);
   trace_end(h, PH_SPLIT, st, 2);
   return scheme_I_gemm(h, hatA, pl.rows_a, hatB, pl.rows_b, pl.cols, v.M, v.N, k, p, EA, FB, alpha, beta, C, ldc,
                        out_mode, partials, st, f8);
@@ -649,20 +651,22 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   host_crt_tables(nm, &ct);
   const bool do_a = phase != 1, do_b = phase != 2;
   trace_begin(h, PH_SCAN, st);
-  if (do_a) launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, maxA, h->status, st);
-  if (do_b) launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, maxB, h->status, st);
+  const unsigned long long* mA = v.maxA ? v.maxA : maxA;
+  const unsigned long long* mB = v.maxB ? v.maxB : maxB;
+  if (do_a && !v.maxA) launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, maxA, h->status, st);
+  if (do_b && !v.maxB) launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, maxB, h->status, st);
   if (norm && do_a)
-    launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, maxA, reinterpret_cast<unsigned long long*>(ws + pl.off_accA),
+    launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, mA, reinterpret_cast<unsigned long long*>(ws + pl.off_accA),
                    nEA, st);
   if (norm && do_b)
-    launch_norm<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, maxB, reinterpret_cast<unsigned long long*>(ws + pl.off_accB),
+    launch_norm<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, mB, reinterpret_cast<unsigned long long*>(ws + pl.off_accB),
                    nEB, st);
   trace_end(h, PH_SCAN, st, (do_a + do_b) * (norm ? 3 : 1));
   trace_begin(h, PH_SPLIT, st);
   if (do_a)
-    launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, maxA, resA, EA, st, norm ? nEA : nullptr, tc);
+    launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, mA, resA, EA, st, norm ? nEA : nullptr, tc);
   if (do_b)
-    launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, maxB, resB, FB, st, norm ? nEB : nullptr, tc);
+    launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, mB, resB, FB, st, norm ? nEB : nullptr, tc);
   trace_end(h, PH_SPLIT, st, do_a + do_b);
   if (phase == 1) return cuda_err(cudaGetLastError());
   CUtensorMap ta, tb;
@@ -780,12 +784,15 @@ template <typename T>
 static emu_status_t real_gemm(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n, int64_t k,
                               double alpha, const T* A, int64_t lda, const T* B, int64_t ldb,
                               double beta, T* C, int64_t ldc, emu_scheme_t scheme, int p_or_nm,
-                              emu_stream_t stream) {
+                              emu_stream_t stream, const unsigned long long* maxA = nullptr,
+                              const unsigned long long* maxB = nullptr) {
   emu_status_t s = gemm_common(h, layout, m, n, k, A, lda, B, ldb, C, ldc, scheme, p_or_nm);
   if (s != EMU_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   View v;
   normalize(layout, m, n, A, lda, B, ldb, &v);
+  v.maxA = maxA;
+  v.maxB = maxB;
   if (v.M == 0 || v.N == 0) return EMU_OK;
   if (k == 0) {
     launch_scale_c<T>(C, ldc, v.M, v.N, beta, st);
@@ -797,6 +804,14 @@ static emu_status_t real_gemm(emu_handle_t h, emu_layout_t layout, int64_t m, in
                            st, nullptr, scheme == EMU_SCHEME_I_F8);
   return run_scheme_II<T>(h, v, k, p_or_nm, 1, alpha, 0.0, beta, 0.0, C, ldc, out == 0 ? II_F64 : II_F32,
                           nullptr, st, scheme == EMU_SCHEME_II_NORM);
+}
+
+emu_status_t emu::dgemm_scanned(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n, int64_t k, double alpha,
+                                const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
+                                emu_scheme_t scheme, int p_or_nm, const unsigned long long* maxA,
+                                const unsigned long long* maxB, emu_stream_t stream) {
+  return real_gemm<double>(h, layout, m, n, k, alpha, A, lda, B, ldb, 0.0, C, ldc, scheme, p_or_nm, stream, maxA,
+                           maxB);
 }
 
 extern "C" {

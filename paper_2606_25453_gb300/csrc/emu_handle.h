@@ -42,6 +42,10 @@ struct View {
   const void* B;
   int64_t ldB;
   bool b_kcontig;
+  // the largest |x| (IEEE bits) of every row of A and column of B, if the
+  // caller scanned them already
+  const unsigned long long* maxA = nullptr;
+  const unsigned long long* maxB = nullptr;
 };
 void normalize(emu_layout_t layout, int64_t m, int64_t n, const void* A, int64_t lda, const void* B,
                int64_t ldb, View* v);
@@ -70,6 +74,13 @@ emu_status_t scheme_I_gemm(emu_handle_s* h, const int8_t* hatA, int64_t rows_a, 
                            int64_t cols, int64_t M, int64_t N, int64_t k, int p, const int32_t* EA,
                            const int32_t* FB, double alpha, double beta, void* C, int64_t ldc, int out_mode,
                            int32_t* partials, cudaStream_t st, bool f8);
+
+// emu_dgemm with beta = 0 on operands whose row and column maxima are already
+// known (maxA, maxB: View's, in the row-major view's order).
+emu_status_t dgemm_scanned(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n, int64_t k, double alpha,
+                           const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
+                           emu_scheme_t scheme, int p_or_nm, const unsigned long long* maxA,
+                           const unsigned long long* maxB, emu_stream_t stream);
 
 // C = beta * C for products with k == 0 (beta == 0 writes zeros, C is not read).
 template <typename T>

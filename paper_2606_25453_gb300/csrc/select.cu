@@ -12,8 +12,12 @@
 #include <cstring>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "emu_handle.h"
 #include "emu_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace emu {
 
@@ -29,17 +33,17 @@ struct SelState {
   bool loaded = false;
   float* params_II = nullptr;  // Scheme II, norm scaling: classes N = 6, 8, .., 20
   bool loaded_II = false;
-  // auto-precision buffers, grown on demand: device [feat 128 | prob 8 |
-  // probe idx | probe results], and a pinned host copy of the parts read
-  // back, so that each decision costs one device-to-host copy
+  // auto-precision buffers, grown on demand (layout: auto_impl): device
+  // memory, and pinned host memory that the kernels write their few results
+  // into
   uint8_t* dev = nullptr;
   size_t dev_bytes = 0;
   uint8_t* host = nullptr;
   size_t host_bytes = 0;
-  // side stream for the probe's reference sums (they depend on A and B
-  // only, so they run beside the feature pass and the product)
+  // side stream for the decision and the probe's reference sums (they depend
+  // on A and B only, so they run beside the scan and the product)
   cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_probe = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_decide = nullptr, ev_probe = nullptr;
 };
 SelState* sel_of(emu_handle_s* h) {
   if (!h->selector) h->selector = new SelState();
@@ -64,8 +68,37 @@ struct FeatOperand {
   bool kcontig;
   int64_t rows, stride;
 };
-__global__ void feat_hist_kernel(FeatOperand oa, FeatOperand ob, int nblk_a, int64_t k,
-                                 unsigned int* __restrict__ hist_all) {
+// The block that finishes last turns the histograms into the features and,
+// with a network loaded (prm), its class probabilities: one launch decides.
+// It is latency bound (a few microseconds of dependent loads), so there is no
+// second and third kernel, and the results go straight to `out` (feat[128 |
+// prob], pinned host memory in the auto entry points, beside the device copy
+// `feat`), which spares the copy back.  The histograms and the counter are
+// zero before and after the launch.
+struct FeatDecide {
+  unsigned int* done;  // blocks-finished counter
+  float log2k_16, ltol_16;
+  const float* prm;  // null: features only
+  float* feat;       // device, 66 floats
+  float* out;        // null: no second copy; else features at 0, probabilities at 128
+};
+__device__ void feat_decide(const FeatDecide& d, unsigned int* hist, float* sm);
+// Slot of parameter i in the decision's shared copy.
+constexpr int kDecP = kHid + 1 + (kIn - kHid);  // padded row of W1 and W2 (67 floats)
+constexpr int kDecW2 = kHid * kDecP, kDecW3 = 2 * kHid * kDecP, kDecB = kDecW3 + kOut * kDecP;
+constexpr int kDecFloats = kDecB + 2 * kHid + kOut;
+__device__ __forceinline__ int dec_slot(int i) {
+  if (i < kOffB1) return (i / kIn) * kDecP + i % kIn;
+  if (i < kOffW2) return kDecB + i - kOffB1;
+  if (i < kOffB2) return kDecW2 + ((i - kOffW2) / kHid) * kDecP + (i - kOffW2) % kHid;
+  if (i < kOffW3) return kDecB + kHid + i - kOffB2;
+  if (i < kOffB3) return kDecW3 + ((i - kOffW3) / kHid) * kDecP + (i - kOffW3) % kHid;
+  return kDecB + 2 * kHid + i - kOffB3;
+}
+
+__global__ void __launch_bounds__(256) feat_hist_kernel(FeatOperand oa, FeatOperand ob, int nblk_a, int64_t k,
+                                                        unsigned int* __restrict__ hist_all, FeatDecide dec) {
+  extern __shared__ float dyn[];  // the network, in the last block
   __shared__ unsigned int sh[32];
   __shared__ unsigned long long shmax;
   if (threadIdx.x < 32) sh[threadIdx.x] = 0;
@@ -101,26 +134,82 @@ __global__ void feat_hist_kernel(FeatOperand oa, FeatOperand ob, int nblk_a, int
         int d = E - exp_bits(ab);
         bin = d < 0 ? 0 : (d / 3 > 31 ? 31 : d / 3);
       }
-      atomicAdd(&sh[bin], 1u);
+      // most elements of a vector share a few bins: one add per warp and bin
+      const unsigned same = __match_any_sync(__activemask(), bin);
+      if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&sh[bin], static_cast<unsigned>(__popc(same)));
     }
   }
   __syncthreads();
   if (threadIdx.x < 32 && sh[threadIdx.x]) atomicAdd(&hist[threadIdx.x], sh[threadIdx.x]);
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(dec.done, 1u) + 1 == gridDim.x;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  feat_decide(dec, hist_all, dyn);
 }
 
-__global__ void feat_finalize_kernel(const unsigned int* __restrict__ hist, double log2k, double ltol,
-                                     float* __restrict__ feat) {
-  int t = threadIdx.x;
-  __shared__ float tot[2];
+// The last block (256 threads) of feat_hist_kernel.
+__device__ void feat_decide(const FeatDecide& d, unsigned int* hist, float* sm) {
+  __shared__ unsigned int hs[64];
+  __shared__ float x[kIn + 2], h1[kHid], h2[kHid], z[kOut], tot[2];
+  const int t = threadIdx.x;
+  // rows of the weight matrices are padded to an odd length, so that 64
+  // neurons read 32 different banks
+  if (d.prm)
+    for (int i = t; i < kNParam; i += 256) sm[dec_slot(i)] = __ldg(d.prm + i);
+  if (t < 64) {
+    hs[t] = __ldcg(hist + t);
+    hist[t] = 0;
+  }
+  if (t == 64) *d.done = 0;
+  __syncthreads();
   if (t < 2) {
     unsigned int s = 0;
-    for (int i = 0; i < 32; ++i) s += hist[t * 32 + i];
+    for (int i = 0; i < 32; ++i) s += hs[t * 32 + i];
     tot[t] = s ? static_cast<float>(s) : 1.0f;
   }
   __syncthreads();
-  if (t < 64) feat[t] = static_cast<float>(hist[t]) / tot[t / 32];
-  if (t == 64) feat[64] = static_cast<float>(log2k / 16.0);
-  if (t == 65) feat[65] = static_cast<float>(ltol / 16.0);
+  if (t < kIn) {
+    const float f = t < 64 ? static_cast<float>(hs[t]) / tot[t / 32] : t == 64 ? d.log2k_16 : d.ltol_16;
+    x[t] = f;
+    d.feat[t] = f;
+    if (d.out) d.out[t] = f;
+  }
+  if (!d.prm) return;
+  __syncthreads();
+  // the arithmetic of mlp_forward_kernel, in its order
+  float s = 0.f;
+  if (t < kHid) {
+    s = sm[kDecB + t];
+#pragma unroll 11
+    for (int i = 0; i < kIn; ++i) s = fmaf(sm[t * kDecP + i], x[i], s);
+    h1[t] = s > 0.f ? s : 0.f;
+  }
+  __syncthreads();
+  if (t < kHid) {
+    s = sm[kDecB + kHid + t];
+#pragma unroll 16
+    for (int i = 0; i < kHid; ++i) s = fmaf(sm[kDecW2 + t * kDecP + i], h1[i], s);
+    h2[t] = s > 0.f ? s : 0.f;
+  }
+  __syncthreads();
+  if (t < kOut) {
+    s = sm[kDecB + 2 * kHid + t];
+#pragma unroll 16
+    for (int i = 0; i < kHid; ++i) s = fmaf(sm[kDecW3 + t * kDecP + i], h2[i], s);
+    z[t] = s;
+  }
+  __syncthreads();
+  if (t < kOut) {
+    float mx = z[0];
+    for (int o = 1; o < kOut; ++o) mx = fmaxf(mx, z[o]);
+    float den = 0.f;
+    for (int o = 0; o < kOut; ++o) den += expf(z[o] - mx);
+    d.out[128 + t] = expf(z[t] - mx) / den;
+  }
 }
 
 // ---------------------------------------------------------------- MLP
@@ -232,27 +321,32 @@ __device__ __forceinline__ DD dd_add(DD a, DD b) {
   return {t, __dsub_rn(e, __dsub_rn(t, s))};
 }
 
-// One block of kProbeThreads per sampled entry (i, j): compensated dot
-// product (TwoProduct by fma, TwoSum accumulation) per thread over a strided
-// share of K, threads combined by double-double adds (warp shuffles, then
-// the warps' partial results through shared memory).  A block per entry
-// keeps many independent loads in flight: one warp walking all of K waited
-// on one strided load per step.
-constexpr int kProbeThreads = 256;
-__global__ void __launch_bounds__(kProbeThreads) probe_dd_kernel(const double* __restrict__ A, int64_t lda,
-                                                                bool a_kcontig, const double* __restrict__ B,
-                                                                int64_t ldb, bool b_kcontig, int64_t k, int count,
-                                                                const int32_t* __restrict__ idx,
-                                                                double* __restrict__ ref, double* __restrict__ absab) {
-  __shared__ double sh[3][kProbeThreads / 32];
-  const int w = blockIdx.x, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  if (w >= count) return;
+// Per sampled entry (i, j) a cluster of eight one-warp blocks: compensated
+// dot product (TwoProduct by fma, TwoSum accumulation) per thread over a
+// strided share of K (256 threads per entry), threads combined by
+// double-double adds (warp shuffles, then the warps' partial results through
+// the first block's shared memory).  FP64 issue bounds it (two results per
+// clock and SM), and it runs beside the product whose persistent GEMM wants
+// every SM: eight warps of one block on each of 64 SMs held those SMs back,
+// 64 x 8 single warps spread over the whole GPU do not.
+constexpr int kProbeWarps = 8, kProbeThreads = 32 * kProbeWarps;
+__global__ void __cluster_dims__(kProbeWarps, 1, 1) __launch_bounds__(32)
+    probe_dd_kernel(const double* __restrict__ A, int64_t lda, bool a_kcontig, const double* __restrict__ B,
+                    int64_t ldb, bool b_kcontig, int64_t k, int count, const int32_t* __restrict__ idx,
+                    double* __restrict__ ref, double* __restrict__ absab) {
+  __shared__ double sh[3][kProbeWarps];
+  cg::cluster_group cl = cg::this_cluster();
+  const int w = blockIdx.x / kProbeWarps, lane = threadIdx.x, wp = blockIdx.x % kProbeWarps;
   const int64_t i = idx[2 * w], j = idx[2 * w + 1];
+  const double* const pa = a_kcontig ? A + i * lda : A + i;
+  const double* const pb = b_kcontig ? B + j * ldb : B + j;
+  const int64_t sa = a_kcontig ? 1 : lda, sb = b_kcontig ? 1 : ldb;
   DD acc{0.0, 0.0};
   double ab = 0.0;
-  for (int64_t h = threadIdx.x; h < k; h += kProbeThreads) {
-    const double a = a_kcontig ? A[i * lda + h] : A[h * lda + i];
-    const double b = b_kcontig ? B[j * ldb + h] : B[h * ldb + j];
+#pragma unroll 4
+  for (int64_t h = wp * 32 + lane; h < k; h += kProbeThreads) {
+    const double a = __ldg(pa + h * sa);
+    const double b = __ldg(pb + h * sb);
     const double p = __dmul_rn(a, b);
     const double e = __fma_rn(a, b, -p);
     acc = dd_add(acc, DD{p, e});
@@ -263,16 +357,18 @@ __global__ void __launch_bounds__(kProbeThreads) probe_dd_kernel(const double* _
     acc = dd_add(acc, other);
     ab = __dadd_rn(ab, __shfl_xor_sync(0xffffffffu, ab, o));
   }
+  cl.sync();  // the first block runs: its shared memory may be written
   if (lane == 0) {
-    sh[0][wp] = acc.hi;
-    sh[1][wp] = acc.lo;
-    sh[2][wp] = ab;
+    double* dst = cl.map_shared_rank(&sh[0][0], 0);
+    dst[wp] = acc.hi;
+    dst[kProbeWarps + wp] = acc.lo;
+    dst[2 * kProbeWarps + wp] = ab;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  cl.sync();
+  if (wp == 0 && lane == 0) {
     DD t{sh[0][0], sh[1][0]};
     double tab = sh[2][0];
-    for (int q = 1; q < kProbeThreads / 32; ++q) {
+    for (int q = 1; q < kProbeWarps; ++q) {
       t = dd_add(t, DD{sh[0][q], sh[1][q]});
       tab = __dadd_rn(tab, sh[2][q]);
     }
@@ -282,19 +378,30 @@ __global__ void __launch_bounds__(kProbeThreads) probe_dd_kernel(const double* _
   }
 }
 
-// idx pairs (i, j) -> (j, i), for gathering entries of a column-major C.
-__global__ void swap_pairs_kernel(const int32_t* __restrict__ idx, int count, int32_t* __restrict__ out) {
-  int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w < count) {
-    out[2 * w] = idx[2 * w + 1];
-    out[2 * w + 1] = idx[2 * w];
+// Probe entries: a deterministic spread over C (caller's coordinates), the
+// xorshift sequence from the shape.
+__global__ void probe_idx_kernel(uint64_t x, int64_t m, int64_t n, int count, int32_t* __restrict__ idx) {
+  for (int q = 0; q < 2 * count; ++q) {
+    x ^= x << 13;
+    x ^= x >> 7;
+    x ^= x << 17;
+    idx[q] = static_cast<int32_t>(x % static_cast<uint64_t>(q & 1 ? n : m));
   }
 }
 
-__global__ void gather_kernel(const double* __restrict__ C, int64_t ldc, int count, const int32_t* __restrict__ idx,
-                              double* __restrict__ out) {
-  int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w < count) out[w] = C[static_cast<int64_t>(idx[2 * w]) * ldc + idx[2 * w + 1]];
+// The probed entries of C with their reference sums, to pinned host memory:
+// out = [ref (hi, lo) | sum |a||b| | C entry], `count` of each.  idx holds
+// the caller's (i, j); colmajor: C's rows are the caller's columns.
+__global__ void judge_kernel(const double* __restrict__ C, int64_t ldc, bool colmajor, int count,
+                             const int32_t* __restrict__ idx, const double* __restrict__ ref,
+                             const double* __restrict__ ab, double* __restrict__ out) {
+  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  if (w >= count) return;
+  const int64_t i = idx[2 * w], j = idx[2 * w + 1];
+  out[2 * w] = ref[2 * w];
+  out[2 * w + 1] = ref[2 * w + 1];
+  out[2 * static_cast<int64_t>(count) + w] = ab[w];
+  out[3 * static_cast<int64_t>(count) + w] = C[colmajor ? j * ldc + i : i * ldc + j];
 }
 
 }  // namespace
@@ -308,6 +415,7 @@ void selector_release(emu_handle_s* h) {
   if (s->host) cudaFreeHost(s->host);
   if (s->side) cudaStreamDestroy(s->side);
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
+  if (s->ev_decide) cudaEventDestroy(s->ev_decide);
   if (s->ev_probe) cudaEventDestroy(s->ev_probe);
   delete s;
   h->selector = nullptr;
@@ -319,12 +427,14 @@ using namespace emu;
 
 namespace {
 
-// Features of one product into feat (device float[66]); needs 8*(m+n)+256
-// bytes of scratch (maxbits + histogram).
-emu_status_t features_impl(emu_handle_s* h, const View& v, int64_t k, double tol, int64_t sample, float* feat,
-                           uint8_t* scratch, cudaStream_t st) {
+// Features of one product into feat (device float[66]); needs feat_scratch
+// bytes of scratch (histograms and the blocks-finished counter; zeroed: they
+// are zero already, as an earlier call leaves them).  prm: also
+// the network's class probabilities; out: see FeatDecide.
+emu_status_t features_impl(const View& v, int64_t k, double tol, int64_t sample, float* feat, uint8_t* scratch,
+                           cudaStream_t st, bool zeroed = false, const float* prm = nullptr, float* out = nullptr) {
   auto* hist = reinterpret_cast<unsigned int*>(scratch);
-  cudaMemsetAsync(hist, 0, 64 * sizeof(unsigned int), st);
+  if (!zeroed) cudaMemsetAsync(hist, 0, 65 * sizeof(unsigned int), st);
   int64_t sa = sample > 0 ? std::max<int64_t>(1, v.M / sample) : 1;
   int64_t sb = sample > 0 ? std::max<int64_t>(1, v.N / sample) : 1;
   int64_t na = (v.M + sa - 1) / sa, nb = (v.N + sb - 1) / sb;
@@ -334,8 +444,10 @@ emu_status_t features_impl(emu_handle_s* h, const View& v, int64_t k, double tol
   }
   const FeatOperand oa{static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, sa};
   const FeatOperand ob{static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, sb};
-  feat_hist_kernel<<<static_cast<unsigned>(na + nb), 256, 0, st>>>(oa, ob, static_cast<int>(na), k, hist);
-  feat_finalize_kernel<<<1, 96, 0, st>>>(hist, std::log2(static_cast<double>(k)), -std::log10(tol), feat);
+  const FeatDecide dec{hist + 64, static_cast<float>(std::log2(static_cast<double>(k)) / 16.0),
+                       static_cast<float>(-std::log10(tol) / 16.0), prm, feat, out};
+  feat_hist_kernel<<<static_cast<unsigned>(na + nb), 256, prm ? kDecFloats * sizeof(float) : 0, st>>>(
+      oa, ob, static_cast<int>(na), k, hist, dec);
   return cudaGetLastError() == cudaSuccess ? EMU_OK : EMU_ERR_CUDA;
 }
 
@@ -390,7 +502,7 @@ emu_status_t bound_impl(emu_handle_s* h, emu_layout_t layout, int64_t m, int64_t
   emu_status_t s = handle_workspace(h, need, st, &ws);
   if (s != EMU_OK) return s;
   float* feat = reinterpret_cast<float*>(ws + feat_scratch(v));
-  s = features_impl(h, v, k, tol, 64, feat, ws, st);
+  s = features_impl(v, k, tol, 64, feat, ws, st);
   if (s != EMU_OK) return s;
   float f[kIn];
   if (cudaMemcpyAsync(f, feat, sizeof(f), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -417,7 +529,7 @@ emu_status_t emu_sel_features(emu_handle_t h, emu_layout_t layout, int64_t m, in
   uint8_t* ws = nullptr;
   emu_status_t s = handle_workspace(h, feat_scratch(v), st, &ws);
   if (s != EMU_OK) return s;
-  return features_impl(h, v, k, tol, sample, feat, ws, st);
+  return features_impl(v, k, tol, sample, feat, ws, st);
 }
 
 emu_status_t emu_sel_forward(emu_handle_t h, int64_t batch, const float* prm, const float* X, float* P, float* act,
@@ -490,7 +602,7 @@ emu_status_t emu_probe_dd(emu_handle_t h, emu_layout_t layout, int64_t m, int64_
   // entries are given in the caller's (i, j) of C; the kernel reads A rows
   // and B columns directly in the caller's layout
   bool a_k = layout == EMU_ROW_MAJOR, b_k = layout != EMU_ROW_MAJOR;
-  probe_dd_kernel<<<count, kProbeThreads, 0, static_cast<cudaStream_t>(stream)>>>(A, lda, a_k, B, ldb, b_k, k,
+  probe_dd_kernel<<<count * kProbeWarps, 32, 0, static_cast<cudaStream_t>(stream)>>>(A, lda, a_k, B, ldb, b_k, k,
                                                                                  count, idx, ref, absab);
   return cudaGetLastError() == cudaSuccess ? EMU_OK : EMU_ERR_CUDA;
 }
@@ -521,13 +633,15 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
   SelState* ss = sel_of(h);
   View v;
   normalize(layout, m, n, A, lda, B, ldb, &v);
-  // selector buffers: features and probabilities (136 floats), then the
-  // probe's indices, its results [ref (hi, lo) | sum |a||b| | C entry], and
-  // the swapped index pairs of a column-major gather
+  // device: features | histograms | probe indices | probe results [ref (hi,
+  // lo) | sum |a||b|] | row and column maxima; pinned host memory:
+  // features, probabilities | probe results with the C entries
   const int pc = std::max(probe, 1);
-  const size_t off_idx = 1024, off_res = off_idx + (8 * static_cast<size_t>(pc) + 255) / 256 * 256;
-  const size_t dev_need = off_res + 40 * static_cast<size_t>(pc);
-  const size_t host_need = std::max<size_t>(1024, 32 * static_cast<size_t>(pc));
+  const size_t idx_bytes = (8 * static_cast<size_t>(pc) + 255) / 256 * 256;
+  const size_t off_hist = 1024, off_idx = off_hist + feat_scratch(v), off_res = off_idx + idx_bytes;
+  const size_t off_max = off_res + (24 * static_cast<size_t>(pc) + 255) / 256 * 256;
+  const size_t dev_need = off_max + 8 * static_cast<size_t>(v.M + v.N);
+  const size_t host_need = 1024 + 32 * static_cast<size_t>(pc);
   if (dev_need > ss->dev_bytes) {
     if (ss->dev) cudaFree(ss->dev);
     ss->dev = nullptr;
@@ -536,6 +650,8 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
       cudaGetLastError();
       return EMU_ERR_ALLOC;
     }
+    // the decision's histograms start, and are left, at zero
+    if (cudaMemset(ss->dev, 0, off_idx) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return EMU_ERR_CUDA;
     ss->dev_bytes = dev_need;
   }
   if (host_need > ss->host_bytes) {
@@ -548,60 +664,43 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
     }
     ss->host_bytes = host_need;
   }
-  float* feat = reinterpret_cast<float*>(ss->dev);
-  float* prob = feat + 128;
-  // probe entries: a deterministic spread over C (caller's coordinates),
-  // uploaded once for every attempt (row-major view: (i, j); column-major C:
-  // element (i, j) sits at row j, column i of the row-major view); their
-  // double-double reference sums depend on A and B only, so they run on a
-  // side stream beside the feature pass and the product
+  if (!ss->side && (cudaStreamCreateWithFlags(&ss->side, cudaStreamNonBlocking) != cudaSuccess ||
+                    cudaEventCreateWithFlags(&ss->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+                    cudaEventCreateWithFlags(&ss->ev_decide, cudaEventDisableTiming) != cudaSuccess ||
+                    cudaEventCreateWithFlags(&ss->ev_probe, cudaEventDisableTiming) != cudaSuccess))
+    return EMU_ERR_CUDA;
   auto* d_idx = reinterpret_cast<int32_t*>(ss->dev + off_idx);
   auto* d_ref = reinterpret_cast<double*>(ss->dev + off_res);
   auto* d_ab = d_ref + 2 * pc;
-  auto* d_c = d_ab + pc;
-  auto* d_sw = reinterpret_cast<int32_t*>(d_c + pc);  // gather indices for column-major C
+  auto* maxA = reinterpret_cast<unsigned long long*>(ss->dev + off_max);
+  auto* maxB = maxA + v.M;
+  auto* h_dec = reinterpret_cast<float*>(ss->host);
+  auto* h_res = reinterpret_cast<double*>(ss->host + 1024);
+  const bool loaded = scheme_II ? ss->loaded_II : ss->loaded;
+  // The decision (features and network, on sampled vectors) and then the
+  // probe's double-double reference sums run on the side stream; the
+  // exponent scan of the whole operands, which every attempt's product needs
+  // whatever p it uses, runs beside them on the caller's stream, so that the
+  // host waits for the decision while the GPU scans.
+  if (cudaEventRecord(ss->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ss->side, ss->ev_fork, 0) != cudaSuccess)
+    return EMU_ERR_CUDA;
+  emu_status_t s = features_impl(v, k, tol, 64, reinterpret_cast<float*>(ss->dev), ss->dev + off_hist, ss->side,
+                                 true, loaded ? (scheme_II ? ss->params_II : ss->params) : nullptr, h_dec);
+  if (s != EMU_OK) return s;
+  if (cudaEventRecord(ss->ev_decide, ss->side) != cudaSuccess) return EMU_ERR_CUDA;
+  trace_begin(h, PH_SCAN, st);
+  launch_scan<double>(static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, k, 1, maxA, h->status, st);
+  launch_scan<double>(static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+  trace_end(h, PH_SCAN, st, 2);
   if (probe > 0) {
-    if (!ss->side && (cudaStreamCreateWithFlags(&ss->side, cudaStreamNonBlocking) != cudaSuccess ||
-                      cudaEventCreateWithFlags(&ss->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-                      cudaEventCreateWithFlags(&ss->ev_probe, cudaEventDisableTiming) != cudaSuccess))
-      return EMU_ERR_CUDA;
-    auto* hidx = reinterpret_cast<int32_t*>(ss->host);
-    uint64_t x = 0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(m * 1315423911u + n * 2654435761u + k);
-    for (int q = 0; q < probe; ++q) {
-      x ^= x << 13;
-      x ^= x >> 7;
-      x ^= x << 17;
-      hidx[2 * q] = static_cast<int32_t>(x % static_cast<uint64_t>(m));
-      x ^= x << 13;
-      x ^= x >> 7;
-      x ^= x << 17;
-      hidx[2 * q + 1] = static_cast<int32_t>(x % static_cast<uint64_t>(n));
-    }
-    // (the host buffer is next written by the features' copy, which the
-    // stream orders after this one)
-    if (cudaMemcpyAsync(d_idx, hidx, 8 * static_cast<size_t>(probe), cudaMemcpyHostToDevice, st) != cudaSuccess)
-      return EMU_ERR_CUDA;
-    if (layout != EMU_ROW_MAJOR) swap_pairs_kernel<<<(probe + 127) / 128, 128, 0, st>>>(d_idx, probe, d_sw);
-    if (cudaEventRecord(ss->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ss->side, ss->ev_fork, 0) != cudaSuccess)
-      return EMU_ERR_CUDA;
-    emu_status_t s = emu_probe_dd(h, layout, m, n, k, A, lda, B, ldb, probe, d_idx, d_ref, d_ab, ss->side);
+    probe_idx_kernel<<<1, 1, 0, ss->side>>>(
+        0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(m * 1315423911u + n * 2654435761u + k), m, n, probe, d_idx);
+    s = emu_probe_dd(h, layout, m, n, k, A, lda, B, ldb, probe, d_idx, d_ref, d_ab, ss->side);
     if (s != EMU_OK) return s;
     if (cudaEventRecord(ss->ev_probe, ss->side) != cudaSuccess) return EMU_ERR_CUDA;
   }
-  {  // the feature scan needs scratch for the row / column maxima and histograms
-    uint8_t* ws = nullptr;
-    emu_status_t s = handle_workspace(h, feat_scratch(v), st, &ws);
-    if (s != EMU_OK) return s;
-    s = features_impl(h, v, k, tol, 64, feat, ws, st);
-    if (s != EMU_OK) return s;
-  }
-  const bool loaded = scheme_II ? ss->loaded_II : ss->loaded;
-  if (loaded) mlp_forward_kernel<<<1, kHid, 0, st>>>(scheme_II ? ss->params_II : ss->params, feat, 1, prob, nullptr);
-  // one copy back: features and (if a network is loaded) probabilities
-  if (cudaMemcpyAsync(ss->host, feat, sizeof(float) * (128 + kOut), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return EMU_ERR_CUDA;
-  const float* f = reinterpret_cast<const float*>(ss->host);
+  if (cudaEventSynchronize(ss->ev_decide) != cudaSuccess) return EMU_ERR_CUDA;
+  const float* f = h_dec;
   const float* pr = f + 128;
   // value of class c and the largest value: p = 3 + c up to EMU_P_MAX, or
   // N = 6 + 2c up to EMU_NM_MAX
@@ -624,18 +723,16 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
     p = cls == kOut - 1 ? top : base_v + step * cls;
   }
   for (int attempt = 0; attempt < 3; ++attempt) {
-    emu_status_t s = emu_dgemm(h, layout, m, n, k, alpha, A, lda, B, ldb, 0.0, C, ldc,
-                               scheme_II ? EMU_SCHEME_II_NORM : EMU_SCHEME_I, p, stream);
+    s = dgemm_scanned(h, layout, m, n, k, alpha, A, lda, B, ldb, C, ldc,
+                      scheme_II ? EMU_SCHEME_II_NORM : EMU_SCHEME_I, p, maxA, maxB, stream);
     if (s != EMU_OK) return s;
     *p_used = p;
     if (probe == 0) return EMU_OK;
     if (attempt == 0 && cudaStreamWaitEvent(st, ss->ev_probe, 0) != cudaSuccess) return EMU_ERR_CUDA;
-    gather_kernel<<<(probe + 127) / 128, 128, 0, st>>>(C, ldc, probe, layout == EMU_ROW_MAJOR ? d_idx : d_sw, d_c);
-    // one copy back: [ref | ab | C entries]
-    if (cudaMemcpyAsync(ss->host, d_ref, 32 * static_cast<size_t>(probe), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return EMU_ERR_CUDA;
-    const double* ref = reinterpret_cast<const double*>(ss->host);
+    judge_kernel<<<(probe + 127) / 128, 128, 0, st>>>(C, ldc, layout != EMU_ROW_MAJOR, probe, d_idx, d_ref, d_ab,
+                                                      h_res);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return EMU_ERR_CUDA;
+    const double* ref = h_res;
     const double* ab = ref + 2 * probe;
     const double* cv = ab + probe;
     double worst = 0.0;
