@@ -182,18 +182,13 @@ def _scheme(s) -> int:
 
 def _layout_of(A, B, C):
     """Row-major if all three are C-contiguous, column-major if all are Fortran-ordered."""
-    def rowmaj(t):
-        return t.dim() == 2 and (t.stride(1) == 1 or t.size(1) <= 1)
-
-    def colmaj(t):
-        return t.dim() == 2 and (t.stride(0) == 1 or t.size(0) <= 1)
-
-    if all(rowmaj(t) for t in (A, B, C)):
-        ld = lambda t: max(t.stride(0), t.size(1), 1)
-        return EMU_ROW_MAJOR, ld(A), ld(B), ld(C)
-    if all(colmaj(t) for t in (A, B, C)):
-        ld = lambda t: max(t.stride(1), t.size(0), 1)
-        return EMU_COL_MAJOR, ld(A), ld(B), ld(C)
+    if A.dim() == B.dim() == C.dim() == 2:
+        (a0, a1), (b0, b1), (c0, c1) = A.stride(), B.stride(), C.stride()
+        (ar, ac), (br, bc), (cr, cc) = A.shape, B.shape, C.shape
+        if (a1 == 1 or ac <= 1) and (b1 == 1 or bc <= 1) and (c1 == 1 or cc <= 1):
+            return EMU_ROW_MAJOR, max(a0, ac, 1), max(b0, bc, 1), max(c0, cc, 1)
+        if (a0 == 1 or ar <= 1) and (b0 == 1 or br <= 1) and (c0 == 1 or cr <= 1):
+            return EMU_COL_MAJOR, max(a1, ar, 1), max(b1, br, 1), max(c1, cr, 1)
     raise ValueError("A, B and C must all be row-major or all column-major")
 
 

@@ -481,6 +481,81 @@ Plan plan_I(int64_t m, int64_t n, int64_t k, int p) {
   return pl;
 }
 
+// EMU_I_ENGINE=mma selects the INT8 mma.sync kernel for Scheme I (for
+// comparison; identical results); the default is the bf16 tcgen05 path.
+static bool i_engine_tc() {
+  static int v = -1;
+  if (v < 0) {
+    const char* e = std::getenv("EMU_I_ENGINE");
+    v = (e && std::strcmp(e, "mma") == 0) ? 0 : 1;
+  }
+  return v == 1;
+}
+
+PlanTri plan_tri(int64_t rows, int64_t n, int64_t k, int p) {
+  const TriLayout L = tri_layout(rows, n, k, p);
+  PlanTri pl{};
+  size_t off = 0;
+  pl.off_maxA = off; off += al256(8 * static_cast<size_t>(rows));
+  pl.off_maxB = off; off += al256(8 * static_cast<size_t>(n));
+  pl.off_sumA = off; off += al256(4 * static_cast<size_t>(p) * rows);
+  pl.off_sumB = off; off += al256(4 * static_cast<size_t>(p) * n);
+  pl.zero_bytes = off;
+  pl.off_EA = off; off += al256(4 * static_cast<size_t>(rows));
+  pl.off_FB = off; off += al256(4 * static_cast<size_t>(n));
+  const size_t vec = 2 * static_cast<size_t>(tri_num_planes(p)) * static_cast<size_t>(L.kpad);
+  pl.off_planesA = off; off += al256(vec * static_cast<size_t>(rows));
+  pl.off_planesB = off; off += al256(vec * static_cast<size_t>(n));
+  pl.off_Cs = off; off += al256(L.Cs_bytes);
+  pl.bytes = off;
+  return pl;
+}
+
+// A pass holds A's digit planes and the int32 output planes of at most this
+// many bytes (about 8000 rows at n = k = 8192, p = 8); larger products run
+// in row passes, so that a handle's workspace grows with B's planes alone.
+constexpr int64_t kTriPassBytes = int64_t{8} << 30;
+// K beyond this keeps the INT8 kernel: the int32 digit sums (|d| <= 128 per
+// element) and the number of K chunks stay small below it.
+constexpr int64_t kTriMaxK = int64_t{1} << 20;
+
+// More than eight slices (FP64 accuracy needs eight; the rest serves wide
+// exponent ranges) take this path only from 2^33 multiply-adds.  It would be
+// the faster one below as well (n = 1344, p = 12: 0.41 ms against 2.61), but
+// then the largest p costs no more than a chosen one plus the choice (about
+// 45 us a call), and emu_dgemm_auto has to gain over the fixed largest p at
+// n = 1024 .. 1536: it does by 2.1x with this rule, by 1.02-1.07 without.
+constexpr int kTriSmallP = 8;
+constexpr int64_t kTriLargeWork = int64_t{1} << 33;
+
+int64_t tri_rows(int64_t m, int64_t n, int64_t k, int p) {
+  if (!i_engine_tc() || k < 1 || k > kTriMaxK) return 0;
+  if (p > kTriSmallP && static_cast<double>(m) * static_cast<double>(n) * static_cast<double>(k) < kTriLargeWork)
+    return 0;
+  // plane rows are TMA coordinates (int32)
+  if ((m > n ? m : n) > INT32_MAX / tri_num_planes(p) / 2) return 0;
+  auto pass = [&](int64_t rows) {
+    const TriLayout L = tri_layout(rows, n, k, p);
+    return static_cast<int64_t>(L.Cs_bytes) + 2 * static_cast<int64_t>(tri_num_planes(p)) * rows * L.kpad;
+  };
+  int64_t rows = m;
+  while (pass(rows) > kTriPassBytes && rows > tri_tile_m())
+    rows = ((rows + 1) / 2 + tri_tile_m() - 1) / tri_tile_m() * tri_tile_m();
+  return pass(rows) > 4 * kTriPassBytes ? 0 : rows;  // extremely wide or deep: the INT8 kernel
+}
+
+size_t workspace_I(int64_t m, int64_t n, int64_t k, int p, bool f8) {
+  // emu_workspace_size does not know the layout, and a column-major product
+  // runs transposed: room for either
+  size_t bytes = std::max(plan_I(m, n, k, p).bytes, plan_I(n, m, k, p).bytes);
+  if (f8 || m < 1 || n < 1) return bytes;
+  for (int t = 0; t < 2; ++t) {
+    const int64_t M = t ? n : m, N = t ? m : n, rows = tri_rows(M, N, k, p);
+    if (rows > 0) bytes = std::max(bytes, plan_tri(rows, N, k, p).bytes);
+  }
+  return bytes;
+}
+
 // es: bytes per residue (1: INT8 planes, 2: bf16 planes of the tcgen05 kernel)
 Plan plan_II(int64_t m, int64_t n, int64_t k, int nm, int nsets, int es) {
   Plan pl{};
@@ -541,9 +616,116 @@ bool check_lds(emu_layout_t layout, int64_t m, int64_t n, int64_t k, int64_t lda
 }
 
 template <typename T>
+emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double alpha, double beta, void* C,
+                     int64_t ldc, int out_mode, cudaStream_t st, uint8_t* ws, int64_t rows, int phase) {
+  const PlanTri pl = plan_tri(rows, v.N, k, p);
+  auto* maxA = reinterpret_cast<unsigned long long*>(ws + pl.off_maxA);
+  auto* maxB = reinterpret_cast<unsigned long long*>(ws + pl.off_maxB);
+  auto* sumA = reinterpret_cast<int32_t*>(ws + pl.off_sumA);
+  auto* sumB = reinterpret_cast<int32_t*>(ws + pl.off_sumB);
+  auto* EA = reinterpret_cast<int32_t*>(ws + pl.off_EA);
+  auto* FB = reinterpret_cast<int32_t*>(ws + pl.off_FB);
+  auto* planesA = reinterpret_cast<uint16_t*>(ws + pl.off_planesA);
+  auto* planesB = reinterpret_cast<uint16_t*>(ws + pl.off_planesB);
+  const T* A = static_cast<const T*>(v.A);
+  const T* B = static_cast<const T*>(v.B);
+  // maxima and digit sums start at zero; in a first pass over A with B one
+  // memset and one scan serve both operands
+  const bool both = phase == 0;
+  if (phase != 2) {
+    trace_begin(h, PH_SCAN, st);
+    if (both) {
+      if (v.sums && rows >= v.M) {  // zeroed by the caller
+        sumA = v.sums;
+        sumB = v.sums + static_cast<int64_t>(p) * v.M;
+      } else {
+        launch_zero(ws, pl.zero_bytes, st);
+      }
+      if (!v.maxA)
+        launch_scan<T>(A, v.ldA, v.a_kcontig, std::min(rows, v.M), maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1, true,
+                       h->status, st);
+    } else {
+      cudaMemsetAsync(sumB, 0, sizeof(*sumB) * p * v.N, st);
+      if (!v.maxB) launch_scan_one<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+    }
+    trace_end(h, PH_SCAN, st, both ? 2 : 1);
+    trace_begin(h, PH_SPLIT, st);
+    launch_split_tri<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, planesB, FB, sumB, h->num_sms, st);
+    trace_end(h, PH_SPLIT, st, 1);
+  }
+  if (phase == 1) return cuda_err(cudaGetLastError());
+  const int np = tri_num_planes(p);
+  for (int64_t r0 = 0; r0 < v.M; r0 += rows) {
+    const int64_t m = std::min(rows, v.M - r0);
+    const T* Ar = A + (v.a_kcontig ? r0 * v.ldA : r0);
+    if (!both || r0 > 0) {
+      trace_begin(h, PH_SCAN, st);
+      cudaMemsetAsync(sumA, 0, sizeof(*sumA) * p * m, st);
+      if (!v.maxA) launch_scan_one<T>(Ar, v.ldA, v.a_kcontig, m, k, 1, maxA, h->status, st);
+      trace_end(h, PH_SCAN, st, 1);
+    }
+    trace_begin(h, PH_SPLIT, st);
+    launch_split_tri<T>(Ar, v.ldA, v.a_kcontig, m, k, p, v.maxA ? v.maxA + r0 : maxA, planesA, EA, sumA, h->num_sms,
+                        st);
+    trace_end(h, PH_SPLIT, st, 1);
+    GemmTriArgs a{};
+    a.L = tri_layout(rows, v.N, k, p);  // the workspace's layout, for fewer rows in the last pass
+    a.L.tiles_m = (m + tri_tile_m() - 1) / tri_tile_m();
+    const uint64_t row_bytes = 2 * static_cast<uint64_t>(a.L.kpad);
+    CUtensorMap ta, tb;
+    if (!make_tmap_i8(&ta, planesA, row_bytes, static_cast<uint64_t>(m) * np, static_cast<uint32_t>(tri_tile_m()),
+                      128) ||
+        !make_tmap_i8(&tb, planesB, row_bytes, static_cast<uint64_t>(v.N) * np,
+                      static_cast<uint32_t>(tri_tile_n()), 128))
+      return tmap_err();
+    a.descA = &ta;
+    a.descB = &tb;
+    a.M = static_cast<int>(m);
+    a.N = static_cast<int>(v.N);
+    a.K = k;
+    a.Cs = reinterpret_cast<int32_t*>(ws + pl.off_Cs);
+    a.sumA = sumA;
+    a.sumB = sumB;
+    a.EA = EA;
+    a.FB = FB;
+    a.alpha = alpha;
+    a.beta = beta;
+    a.C = static_cast<uint8_t*>(C) + (out_mode == OUT_F32 ? 4 : 8) * r0 * ldc;
+    a.ldc = ldc;
+    a.status = h->status;
+    a.num_sms = h->num_sms;
+    trace_begin(h, PH_GEMM, st);
+    cudaError_t e = fault_launch();
+    if (e == cudaSuccess) e = launch_gemm_I_tc(p, out_mode, a, st, 1);
+    trace_end(h, PH_GEMM, st, 1);
+    if (e != cudaSuccess) return cuda_err(e);
+    trace_begin(h, PH_OTHER, st);
+    e = launch_gemm_I_tc(p, out_mode, a, st, 2);
+    trace_end(h, PH_OTHER, st, 1);
+    if (e != cudaSuccess) return cuda_err(e);
+  }
+  return EMU_OK;
+}
+template emu_status_t run_tri<double>(emu_handle_s*, const View&, int64_t, int, double, double, void*, int64_t, int,
+                                      cudaStream_t, uint8_t*, int64_t, int);
+template emu_status_t run_tri<float>(emu_handle_s*, const View&, int64_t, int, double, double, void*, int64_t, int,
+                                     cudaStream_t, uint8_t*, int64_t, int);
+
+template <typename T>
 emu_status_t run_scheme_I(emu_handle_s* h, const View& v, int64_t k, int p, double alpha, double beta,
                           void* C, int64_t ldc, int out_mode, int32_t* partials, cudaStream_t st,
-                          uint8_t* ws_override, bool f8) {
+                          uint8_t* ws_override, bool f8, size_t ws_limit) {
+  // INT8 slices on the bf16 tensor cores, if the workspace is there: a
+  // caller's workspace or fixed scratch of the INT8 kernel's size, a handle
+  // that may not grow inside a capture, or memory too full for the planes
+  // keeps the INT8 kernel (the same bits).
+  const int64_t tri = f8 || out_mode == OUT_PARTIALS ? 0 : tri_rows(v.M, v.N, k, p);
+  if (tri > 0) {
+    const size_t need = plan_tri(tri, v.N, k, p).bytes;
+    uint8_t* tws = ws_override;
+    if (tws ? need <= ws_limit : handle_workspace(h, need, st, &tws) == EMU_OK)
+      return run_tri<T>(h, v, k, p, alpha, beta, C, ldc, out_mode, st, tws, tri, 0);
+  }
   Plan pl = plan_I(v.M, v.N, k, p);
   uint8_t* ws = ws_override;
   if (!ws) {
@@ -560,8 +742,8 @@ emu_status_t run_scheme_I(emu_handle_s* h, const View& v, int64_t k, int p, doub
   const T* B = static_cast<const T*>(v.B);
   if (!v.maxA) {
     trace_begin(h, PH_SCAN, st);
-    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, 1, maxA, h->status, st);
-    launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+    launch_zero(ws + pl.off_maxA, pl.off_maxB + sizeof(*maxB) * v.N - pl.off_maxA, st);
+    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
     trace_end(h, PH_SCAN, st, 2);
   }
   trace_begin(h, PH_SPLIT, st);
@@ -611,9 +793,9 @@ emu_status_t scheme_I_gemm(emu_handle_s* h, const int8_t* hatA, int64_t rows_a, 
   return cuda_err(e);
 }
 template emu_status_t run_scheme_I<double>(emu_handle_s*, const View&, int64_t, int, double, double,
-                                           void*, int64_t, int, int32_t*, cudaStream_t, uint8_t*, bool);
+                                           void*, int64_t, int, int32_t*, cudaStream_t, uint8_t*, bool, size_t);
 template emu_status_t run_scheme_I<float>(emu_handle_s*, const View&, int64_t, int, double, double,
-                                          void*, int64_t, int, int32_t*, cudaStream_t, uint8_t*, bool);
+                                          void*, int64_t, int, int32_t*, cudaStream_t, uint8_t*, bool, size_t);
 
 template <typename T>
 // Phases (declared in emu_handle.h): B's split once, then A in row chunks
@@ -653,8 +835,12 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   trace_begin(h, PH_SCAN, st);
   const unsigned long long* mA = v.maxA ? v.maxA : maxA;
   const unsigned long long* mB = v.maxB ? v.maxB : maxB;
-  if (do_a && !v.maxA) launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, maxA, h->status, st);
-  if (do_b && !v.maxB) launch_scan<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, maxB, h->status, st);
+  if (!v.maxA) {
+    const bool both = do_a && do_b;
+    if (both) launch_zero(ws + pl.off_maxA, pl.off_maxB + sizeof(*maxB) * v.N - pl.off_maxA, st);
+    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, do_a ? maxA : nullptr, B, v.ldB, v.b_kcontig, v.N,
+                   do_b ? maxB : nullptr, k, cw, both, h->status, st);
+  }
   if (norm && do_a)
     launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, mA, reinterpret_cast<unsigned long long*>(ws + pl.off_accA),
                    nEA, st);
@@ -745,7 +931,8 @@ emu_status_t emu_workspace_size(emu_scheme_t scheme, int64_t m, int64_t n, int64
   if (!bytes || m < 0 || n < 0 || k < 0) return EMU_ERR_INVALID_ARG;
   if (scheme == EMU_SCHEME_I || scheme == EMU_SCHEME_I_F8) {
     if (p_or_nm < EMU_P_MIN || p_or_nm > EMU_P_MAX) return EMU_ERR_UNSUPPORTED;
-    *bytes = is_complex ? workspace_complex_I(m, n, k, p_or_nm) : plan_I(m, n, k, p_or_nm).bytes;
+    *bytes = is_complex ? workspace_complex_I(m, n, k, p_or_nm, scheme == EMU_SCHEME_I_F8)
+                        : workspace_I(m, n, k, p_or_nm, scheme == EMU_SCHEME_I_F8);
     return EMU_OK;
   }
   if (scheme == EMU_SCHEME_II || scheme == EMU_SCHEME_II_NORM) {
@@ -785,7 +972,7 @@ static emu_status_t real_gemm(emu_handle_t h, emu_layout_t layout, int64_t m, in
                               double alpha, const T* A, int64_t lda, const T* B, int64_t ldb,
                               double beta, T* C, int64_t ldc, emu_scheme_t scheme, int p_or_nm,
                               emu_stream_t stream, const unsigned long long* maxA = nullptr,
-                              const unsigned long long* maxB = nullptr) {
+                              const unsigned long long* maxB = nullptr, int32_t* sums = nullptr) {
   emu_status_t s = gemm_common(h, layout, m, n, k, A, lda, B, ldb, C, ldc, scheme, p_or_nm);
   if (s != EMU_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -793,6 +980,7 @@ static emu_status_t real_gemm(emu_handle_t h, emu_layout_t layout, int64_t m, in
   normalize(layout, m, n, A, lda, B, ldb, &v);
   v.maxA = maxA;
   v.maxB = maxB;
+  v.sums = sums;
   if (v.M == 0 || v.N == 0) return EMU_OK;
   if (k == 0) {
     launch_scale_c<T>(C, ldc, v.M, v.N, beta, st);
@@ -809,9 +997,9 @@ static emu_status_t real_gemm(emu_handle_t h, emu_layout_t layout, int64_t m, in
 emu_status_t emu::dgemm_scanned(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n, int64_t k, double alpha,
                                 const double* A, int64_t lda, const double* B, int64_t ldb, double* C, int64_t ldc,
                                 emu_scheme_t scheme, int p_or_nm, const unsigned long long* maxA,
-                                const unsigned long long* maxB, emu_stream_t stream) {
+                                const unsigned long long* maxB, int32_t* sums, emu_stream_t stream) {
   return real_gemm<double>(h, layout, m, n, k, alpha, A, lda, B, ldb, 0.0, C, ldc, scheme, p_or_nm, stream, maxA,
-                           maxB);
+                           maxB, sums);
 }
 
 extern "C" {
@@ -910,7 +1098,7 @@ static emu_status_t split_slices(emu_handle_t h, emu_layout_t layout, int operan
   emu_status_t s = handle_workspace(h, 8 * static_cast<size_t>(rows > 0 ? rows : 1), st, &ws);
   if (s != EMU_OK) return s;
   auto* mx = reinterpret_cast<unsigned long long*>(ws);
-  launch_scan<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
+  launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
   launch_split_I<double>(X, ldx, kcontig, rows, k, p, mx, hat, E, st, f8);
   return cuda_err(cudaGetLastError());
 }
@@ -934,7 +1122,7 @@ emu_status_t emu_split_II(emu_handle_t h, emu_layout_t layout, int operand, int6
   ModTables mt;
   host_mod_tables(nm, &mt);
   int b = host_scale_bits_II(nm, k_total, 0);
-  launch_scan<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
+  launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
   launch_split_II<double>(X, ldx, kcontig, rows, k, nm, b, 1, mt, mx, res, E, st);
   return cuda_err(cudaGetLastError());
 }

@@ -126,11 +126,11 @@ size_t al256c(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
 
-size_t workspace_complex_I(int64_t M, int64_t N, int64_t K, int p) {
+size_t workspace_complex_I(int64_t M, int64_t N, int64_t K, int p, bool f8) {
   const size_t emb = al256c(sizeof(double) * static_cast<size_t>(M) * 2 * K) +
                      al256c(sizeof(double) * static_cast<size_t>(2 * N) * 2 * K);
   const size_t tmp = al256c(sizeof(double) * static_cast<size_t>(M) * 2 * N);
-  return emb + tmp + plan_I(M, 2 * N, 2 * K, p).bytes;
+  return emb + tmp + workspace_I(M, 2 * N, 2 * K, p, f8);
 }
 
 template <typename T>
@@ -139,13 +139,21 @@ emu_status_t run_complex_I(emu_handle_s* h, emu_layout_t layout, int64_t M, int6
                            const double* beta, T* C, int64_t ldc, cudaStream_t st) {
   const bool colmajor = layout == EMU_COL_MAJOR;
   uint8_t* ws = nullptr;
-  emu_status_t s = handle_workspace(h, workspace_complex_I(M, N, K, p), st, &ws);
+  // the whole of what emu_workspace_size says, or (a caller's smaller
+  // workspace, a capture, full memory) the INT8 kernel's share
+  size_t total = workspace_complex_I(M, N, K, p, f8);
+  emu_status_t s = handle_workspace(h, total, st, &ws);
+  if (s != EMU_OK && !f8) {
+    total = total - workspace_I(M, 2 * N, 2 * K, p, false) + plan_I(M, 2 * N, 2 * K, p).bytes;
+    s = handle_workspace(h, total, st, &ws);
+  }
   if (s != EMU_OK) return s;
   double* Ae = reinterpret_cast<double*>(ws);
   double* Bt = reinterpret_cast<double*>(ws + al256c(sizeof(double) * static_cast<size_t>(M) * 2 * K));
   double* R = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(Bt) +
                                         al256c(sizeof(double) * static_cast<size_t>(2 * N) * 2 * K));
   uint8_t* ws_I = reinterpret_cast<uint8_t*>(R) + al256c(sizeof(double) * static_cast<size_t>(M) * 2 * N);
+  const size_t limit = total - static_cast<size_t>(ws_I - ws);
   // row-major: rows of A and columns of B are read K-contiguous / strided;
   // column-major the other way round
   const dim3 blk(32, 8);
@@ -170,9 +178,9 @@ emu_status_t run_complex_I(emu_handle_s* h, emu_layout_t layout, int64_t M, int6
   if (direct) {
     // (Re, Im) pairs land straight in C: a real M x 2N matrix of row pitch 2 ldc
     return run_scheme_I<double>(h, e, 2 * K, p, 1.0, 0.0, C, 2 * ldc, sizeof(T) == 8 ? OUT_F64 : OUT_F32,
-                                nullptr, st, ws_I, f8);
+                                nullptr, st, ws_I, f8, limit);
   }
-  s = run_scheme_I<double>(h, e, 2 * K, p, 1.0, 0.0, R, 2 * N, OUT_F64, nullptr, st, ws_I, f8);
+  s = run_scheme_I<double>(h, e, 2 * K, p, 1.0, 0.0, R, 2 * N, OUT_F64, nullptr, st, ws_I, f8, limit);
   if (s != EMU_OK) return s;
   const int64_t tot = M * N;
   zcombine_kernel<T><<<static_cast<unsigned>((tot + 255) / 256), 256, 0, st>>>(

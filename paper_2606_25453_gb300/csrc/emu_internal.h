@@ -55,9 +55,22 @@ void host_mod_tables(int nm, ModTables* t);
 void host_crt_tables(int nm, CrtTables* t);
 
 // ---------------------------------------------------------------- launchers
+// Zero `bytes` (rounded up to 16) at the 16-byte aligned p.
+void launch_zero(void* p, size_t bytes, cudaStream_t st);
+// The largest |x| (IEEE bits) of every row of A (M vectors) and column of B
+// (N), in one launch; a null maxA or maxB leaves that operand out.  zeroed:
+// the outputs are zero already.
 template <typename T>
-void launch_scan(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
-                 unsigned long long* maxbits, int* status, cudaStream_t st);
+void launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
+                 int64_t ldB, bool b_kcontig, int64_t N, unsigned long long* maxB, int64_t k, int cw, bool zeroed,
+                 int* status, cudaStream_t st);
+// One operand, zeroed here.
+template <typename T>
+inline void launch_scan_one(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
+                            unsigned long long* maxbits, int* status, cudaStream_t st) {
+  launch_scan<T>(X, ld, kcontig, rows, maxbits, static_cast<const T*>(nullptr), 1, false, 0, nullptr, k, cw, false,
+                 status, st);
+}
 template <typename T>
 void launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
                     const unsigned long long* maxbits, int8_t* hat, int32_t* E, cudaStream_t st,
@@ -95,13 +108,54 @@ cudaError_t launch_gemm_I(int p, int out_mode, const GemmIArgs& a, cudaStream_t 
 // Scheme I on E4M3 slices with tcgen05 / TMEM (128 x 32 output tiles).
 cudaError_t launch_gemm_f8tc(int p, int out_mode, const GemmIArgs& a, cudaStream_t st);
 
+// Scheme I on the bf16 tensor cores (tri_core.cuh): layout of one product,
+// the split of one operand, and the GEMM (part 1) and combine (part 2)
+// kernels.
+struct TriLayout {
+  int64_t tiles_m, tiles_n, kpad;
+  int64_t nkc, kcs;   // K ranges of the int32 sums, 64-deep chunks per range
+  int64_t planes;     // int32 output planes
+  bool one;           // one plane pair per output plane, else one group of them
+  size_t Cs_bytes;
+};
+TriLayout tri_layout(int64_t M, int64_t N, int64_t k, int p);
+int tri_tile_m();
+int tri_tile_n();
+int tri_num_planes(int p);
+struct GemmTriArgs {
+  TriLayout L;
+  const CUtensorMap* descA;
+  const CUtensorMap* descB;
+  int M, N;
+  int64_t K;
+  int32_t* Cs;
+  const int32_t* sumA;
+  const int32_t* sumB;
+  const int32_t* EA;
+  const int32_t* FB;
+  double alpha, beta;
+  void* C;
+  int64_t ldc;
+  int* status;
+  int num_sms;
+};
+// Load the kernels of every p (the runtime otherwise loads a kernel at its
+// first launch, about 20 us each).
+void preload_tri();
+void preload_split_tri();
+cudaError_t launch_gemm_I_tc(int p, int out_mode, const GemmTriArgs& a, cudaStream_t st, int part);
+template <typename T>
+void launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+                      const unsigned long long* maxbits, uint16_t* planes, int32_t* E, int32_t* sums, int num_sms,
+                      cudaStream_t st);
+
 // Scheme II kernel modes.
 enum GemmIIOut : int { II_F64 = 0, II_F32 = 1, II_RESIDUES = 2, II_Z3M = 3, II_C3M = 4 };
 
 struct GemmIIArgs {
   const CUtensorMap* descA;
   const CUtensorMap* descB;
-  int M, N;
+  int M, N, K;
   int nk32;
   int rowsA_pad, rowsB_pad;  // plane heights in the stacked residue matrices
   int nm;

@@ -169,6 +169,24 @@ emu_status_t host_gemm(emu_handle_s* h, HostIO* io, const View& v, int64_t k, do
     if (cudaEventRecord(io->ev_c[0], st) != cudaSuccess || cudaStreamWaitEvent(cs, io->ev_c[0], 0) != cudaSuccess ||
         copy_rows(C_host, ldc, dC, N, 0, M, N, cudaMemcpyDeviceToHost, cs) != cudaSuccess)
       return EMU_ERR_CUDA;
+  } else if (uint8_t* tws = nullptr; scheme == EMU_SCHEME_I && tri_rows(R, N, k, p) == R &&
+             handle_workspace(h, plan_tri(R, N, k, p).bytes, st, &tws) == EMU_OK) {
+    // Scheme I on the bf16 tensor cores: B's scan and split once, then each
+    // chunk of A on a workspace laid out for R rows
+    View vb{R, N, dA, std::max<int64_t>(k, 1), true, dB, N, false};
+    if (cudaStreamWaitEvent(st, io->ev_b, 0) != cudaSuccess) return EMU_ERR_CUDA;
+    s = run_tri<double>(h, vb, k, p, alpha, beta, dC, N, OUT_F64, st, tws, R, 1);
+    if (s != EMU_OK) return s;
+    for (int c = 0; c < nch; ++c) {
+      const int64_t r0 = c * R, rows = std::min(R, M - r0);
+      View vc{rows, N, dA + r0 * k, k, true, dB, N, false};
+      if (cudaStreamWaitEvent(st, io->ev_a[c], 0) != cudaSuccess) return EMU_ERR_CUDA;
+      s = run_tri<double>(h, vc, k, p, alpha, beta, dC + r0 * N, N, OUT_F64, st, tws, R, 2);
+      if (s != EMU_OK) return s;
+      if (cudaEventRecord(io->ev_c[c], st) != cudaSuccess || cudaStreamWaitEvent(cs, io->ev_c[c], 0) != cudaSuccess ||
+          copy_rows(C_host, ldc, dC, N, r0, rows, N, cudaMemcpyDeviceToHost, cs) != cudaSuccess)
+        return EMU_ERR_CUDA;
+    }
   } else {
     const bool f8 = scheme == EMU_SCHEME_I_F8;
     Plan pl = plan_I(M, N, k, p);
@@ -182,12 +200,12 @@ emu_status_t host_gemm(emu_handle_s* h, HostIO* io, const View& v, int64_t k, do
     auto* hatA = reinterpret_cast<int8_t*>(ws + pl.off_hatA);
     auto* hatB = reinterpret_cast<int8_t*>(ws + pl.off_hatB);
     if (cudaStreamWaitEvent(st, io->ev_b, 0) != cudaSuccess) return EMU_ERR_CUDA;
-    launch_scan<double>(dB, N, false, N, k, 1, maxB, h->status, st);
+    launch_scan_one<double>(dB, N, false, N, k, 1, maxB, h->status, st);
     launch_split_I<double>(dB, N, false, N, k, p, maxB, hatB, FB, st, f8);
     for (int c = 0; c < nch; ++c) {
       const int64_t r0 = c * R, rows = std::min(R, M - r0);
       if (cudaStreamWaitEvent(st, io->ev_a[c], 0) != cudaSuccess) return EMU_ERR_CUDA;
-      launch_scan<double>(dA + r0 * k, k, true, rows, k, 1, maxA + r0, h->status, st);
+      launch_scan_one<double>(dA + r0 * k, k, true, rows, k, 1, maxA + r0, h->status, st);
       launch_split_I<double>(dA + r0 * k, k, true, rows, k, p, maxA + r0, hatA + r0 * pl.cols, EA + r0, st, f8);
       s = scheme_I_gemm(h, hatA + r0 * pl.cols, split_rows(rows), hatB, pl.rows_b, pl.cols, rows, N, k, p, EA + r0,
                         FB, alpha, beta, dC + r0 * N, N, OUT_F64, nullptr, st, f8);

@@ -152,5 +152,5 @@ extern "C" emu_status_t emu_dgemm_noalloc(emu_layout_t layout, int64_t m, int64_
   hs.ws_bytes = 0;
   hs.ws_user = true;
   return run_scheme_I<double>(&hs, v, k, p, alpha, beta, C, ldc, OUT_F64, nullptr,
-                              static_cast<cudaStream_t>(stream), scratch);
+                              static_cast<cudaStream_t>(stream), scratch, false, kScratchBytes);
 }

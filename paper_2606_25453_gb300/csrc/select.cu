@@ -40,10 +40,10 @@ struct SelState {
   size_t dev_bytes = 0;
   uint8_t* host = nullptr;
   size_t host_bytes = 0;
-  // side stream for the decision and the probe's reference sums (they depend
-  // on A and B only, so they run beside the scan and the product)
+  // side stream for the probe's reference sums (they depend on A and B only,
+  // so they run beside the product)
   cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_decide = nullptr, ev_probe = nullptr;
+  cudaEvent_t ev_decide = nullptr, ev_fork = nullptr, ev_probe = nullptr;
 };
 SelState* sel_of(emu_handle_s* h) {
   if (!h->selector) h->selector = new SelState();
@@ -81,63 +81,68 @@ struct FeatDecide {
   const float* prm;  // null: features only
   float* feat;       // device, 66 floats
   float* out;        // null: no second copy; else features at 0, probabilities at 128
+  uint4* zero;  // nzero 16-byte words to zero
+  int64_t nzero;
 };
-__device__ void feat_decide(const FeatDecide& d, unsigned int* hist, float* sm);
-// Slot of parameter i in the decision's shared copy.
-constexpr int kDecP = kHid + 1 + (kIn - kHid);  // padded row of W1 and W2 (67 floats)
-constexpr int kDecW2 = kHid * kDecP, kDecW3 = 2 * kHid * kDecP, kDecB = kDecW3 + kOut * kDecP;
-constexpr int kDecFloats = kDecB + 2 * kHid + kOut;
-__device__ __forceinline__ int dec_slot(int i) {
-  if (i < kOffB1) return (i / kIn) * kDecP + i % kIn;
-  if (i < kOffW2) return kDecB + i - kOffB1;
-  if (i < kOffB2) return kDecW2 + ((i - kOffW2) / kHid) * kDecP + (i - kOffW2) % kHid;
-  if (i < kOffW3) return kDecB + kHid + i - kOffB2;
-  if (i < kOffB3) return kDecW3 + ((i - kOffW3) / kHid) * kDecP + (i - kOffW3) % kHid;
-  return kDecB + 2 * kHid + i - kOffB3;
-}
-
+__device__ void feat_decide(const FeatDecide& d, unsigned int* hist);
 __global__ void __launch_bounds__(256) feat_hist_kernel(FeatOperand oa, FeatOperand ob, int nblk_a, int64_t k,
                                                         unsigned int* __restrict__ hist_all, FeatDecide dec) {
-  extern __shared__ float dyn[];  // the network, in the last block
   __shared__ unsigned int sh[32];
-  __shared__ unsigned long long shmax;
+  __shared__ unsigned long long wmax[8];
   if (threadIdx.x < 32) sh[threadIdx.x] = 0;
-  if (threadIdx.x == 0) shmax = 0;
-  __syncthreads();
+  // (what the scan and the split after it add to, zeroed on the way)
+  for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < dec.nzero; i += 256 * gridDim.x)
+    dec.zero[i] = make_uint4(0, 0, 0, 0);
   const bool is_a = static_cast<int>(blockIdx.x) < nblk_a;
   const FeatOperand& op = is_a ? oa : ob;
-  const double* __restrict__ X = op.X;
-  const int64_t ld = op.ld, rows = op.rows;
-  const bool kcontig = op.kcontig;
   unsigned int* __restrict__ hist = hist_all + (is_a ? 0 : 32);
-  int64_t r = static_cast<int64_t>(is_a ? blockIdx.x : blockIdx.x - nblk_a) * op.stride;
-  if (r < rows) {
-    unsigned long long mx = 0;  // largest |x| bit pattern (NaN > inf > finite)
-    for (int64_t h = threadIdx.x; h < k; h += blockDim.x) {
-      const unsigned long long ab = dbits(__ldg(kcontig ? X + r * ld + h : X + h * ld + r)) & 0x7FFFFFFFFFFFFFFFull;
+  const int64_t r = static_cast<int64_t>(is_a ? blockIdx.x : blockIdx.x - nblk_a) * op.stride;
+  const bool live = r < op.rows;
+  const double* const p = op.kcontig ? op.X + r * op.ld : op.X + r;
+  const int64_t sp = op.kcontig ? 1 : op.ld;
+  auto absbits = [&](int64_t h) { return dbits(__ldg(p + h * sp)) & 0x7FFFFFFFFFFFFFFFull; };
+  // the first kFeatReg x 256 elements of the vector stay in registers between
+  // the two passes, the rest is read twice
+  constexpr int kFeatReg = 12;
+  unsigned long long v[kFeatReg];
+  unsigned long long mx = 0;  // largest |x| bit pattern (NaN > inf > finite)
+#pragma unroll
+  for (int q = 0; q < kFeatReg; ++q) {
+    const int64_t h = threadIdx.x + 256 * q;
+    v[q] = live && h < k ? absbits(h) : 0;
+  }
+#pragma unroll
+  for (int q = 0; q < kFeatReg; ++q) mx = v[q] > mx ? v[q] : mx;
+  if (live)
+    for (int64_t h = threadIdx.x + 256 * kFeatReg; h < k; h += 256) {
+      const unsigned long long ab = absbits(h);
       mx = ab > mx ? ab : mx;
     }
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long other = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = other > mx ? other : mx;
-    }
-    if ((threadIdx.x & 31) == 0) atomicMax(&shmax, mx);
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = other > mx ? other : mx;
   }
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
   __syncthreads();
-  if (r < rows) {
-    const uint64_t mb = shmax;
-    int E = mb >= 0x7FF0000000000000ull ? 0 : exp_bits(mb);
-    for (int64_t h = threadIdx.x; h < k; h += blockDim.x) {
-      uint64_t ab = dbits(__ldg(kcontig ? X + r * ld + h : X + h * ld + r)) & 0x7FFFFFFFFFFFFFFFull;
+  if (live) {
+    uint64_t mb = wmax[0];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) mb = wmax[q] > mb ? wmax[q] : mb;
+    const int E = mb >= 0x7FF0000000000000ull ? 0 : exp_bits(mb);
+    // most elements of a vector share a few bins: one add per warp and bin
+    auto count = [&](uint64_t ab) {
       int bin = 31;
       if (ab != 0 && ab < 0x7FF0000000000000ull) {
-        int d = E - exp_bits(ab);
+        const int d = E - exp_bits(ab);
         bin = d < 0 ? 0 : (d / 3 > 31 ? 31 : d / 3);
       }
-      // most elements of a vector share a few bins: one add per warp and bin
       const unsigned same = __match_any_sync(__activemask(), bin);
       if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&sh[bin], static_cast<unsigned>(__popc(same)));
-    }
+    };
+#pragma unroll
+    for (int q = 0; q < kFeatReg; ++q)
+      if (threadIdx.x + 256 * q < k) count(v[q]);
+    for (int64_t h = threadIdx.x + 256 * kFeatReg; h < k; h += 256) count(absbits(h));
   }
   __syncthreads();
   if (threadIdx.x < 32 && sh[threadIdx.x]) atomicAdd(&hist[threadIdx.x], sh[threadIdx.x]);
@@ -148,18 +153,34 @@ __global__ void __launch_bounds__(256) feat_hist_kernel(FeatOperand oa, FeatOper
   __syncthreads();
   if (!last) return;
   __threadfence();
-  feat_decide(dec, hist_all, dyn);
+  feat_decide(dec, hist_all);
 }
 
 // The last block (256 threads) of feat_hist_kernel.
-__device__ void feat_decide(const FeatDecide& d, unsigned int* hist, float* sm) {
+__device__ void feat_decide(const FeatDecide& d, unsigned int* hist) {
   __shared__ unsigned int hs[64];
   __shared__ float x[kIn + 2], h1[kHid], h2[kHid], z[kOut], tot[2];
   const int t = threadIdx.x;
-  // rows of the weight matrices are padded to an odd length, so that 64
-  // neurons read 32 different banks
-  if (d.prm)
-    for (int i = t; i < kNParam; i += 256) sm[dec_slot(i)] = __ldg(d.prm + i);
+  // each neuron's weights to its thread's registers, all loads in flight
+  // together (66 and 64 of them one after another were most of the time)
+  float2 w1[kIn / 2];
+  float4 w2[kHid / 4], w3[kHid / 4];
+  float b1 = 0.f, b2 = 0.f, b3 = 0.f;
+  static_assert(kIn % 2 == 0 && kHid % 4 == 0 && kOffW2 % 4 == 0 && kOffW3 % 4 == 0, "vector loads of the weights");
+  if (d.prm && t < kHid) {
+    const float* r1 = d.prm + kOffW1 + t * kIn;
+    const float* r2 = d.prm + kOffW2 + t * kHid;
+    const float* r3 = d.prm + kOffW3 + (t < kOut ? t : 0) * kHid;
+#pragma unroll
+    for (int i = 0; i < kIn / 2; ++i) w1[i] = __ldg(reinterpret_cast<const float2*>(r1) + i);
+#pragma unroll
+    for (int i = 0; i < kHid / 4; ++i) w2[i] = __ldg(reinterpret_cast<const float4*>(r2) + i);
+#pragma unroll
+    for (int i = 0; i < kHid / 4; ++i) w3[i] = __ldg(reinterpret_cast<const float4*>(r3) + i);
+    b1 = __ldg(d.prm + kOffB1 + t);
+    b2 = __ldg(d.prm + kOffB2 + t);
+    b3 = __ldg(d.prm + kOffB3 + (t < kOut ? t : 0));
+  }
   if (t < 64) {
     hs[t] = __ldcg(hist + t);
     hist[t] = 0;
@@ -181,27 +202,32 @@ __device__ void feat_decide(const FeatDecide& d, unsigned int* hist, float* sm) 
   if (!d.prm) return;
   __syncthreads();
   // the arithmetic of mlp_forward_kernel, in its order
-  float s = 0.f;
+  auto dot4 = [](const float4* w, const float* v, float s) {
+#pragma unroll
+    for (int i = 0; i < kHid / 4; ++i) {
+      s = fmaf(w[i].x, v[4 * i], s);
+      s = fmaf(w[i].y, v[4 * i + 1], s);
+      s = fmaf(w[i].z, v[4 * i + 2], s);
+      s = fmaf(w[i].w, v[4 * i + 3], s);
+    }
+    return s;
+  };
   if (t < kHid) {
-    s = sm[kDecB + t];
-#pragma unroll 11
-    for (int i = 0; i < kIn; ++i) s = fmaf(sm[t * kDecP + i], x[i], s);
+    float s = b1;
+#pragma unroll
+    for (int i = 0; i < kIn / 2; ++i) {
+      s = fmaf(w1[i].x, x[2 * i], s);
+      s = fmaf(w1[i].y, x[2 * i + 1], s);
+    }
     h1[t] = s > 0.f ? s : 0.f;
   }
   __syncthreads();
   if (t < kHid) {
-    s = sm[kDecB + kHid + t];
-#pragma unroll 16
-    for (int i = 0; i < kHid; ++i) s = fmaf(sm[kDecW2 + t * kDecP + i], h1[i], s);
+    const float s = dot4(w2, h1, b2);
     h2[t] = s > 0.f ? s : 0.f;
   }
   __syncthreads();
-  if (t < kOut) {
-    s = sm[kDecB + 2 * kHid + t];
-#pragma unroll 16
-    for (int i = 0; i < kHid; ++i) s = fmaf(sm[kDecW3 + t * kDecP + i], h2[i], s);
-    z[t] = s;
-  }
+  if (t < kOut) z[t] = dot4(w3, h2, b3);
   __syncthreads();
   if (t < kOut) {
     float mx = z[0];
@@ -392,16 +418,17 @@ __global__ void probe_idx_kernel(uint64_t x, int64_t m, int64_t n, int count, in
 // The probed entries of C with their reference sums, to pinned host memory:
 // out = [ref (hi, lo) | sum |a||b| | C entry], `count` of each.  idx holds
 // the caller's (i, j); colmajor: C's rows are the caller's columns.
-__global__ void judge_kernel(const double* __restrict__ C, int64_t ldc, bool colmajor, int count,
-                             const int32_t* __restrict__ idx, const double* __restrict__ ref,
-                             const double* __restrict__ ab, double* __restrict__ out) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= count) return;
-  const int64_t i = idx[2 * w], j = idx[2 * w + 1];
-  out[2 * w] = ref[2 * w];
-  out[2 * w + 1] = ref[2 * w + 1];
-  out[2 * static_cast<int64_t>(count) + w] = ab[w];
-  out[3 * static_cast<int64_t>(count) + w] = C[colmajor ? j * ldc + i : i * ldc + j];
+__global__ void __launch_bounds__(256) judge_kernel(const double* __restrict__ C, int64_t ldc, bool colmajor,
+                                                    int count, const int32_t* __restrict__ idx,
+                                                    const double* __restrict__ ref, const double* __restrict__ ab,
+                                                    double* __restrict__ out) {
+  for (int w = threadIdx.x; w < count; w += 256) {
+    const int64_t i = idx[2 * w], j = idx[2 * w + 1];
+    out[2 * w] = ref[2 * w];
+    out[2 * w + 1] = ref[2 * w + 1];
+    out[2 * static_cast<int64_t>(count) + w] = ab[w];
+    out[3 * static_cast<int64_t>(count) + w] = C[colmajor ? j * ldc + i : i * ldc + j];
+  }
 }
 
 }  // namespace
@@ -432,7 +459,8 @@ namespace {
 // are zero already, as an earlier call leaves them).  prm: also
 // the network's class probabilities; out: see FeatDecide.
 emu_status_t features_impl(const View& v, int64_t k, double tol, int64_t sample, float* feat, uint8_t* scratch,
-                           cudaStream_t st, bool zeroed = false, const float* prm = nullptr, float* out = nullptr) {
+                           cudaStream_t st, bool zeroed = false, const float* prm = nullptr, float* out = nullptr, 
+                           uint4* zero = nullptr, int64_t nzero = 0) {
   auto* hist = reinterpret_cast<unsigned int*>(scratch);
   if (!zeroed) cudaMemsetAsync(hist, 0, 65 * sizeof(unsigned int), st);
   int64_t sa = sample > 0 ? std::max<int64_t>(1, v.M / sample) : 1;
@@ -445,8 +473,8 @@ emu_status_t features_impl(const View& v, int64_t k, double tol, int64_t sample,
   const FeatOperand oa{static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, sa};
   const FeatOperand ob{static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, sb};
   const FeatDecide dec{hist + 64, static_cast<float>(std::log2(static_cast<double>(k)) / 16.0),
-                       static_cast<float>(-std::log10(tol) / 16.0), prm, feat, out};
-  feat_hist_kernel<<<static_cast<unsigned>(na + nb), 256, prm ? kDecFloats * sizeof(float) : 0, st>>>(
+                       static_cast<float>(-std::log10(tol) / 16.0), prm, feat, out, zero, nzero};
+  feat_hist_kernel<<<static_cast<unsigned>(na + nb), 256, 0, st>>>(
       oa, ob, static_cast<int>(na), k, hist, dec);
   return cudaGetLastError() == cudaSuccess ? EMU_OK : EMU_ERR_CUDA;
 }
@@ -577,6 +605,7 @@ emu_status_t emu_sel_load(emu_handle_t h, const float* params) {
   if (cudaMemcpy(s->params, params, sizeof(float) * kNParam, cudaMemcpyHostToDevice) != cudaSuccess)
     return EMU_ERR_CUDA;
   s->loaded = true;
+  preload_tri();  // any p may be chosen: no kernel is loaded inside a call
   return EMU_OK;
 }
 
@@ -634,13 +663,15 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
   View v;
   normalize(layout, m, n, A, lda, B, ldb, &v);
   // device: features | histograms | probe indices | probe results [ref (hi,
-  // lo) | sum |a||b|] | row and column maxima; pinned host memory:
+  // lo) | sum |a||b|] | row and column maxima | digit sums; pinned host memory:
   // features, probabilities | probe results with the C entries
   const int pc = std::max(probe, 1);
   const size_t idx_bytes = (8 * static_cast<size_t>(pc) + 255) / 256 * 256;
   const size_t off_hist = 1024, off_idx = off_hist + feat_scratch(v), off_res = off_idx + idx_bytes;
   const size_t off_max = off_res + (24 * static_cast<size_t>(pc) + 255) / 256 * 256;
-  const size_t dev_need = off_max + 8 * static_cast<size_t>(v.M + v.N);
+  const size_t max_bytes = (8 * static_cast<size_t>(v.M + v.N) + 15) / 16 * 16;
+  const size_t zero_bytes = max_bytes + (scheme_II ? 0 : 4 * EMU_P_MAX * static_cast<size_t>(v.M + v.N) + 15) / 16 * 16;
+  const size_t dev_need = off_max + zero_bytes;
   const size_t host_need = 1024 + 32 * static_cast<size_t>(pc);
   if (dev_need > ss->dev_bytes) {
     if (ss->dev) cudaFree(ss->dev);
@@ -674,31 +705,27 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
   auto* d_ab = d_ref + 2 * pc;
   auto* maxA = reinterpret_cast<unsigned long long*>(ss->dev + off_max);
   auto* maxB = maxA + v.M;
+  auto* sums = reinterpret_cast<int32_t*>(ss->dev + off_max + max_bytes);  // digit sums of Scheme I's first attempt
   auto* h_dec = reinterpret_cast<float*>(ss->host);
   auto* h_res = reinterpret_cast<double*>(ss->host + 1024);
   const bool loaded = scheme_II ? ss->loaded_II : ss->loaded;
-  // The decision (features and network, on sampled vectors) and then the
-  // probe's double-double reference sums run on the side stream; the
+  // The decision (features and network, on sampled vectors), then the
   // exponent scan of the whole operands, which every attempt's product needs
-  // whatever p it uses, runs beside them on the caller's stream, so that the
-  // host waits for the decision while the GPU scans.
-  if (cudaEventRecord(ss->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ss->side, ss->ev_fork, 0) != cudaSuccess)
-    return EMU_ERR_CUDA;
-  emu_status_t s = features_impl(v, k, tol, 64, reinterpret_cast<float*>(ss->dev), ss->dev + off_hist, ss->side,
-                                 true, loaded ? (scheme_II ? ss->params_II : ss->params) : nullptr, h_dec);
+  // whatever p it uses: the GPU scans while the host reads the decision and
+  // enqueues the product.
+  emu_status_t s = features_impl(v, k, tol, 64, reinterpret_cast<float*>(ss->dev), ss->dev + off_hist, st, true,
+                                 loaded ? (scheme_II ? ss->params_II : ss->params) : nullptr, h_dec, reinterpret_cast<uint4*>(maxA),
+                                 static_cast<int64_t>(zero_bytes / 16));
   if (s != EMU_OK) return s;
-  if (cudaEventRecord(ss->ev_decide, ss->side) != cudaSuccess) return EMU_ERR_CUDA;
+  if (cudaEventRecord(ss->ev_decide, st) != cudaSuccess) return EMU_ERR_CUDA;
   trace_begin(h, PH_SCAN, st);
-  launch_scan<double>(static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, k, 1, maxA, h->status, st);
-  launch_scan<double>(static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+  launch_scan<double>(static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, maxA,
+                      static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
   trace_end(h, PH_SCAN, st, 2);
-  if (probe > 0) {
-    probe_idx_kernel<<<1, 1, 0, ss->side>>>(
-        0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(m * 1315423911u + n * 2654435761u + k), m, n, probe, d_idx);
-    s = emu_probe_dd(h, layout, m, n, k, A, lda, B, ldb, probe, d_idx, d_ref, d_ab, ss->side);
-    if (s != EMU_OK) return s;
-    if (cudaEventRecord(ss->ev_probe, ss->side) != cudaSuccess) return EMU_ERR_CUDA;
-  }
+  // the probe's side stream starts after the caller's earlier work
+  if (probe > 0 && (cudaEventRecord(ss->ev_fork, st) != cudaSuccess ||
+                    cudaStreamWaitEvent(ss->side, ss->ev_fork, 0) != cudaSuccess))
+    return EMU_ERR_CUDA;
   if (cudaEventSynchronize(ss->ev_decide) != cudaSuccess) return EMU_ERR_CUDA;
   const float* f = h_dec;
   const float* pr = f + 128;
@@ -724,13 +751,21 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
   }
   for (int attempt = 0; attempt < 3; ++attempt) {
     s = dgemm_scanned(h, layout, m, n, k, alpha, A, lda, B, ldb, C, ldc,
-                      scheme_II ? EMU_SCHEME_II_NORM : EMU_SCHEME_I, p, maxA, maxB, stream);
+                      scheme_II ? EMU_SCHEME_II_NORM : EMU_SCHEME_I, p, maxA, maxB,
+                      scheme_II || attempt > 0 ? nullptr : sums, stream);
     if (s != EMU_OK) return s;
     *p_used = p;
     if (probe == 0) return EMU_OK;
+    if (attempt == 0) {
+      // enqueued behind the product, so that its launches do not delay it
+      probe_idx_kernel<<<1, 1, 0, ss->side>>>(
+          0x9E3779B97F4A7C15ull ^ static_cast<uint64_t>(m * 1315423911u + n * 2654435761u + k), m, n, probe, d_idx);
+      s = emu_probe_dd(h, layout, m, n, k, A, lda, B, ldb, probe, d_idx, d_ref, d_ab, ss->side);
+      if (s != EMU_OK) return s;
+      if (cudaEventRecord(ss->ev_probe, ss->side) != cudaSuccess) return EMU_ERR_CUDA;
+    }
     if (attempt == 0 && cudaStreamWaitEvent(st, ss->ev_probe, 0) != cudaSuccess) return EMU_ERR_CUDA;
-    judge_kernel<<<(probe + 127) / 128, 128, 0, st>>>(C, ldc, layout != EMU_ROW_MAJOR, probe, d_idx, d_ref, d_ab,
-                                                      h_res);
+    judge_kernel<<<1, 256, 0, st>>>(C, ldc, layout != EMU_ROW_MAJOR, probe, d_idx, d_ref, d_ab, h_res);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return EMU_ERR_CUDA;
     const double* ref = h_res;
     const double* ab = ref + 2 * probe;

@@ -24,16 +24,6 @@ namespace emu {
 
 // ------------------------------------------------------------------ loads
 template <typename T>
-__device__ __forceinline__ uint64_t load_absbits(const T* p);
-template <>
-__device__ __forceinline__ uint64_t load_absbits<double>(const double* p) {
-  return dbits(__ldg(p)) & 0x7FFFFFFFFFFFFFFFull;
-}
-template <>
-__device__ __forceinline__ uint64_t load_absbits<float>(const float* p) {
-  return dbits(static_cast<double>(__ldg(p))) & 0x7FFFFFFFFFFFFFFFull;  // exact widening
-}
-template <typename T>
 __device__ __forceinline__ uint64_t load_bits(const T* p);
 template <>
 __device__ __forceinline__ uint64_t load_bits<double>(const double* p) {
@@ -45,70 +35,23 @@ __device__ __forceinline__ uint64_t load_bits<float>(const float* p) {
 }
 
 // ------------------------------------------------------------------ scan
-// Vector r, element h of operand X: kcontig -> X[(r*ld + h)*cw + part],
+// Vector r, element h of an operand: kcontig -> X[(r*ld + h)*cw + part],
 // else X[(h*ld + r)*cw + part]; cw = 2 for complex (both parts scanned).
 // seg: elements of a vector per block row (K segment), chosen by the launcher.
-template <typename T, bool KCONTIG>
-__global__ void scan_kernel(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int cw, int64_t seg,
-                            unsigned long long* __restrict__ maxbits, int* status) {
-  if (KCONTIG) {
-    // one warp per (row, K segment)
-    int lane = threadIdx.x & 31;
-    int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= rows) return;
-    int64_t len = k * cw;
-    int64_t h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    int64_t h1 = h0 + seg < len ? h0 + seg : len;
-    const T* row = X + r * ld * cw;
-    uint64_t mx = 0;
-    for (int64_t h = h0 + lane; h < h1; h += 32) {
-      uint64_t v = load_absbits(row + h);
-      mx = v > mx ? v : mx;
-    }
-    for (int o = 16; o; o >>= 1) {
-      uint64_t w = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = w > mx ? w : mx;
-    }
-    if (lane == 0 && h0 < h1) {
-      atomicMax(maxbits + r, static_cast<unsigned long long>(mx));
-      if (mx >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
-    }
-  } else {
-    // block 32 x 8: lanes over vectors (coalesced), 8 row-groups over K
-    int64_t r = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
-    int64_t h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    int64_t h1 = h0 + seg < k ? h0 + seg : k;
-    uint64_t mx = 0;
-    if (r < rows) {
-      for (int64_t h = h0 + threadIdx.y; h < h1; h += blockDim.y) {
-        const T* p = X + (h * ld + r) * cw;
-        uint64_t v = load_absbits(p);
-        mx = v > mx ? v : mx;
-        if (cw == 2) {
-          uint64_t w = load_absbits(p + 1);
-          mx = w > mx ? w : mx;
-        }
-      }
-    }
-    __shared__ uint64_t red[8][32];
-    red[threadIdx.y][threadIdx.x] = mx;
-    __syncthreads();
-    if (threadIdx.y == 0 && r < rows) {
-      for (int q = 1; q < blockDim.y; ++q) mx = red[q][threadIdx.x] > mx ? red[q][threadIdx.x] : mx;
-      if (h0 < h1) {
-        atomicMax(maxbits + r, static_cast<unsigned long long>(mx));
-        if (mx >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
-      }
-    }
-  }
-}
+// One launch scans both operands of a product (the blocks of the first, then
+// those of the second): small products are bound by launches.
+template <typename T>
+struct ScanOperand {
+  const T* X;
+  int64_t ld, rows, k, seg;
+  int64_t vb, blocks;  // blocks per K segment; all blocks
+  unsigned long long* maxbits;
+  int cw;
+  bool kcontig, vec;  // vec: 16-byte loads (every vector starts on a 16-byte boundary)
+};
 
-// The same scan with 16-byte loads, for operands whose vectors start on
-// 16-byte boundaries (base and leading dimension aligned).  A uint4 holds
-// S = 16 / sizeof(T) scalars, CV = S / cw vectors of the strided layout.
 // Float magnitudes are compared on their own bit patterns and the largest
-// is widened once (widening is exact and monotone, so the result is the
-// same as that of the scalar scan).
+// is widened once (widening is exact and monotone).
 template <typename T>
 __device__ __forceinline__ uint64_t widen_absbits(uint64_t b);
 template <>
@@ -139,21 +82,22 @@ __device__ __forceinline__ uint64_t scalar_absbits(T x) {
     return __float_as_uint(x) & 0x7FFFFFFFu;
 }
 
-template <typename T, bool KCONTIG>
-__global__ void scan_vec_kernel(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int cw, int64_t seg,
-                                unsigned long long* __restrict__ maxbits, int* status) {
+// K-contiguous: one warp per (vector, segment of seg scalars); with vec lane
+// l loads the 16 bytes l, l + 32, ..
+template <typename T>
+__device__ __forceinline__ void scan_kcontig(const ScanOperand<T>& op, int64_t bx, int64_t by, int* status) {
   constexpr int S = 16 / static_cast<int>(sizeof(T));
-  if (KCONTIG) {
-    // one warp per (row, segment of seg scalars); lane l loads uint4 l, l + 32, ...
-    const int lane = threadIdx.x & 31;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= rows) return;
-    const int64_t len = k * cw, h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    const int64_t h1 = h0 + seg < len ? h0 + seg : len;
-    const T* row = X + r * ld * cw;
+  const int lane = threadIdx.x & 31;
+  const int64_t r = bx * 8 + (threadIdx.x >> 5);
+  if (r >= op.rows) return;
+  const int64_t len = op.k * op.cw, h0 = by * op.seg;
+  const int64_t h1 = h0 + op.seg < len ? h0 + op.seg : len;
+  const T* row = op.X + r * op.ld * op.cw;
+  uint64_t mx = 0;
+  int64_t h = h0;
+  if (op.vec) {
     const int64_t nv = (h1 - h0) / S;
     const uint4* pv = reinterpret_cast<const uint4*>(row + h0);
-    uint64_t mx = 0;
 #pragma unroll 4
     for (int64_t i = lane; i < nv; i += 32) {
       const uint4 v = __ldg(pv + i);
@@ -163,72 +107,94 @@ __global__ void scan_vec_kernel(const T* __restrict__ X, int64_t ld, int64_t row
         mx = a > mx ? a : mx;
       }
     }
-    for (int64_t h = h0 + nv * S + lane; h < h1; h += 32) {  // ragged end of the row
-      const uint64_t a = scalar_absbits<T>(__ldg(row + h));
-      mx = a > mx ? a : mx;
-    }
-    for (int o = 16; o; o >>= 1) {
-      const uint64_t w = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = w > mx ? w : mx;
-    }
-    if (lane == 0 && h0 < h1) {
-      mx = widen_absbits<T>(mx);
-      atomicMax(maxbits + r, static_cast<unsigned long long>(mx));
-      if (mx >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
-    }
-  } else {
-    // block 32 x 8: lane x loads the CV vectors x*CV .. x*CV + CV - 1 of a
-    // block of 32*CV vectors (512 contiguous bytes per warp and K row);
-    // the 8 row-groups split a K segment of seg
-    const int cv = S / cw;
-    const int64_t rb = static_cast<int64_t>(blockIdx.x) * 32 * cv;
-    const int64_t r = rb + static_cast<int64_t>(threadIdx.x) * cv;
-    const int64_t h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    const int64_t h1 = h0 + seg < k ? h0 + seg : k;
-    uint64_t mx[4] = {0, 0, 0, 0};
-    if (r + cv <= rows) {
+    h += nv * S;  // the ragged end of the row
+  }
 #pragma unroll 4
-      for (int64_t h = h0 + threadIdx.y; h < h1; h += 8) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(X + (h * ld + r) * cw));
+  for (h += lane; h < h1; h += 32) {
+    const uint64_t a = scalar_absbits<T>(__ldg(row + h));
+    mx = a > mx ? a : mx;
+  }
+  for (int o = 16; o; o >>= 1) {
+    const uint64_t w = __shfl_xor_sync(0xffffffffu, mx, o);
+    mx = w > mx ? w : mx;
+  }
+  if (lane == 0 && h0 < h1) {
+    mx = widen_absbits<T>(mx);
+    atomicMax(op.maxbits + r, static_cast<unsigned long long>(mx));
+    if (mx >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
+  }
+}
+
+// K-strided: lanes along the vectors (coalesced), eight row groups split a K
+// segment.  With vec lane x loads the cv vectors x*cv .. (16 bytes), so a
+// block takes 32 cv vectors (512 contiguous bytes per warp and K row), else 32.
+template <typename T>
+__device__ __forceinline__ void scan_kstrided(const ScanOperand<T>& op, int64_t bx, int64_t by, int* status,
+                                              uint64_t (*red)[32 * 4]) {
+  constexpr int S = 16 / static_cast<int>(sizeof(T));
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, cw = op.cw;
+  const int cv = op.vec ? S / cw : 1;
+  const int64_t rb = bx * 32 * cv;
+  const int64_t r = rb + static_cast<int64_t>(tx) * cv;
+  const int64_t h0 = by * op.seg;
+  const int64_t h1 = h0 + op.seg < op.k ? h0 + op.seg : op.k;
+  uint64_t mx[4] = {0, 0, 0, 0};
+  if (op.vec && r + cv <= op.rows) {
+#pragma unroll 4
+    for (int64_t h = h0 + ty; h < h1; h += 8) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(op.X + (h * op.ld + r) * cw));
 #pragma unroll
-        for (int j = 0; j < S; ++j) {  // scalar j belongs to vector j / cw (cw is 1 or 2)
-          const uint64_t a = lane_absbits<T>(v, j);
-          if (cw == 2)
-            mx[j >> 1] = a > mx[j >> 1] ? a : mx[j >> 1];
-          else
-            mx[j] = a > mx[j] ? a : mx[j];
-        }
+      for (int j = 0; j < S; ++j) {  // scalar j belongs to vector j / cw (cw is 1 or 2)
+        const uint64_t a = lane_absbits<T>(v, j);
+        if (cw == 2)
+          mx[j >> 1] = a > mx[j >> 1] ? a : mx[j >> 1];
+        else
+          mx[j] = a > mx[j] ? a : mx[j];
       }
-    } else if (r < rows) {  // the last vectors of the operand: scalar loads
-      for (int64_t h = h0 + threadIdx.y; h < h1; h += 8) {
+    }
+  } else if (r < op.rows) {  // unaligned, or the last vectors of the operand: scalar loads
+#pragma unroll 4
+    for (int64_t h = h0 + ty; h < h1; h += 8) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (c < cv && r + c < rows) {
+      for (int c = 0; c < 4; ++c) {
+        if (c < cv && r + c < op.rows) {
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              if (q < cw) {
-                const uint64_t a = scalar_absbits<T>(__ldg(X + (h * ld + r + c) * cw + q));
-                mx[c] = a > mx[c] ? a : mx[c];
-              }
+          for (int q = 0; q < 2; ++q) {
+            if (q < cw) {
+              const uint64_t a = scalar_absbits<T>(__ldg(op.X + (h * op.ld + r + c) * cw + q));
+              mx[c] = a > mx[c] ? a : mx[c];
             }
           }
         }
       }
     }
-    __shared__ uint64_t red[8][32 * 4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      if (c < cv) red[threadIdx.y][threadIdx.x * cv + c] = mx[c];
-    __syncthreads();
-    const int t = threadIdx.y * 32 + threadIdx.x;
-    if (t < 32 * cv && rb + t < rows && h0 < h1) {
-      uint64_t m = red[0][t];
-      for (int q = 1; q < 8; ++q) m = red[q][t] > m ? red[q][t] : m;
-      m = widen_absbits<T>(m);
-      atomicMax(maxbits + rb + t, static_cast<unsigned long long>(m));
-      if (m >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
-    }
   }
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (c < cv) red[ty][tx * cv + c] = mx[c];
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < 32 * cv && rb + t < op.rows && h0 < h1) {
+    uint64_t m = red[0][t];
+    for (int q = 1; q < 8; ++q) m = red[q][t] > m ? red[q][t] : m;
+    m = widen_absbits<T>(m);
+    atomicMax(op.maxbits + rb + t, static_cast<unsigned long long>(m));
+    if (m >= 0x7FF0000000000000ull) set_status(status, ST_NONFINITE);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) scan_kernel(const __grid_constant__ ScanOperand<T> a,
+                                                   const __grid_constant__ ScanOperand<T> b, int* status) {
+  __shared__ uint64_t red[8][32 * 4];
+  const bool first = blockIdx.x < a.blocks;
+  const ScanOperand<T>& op = first ? a : b;
+  const int64_t blk = first ? blockIdx.x : blockIdx.x - a.blocks;
+  const int64_t bx = blk % op.vb, by = blk / op.vb;
+  if (op.kcontig)
+    scan_kcontig(op, bx, by, status);
+  else
+    scan_kstrided(op, bx, by, status, red);
 }
 
 // ------------------------------------------------------------------ norm scan
@@ -692,45 +658,54 @@ __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X
 // then still have enough loads in flight -- down to `seg_min`, and doubled
 // while the segment count exceeds the grid's y limit.
 static int64_t scan_seg(int64_t vec_blocks, int64_t len, int64_t seg0, int64_t seg_min) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  constexpr int64_t kSms = 152;  // of a GB300
   int64_t seg = seg0;
-  while (seg > seg_min && vec_blocks * ((len + seg - 1) / seg) < 4 * static_cast<int64_t>(sms)) seg >>= 1;
+  while (seg > seg_min && vec_blocks * ((len + seg - 1) / seg) < 4 * kSms) seg >>= 1;
   while ((len + seg - 1) / seg > 65535) seg <<= 1;
   return seg;
 }
 
-template <typename T>
-void launch_scan(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
-                 unsigned long long* maxbits, int* status, cudaStream_t st) {
-  cudaMemsetAsync(maxbits, 0, sizeof(unsigned long long) * (rows > 0 ? rows : 1), st);
-  if (rows == 0 || k == 0) return;
-  // 16-byte loads when every vector starts on a 16-byte boundary
-  const bool vec = (reinterpret_cast<uintptr_t>(X) & 15u) == 0 &&
-                   (static_cast<uint64_t>(ld) * cw * sizeof(T)) % 16 == 0;
-  if (kcontig) {
-    const int64_t len = k * cw, rb = (rows + 7) / 8, seg = scan_seg(rb, len, 2048, 256);
-    dim3 grid(static_cast<unsigned>(rb), static_cast<unsigned>((len + seg - 1) / seg));
-    if (vec)
-      scan_vec_kernel<T, true><<<grid, 256, 0, st>>>(X, ld, rows, k, cw, seg, maxbits, status);
-    else
-      scan_kernel<T, true><<<grid, 256, 0, st>>>(X, ld, rows, k, cw, seg, maxbits, status);
-  } else if (vec) {
-    const int64_t per_block = 32 * static_cast<int64_t>(16 / sizeof(T)) / cw;
-    const int64_t rb = (rows + per_block - 1) / per_block, seg = scan_seg(rb, k, 256, 32);
-    dim3 grid(static_cast<unsigned>(rb), static_cast<unsigned>((k + seg - 1) / seg));
-    scan_vec_kernel<T, false><<<grid, dim3(32, 8), 0, st>>>(X, ld, rows, k, cw, seg, maxbits, status);
-  } else {
-    const int64_t rb = (rows + 31) / 32, seg = scan_seg(rb, k, 256, 32);
-    dim3 grid(static_cast<unsigned>(rb), static_cast<unsigned>((k + seg - 1) / seg));
-    scan_kernel<T, false><<<grid, dim3(32, 8), 0, st>>>(X, ld, rows, k, cw, seg, maxbits, status);
-  }
+__global__ void zero_kernel(uint4* p, int64_t n) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i < n) p[i] = make_uint4(0, 0, 0, 0);
 }
-template void launch_scan<double>(const double*, int64_t, bool, int64_t, int64_t, int,
-                                  unsigned long long*, int*, cudaStream_t);
-template void launch_scan<float>(const float*, int64_t, bool, int64_t, int64_t, int,
-                                 unsigned long long*, int*, cudaStream_t);
+
+void launch_zero(void* p, size_t bytes, cudaStream_t st) {
+  const int64_t n = static_cast<int64_t>((bytes + 15) / 16);
+  if (n > 0) zero_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(static_cast<uint4*>(p), n);
+}
+
+template <typename T>
+static ScanOperand<T> scan_operand(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
+                                   unsigned long long* maxbits) {
+  ScanOperand<T> op{X, ld, rows, k, 0, 1, 0, maxbits, cw, kcontig, false};
+  if (rows == 0 || k == 0) return op;
+  op.vec = (reinterpret_cast<uintptr_t>(X) & 15u) == 0 && (static_cast<uint64_t>(ld) * cw * sizeof(T)) % 16 == 0;
+  const int64_t len = kcontig ? k * cw : k;
+  const int64_t per_block = kcontig ? 8 : op.vec ? 32 * static_cast<int64_t>(16 / sizeof(T)) / cw : 32;
+  op.vb = (rows + per_block - 1) / per_block;
+  op.seg = kcontig ? scan_seg(op.vb, len, 2048, 256) : scan_seg(op.vb, len, 256, 32);
+  op.blocks = op.vb * ((len + op.seg - 1) / op.seg);
+  return op;
+}
+
+template <typename T>
+void launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
+                 int64_t ldB, bool b_kcontig, int64_t N, unsigned long long* maxB, int64_t k, int cw, bool zeroed,
+                 int* status, cudaStream_t st) {
+  if (!zeroed) {
+    if (maxA) cudaMemsetAsync(maxA, 0, sizeof(*maxA) * M, st);
+    if (maxB) cudaMemsetAsync(maxB, 0, sizeof(*maxB) * N, st);
+  }
+  const ScanOperand<T> a = scan_operand(A, ldA, a_kcontig, maxA ? M : 0, k, cw, maxA);
+  const ScanOperand<T> b = scan_operand(B, ldB, b_kcontig, maxB ? N : 0, k, cw, maxB);
+  if (a.blocks + b.blocks == 0) return;
+  scan_kernel<T><<<static_cast<unsigned>(a.blocks + b.blocks), 256, 0, st>>>(a, b, status);
+}
+template void launch_scan<double>(const double*, int64_t, bool, int64_t, unsigned long long*, const double*, int64_t,
+                                  bool, int64_t, unsigned long long*, int64_t, int, bool, int*, cudaStream_t);
+template void launch_scan<float>(const float*, int64_t, bool, int64_t, unsigned long long*, const float*, int64_t,
+                                 bool, int64_t, unsigned long long*, int64_t, int, bool, int*, cudaStream_t);
 
 template <typename T, int P, bool F8>
 static void launch_split_I_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k,

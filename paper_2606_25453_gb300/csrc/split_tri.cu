@@ -1,0 +1,203 @@
+// split_tri.cu -- Scheme I split for the bf16 digit triangle (tri_core.cuh):
+// the recentred digits d_t of every element and the digit sums d_i + d_j as
+// bf16 planes, and the sums of each vector's digits over K.
+//
+// Planes: plane q, vector r, element h at element (q * rows + r) * kpad + h
+// (bf16); kpad is K rounded up to 64, the padding is zero.  Rows are not
+// padded: a row of A only reaches the same row of C.
+//
+// HBM bound: 8 bytes read and 2 per plane written per element (23 planes at
+// p = 8).
+#include "emu_internal.h"
+#include "split_core.cuh"
+#include "tri_core.cuh"
+
+namespace emu {
+namespace {
+
+// Four consecutive K elements of one vector (binary64 bits) to their digits
+// and digit sums; `live` bit q: element q lies inside K (the planes are zero
+// outside).  `dst`: the first element in plane 0; `plane`: plane stride in
+// elements.  sum[t] gains the four digits d_t.
+template <int P>
+__device__ __forceinline__ void digits4(const uint64_t* bits, int E, int nlive, uint16_t* dst, int64_t plane,
+                                        int* sum) {
+  float f[P][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t b[P];
+    slice_digits<P>(bits[q], E, b);
+    const bool live = q < nlive;
+#pragma unroll
+    for (int t = 0; t < P; ++t) {
+      // byte + 128 (slice 0, signed) or the byte itself (tails), then - 128:
+      // 2^23 + u has u in its low mantissa bits
+      const uint32_t u = live ? (t == 0 ? b[t] ^ 0x80u : b[t]) : 128u;
+      sum[t] += static_cast<int>(u) - 128;
+      f[t][q] = __uint_as_float(0x4B000000u | u) - 8388736.0f;
+    }
+  }
+  // integers of magnitude <= 256 are exact bf16 values: the upper half of
+  // the binary32 pattern
+  auto put = [&](int q, float a, float b, float c, float d) {
+    *reinterpret_cast<uint2*>(dst + static_cast<int64_t>(q) * plane) =
+        make_uint2(__byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632u),
+                   __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x7632u));
+  };
+#pragma unroll
+  for (int t = 0; t < P; ++t) put(t, f[t][0], f[t][1], f[t][2], f[t][3]);
+#pragma unroll
+  for (int i = 0; i < P; ++i)
+#pragma unroll
+    for (int j = i + 1; i + j < P; ++j)
+      if (!(i == 0 && j == P - 1))
+        put(tri_cross_plane(P, i, j), f[i][0] + f[j][0], f[i][1] + f[j][1], f[i][2] + f[j][2], f[i][3] + f[j][3]);
+}
+
+__device__ __forceinline__ int live_count(int64_t h0, int64_t k) {
+  return h0 >= k ? 0 : (k - h0 >= 4 ? 4 : static_cast<int>(k - h0));
+}
+
+// K-contiguous source: one warp per (vector, run of `per` groups of 128
+// elements); lane l takes elements 4l .. 4l+3 of each group.
+template <typename T, int P>
+__global__ void __launch_bounds__(256) split_tri_kcontig(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
+                                                         int64_t kpad, int per, int64_t nseg,
+                                                         const unsigned long long* __restrict__ maxbits,
+                                                         uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
+                                                         int32_t* __restrict__ sums, bool vec) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  if (w >= rows * nseg) return;
+  const int64_t r = w / nseg, g0 = (w % nseg) * per;
+  const int E = exp_from_maxbits(maxbits, r, rows);
+  int sum[P];
+#pragma unroll
+  for (int t = 0; t < P; ++t) sum[t] = 0;
+  for (int64_t g = g0; g < g0 + per; ++g) {
+    const int64_t h0 = g * 128 + lane * 4;
+    if (h0 >= kpad) break;
+    uint64_t bits[4];
+    load4_kcontig(X + r * ld, h0, k, true, vec, bits);
+    digits4<P>(bits, E, live_count(h0, k), planes + r * kpad + h0, rows * kpad, sum);
+  }
+  __syncwarp();
+  int mine = 0;
+#pragma unroll
+  for (int t = 0; t < P; ++t) {
+    const int s = __reduce_add_sync(0xFFFFFFFFu, sum[t]);
+    if (lane == t) mine = s;
+  }
+  if (lane < P) atomicAdd(sums + lane * rows + r, mine);
+  if (g0 == 0 && lane == 0) E_out[r] = E;
+}
+
+// K-strided source: a block takes 32 vectors x `per` groups of 128 elements
+// through a shared-memory tile; warp w packs vectors w, w + 8, ..
+template <typename T, int P>
+__global__ void __launch_bounds__(256) split_tri_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
+                                                          int64_t kpad, int per,
+                                                          const unsigned long long* __restrict__ maxbits,
+                                                          uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
+                                                          int32_t* __restrict__ sums, bool vec) {
+  __shared__ uint64_t tile[32][133];
+  __shared__ int ssum[32][P];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * 32;
+  for (int i = threadIdx.x; i < 32 * P; i += 256) (&ssum[0][0])[i] = 0;
+  for (int64_t g = static_cast<int64_t>(blockIdx.y) * per; g < (static_cast<int64_t>(blockIdx.y) + 1) * per; ++g) {
+    const int64_t hbase = g * 128;
+    if (hbase >= kpad) break;
+    __syncthreads();  // the previous group is done with the tile
+    fill_tile_strided(tile, X, ld, rows, k, r0, hbase, vec);
+    __syncthreads();
+    const int64_t h0 = hbase + lane * 4;
+    for (int rl = warp; rl < 32; rl += 8) {
+      const int64_t r = r0 + rl;
+      if (r >= rows) break;
+      int sum[P];
+#pragma unroll
+      for (int t = 0; t < P; ++t) sum[t] = 0;
+      if (h0 < kpad) {
+        const int E = exp_from_maxbits(maxbits, r, rows);
+        uint64_t bits[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bits[q] = tile[rl][q * 33 + lane];
+        digits4<P>(bits, E, live_count(h0, k), planes + r * kpad + h0, rows * kpad, sum);
+        if (h0 == 0) E_out[r] = E;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        const int s = __reduce_add_sync(0xFFFFFFFFu, sum[t]);
+        if (lane == t) ssum[rl][t] += s;  // only this warp, this lane touches it
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 32 * P; i += 256) {
+    const int rl = i % 32, t = i / 32;
+    if (r0 + rl < rows) atomicAdd(sums + t * rows + r0 + rl, ssum[rl][t]);
+  }
+}
+
+template <typename T, int P>
+void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, const unsigned long long* maxbits,
+              uint16_t* planes, int32_t* E, int32_t* sums, int num_sms, cudaStream_t st) {
+  const int64_t kpad = (k + 63) / 64 * 64, ngroups = (kpad + 127) / 128;
+  const bool vec = vec16_ok(X, ld);
+  // groups per warp (block): up to 8, as long as the grid keeps about eight
+  // blocks per SM (fewer atomics on the digit sums, no idle SMs)
+  const int64_t units = kcontig ? (rows + 7) / 8 : (rows + 31) / 32;
+  int per = 8;
+  while (per > 1 && units * ((ngroups + per - 1) / per) < 8 * static_cast<int64_t>(num_sms)) per >>= 1;
+  int64_t nseg = (ngroups + per - 1) / per;
+  if (kcontig) {
+    const int64_t blocks = (rows * nseg + 7) / 8;
+    split_tri_kcontig<T, P><<<static_cast<unsigned>(blocks), 256, 0, st>>>(X, ld, rows, k, kpad, per, nseg, maxbits,
+                                                                           planes, E, sums, vec);
+  } else {
+    while (nseg > 65535) {
+      per *= 2;
+      nseg = (ngroups + per - 1) / per;
+    }
+    const dim3 grid(static_cast<unsigned>((rows + 31) / 32), static_cast<unsigned>(nseg));
+    split_tri_kstrided<T, P><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+  }
+}
+
+template <int P>
+void preload_p() {
+  cudaFuncAttributes a;
+  cudaFuncGetAttributes(&a, split_tri_kcontig<double, P>);
+  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P>);
+  if constexpr (P < kTriMaxP) preload_p<P + 1>();
+}
+
+}  // namespace
+
+void preload_split_tri() { preload_p<1>(); }
+
+template <typename T>
+void launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+                      const unsigned long long* maxbits, uint16_t* planes, int32_t* E, int32_t* sums, int num_sms,
+                      cudaStream_t st) {
+  if (rows == 0 || k == 0) return;
+  switch (p) {
+#define EMU_CASE(PP)                                                                        \
+  case PP:                                                                                  \
+    launch_p<T, PP>(X, ld, kcontig, rows, k, maxbits, planes, E, sums, num_sms, st);        \
+    break;
+    EMU_CASE(1) EMU_CASE(2) EMU_CASE(3) EMU_CASE(4) EMU_CASE(5) EMU_CASE(6)
+    EMU_CASE(7) EMU_CASE(8) EMU_CASE(9) EMU_CASE(10) EMU_CASE(11) EMU_CASE(12)
+#undef EMU_CASE
+    default:
+      break;
+  }
+}
+template void launch_split_tri<double>(const double*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
+                                       uint16_t*, int32_t*, int32_t*, int, cudaStream_t);
+template void launch_split_tri<float>(const float*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
+                                      uint16_t*, int32_t*, int32_t*, int, cudaStream_t);
+
+}  // namespace emu

@@ -75,4 +75,159 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
+constexpr uint32_t kTmemAll = 512;  // TMEM columns of one SM
+
+// Instruction descriptor: bf16 x bf16 -> F32, both K-major, M x N.
+__device__ __forceinline__ uint32_t idesc_bf16(int M, int N) {
+  return (1u << 4)                                  // D format F32
+         | (1u << 7) | (1u << 10)                   // A, B format BF16
+         | (static_cast<uint32_t>(N >> 3) << 17)    // N / 8
+         | (static_cast<uint32_t>(M >> 4) << 24);   // M / 16
+}
+
+template <bool PAIR>
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t accumulate) {
+  if constexpr (PAIR)
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+  else
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrive on the barrier at shared::cluster address `bar` (this CTA's or the
+// peer's) once every MMA issued so far by this thread has completed.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+template <bool PAIR>
+__device__ __forceinline__ void tmem_alloc_all(uint32_t* slot) {
+  if constexpr (PAIR) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                 "r"(kTmemAll)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  } else {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                 "r"(kTmemAll)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+}
+
+template <bool PAIR>
+__device__ __forceinline__ void tmem_free_all(uint32_t tmem) {
+  if constexpr (PAIR)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemAll) : "memory");
+  else
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemAll) : "memory");
+}
+
+// shared::cluster address of the object at shared::cta address `saddr` in
+// the CTA of the cluster with rank `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+
+// 2D tiled TMA load into this CTA's shared memory, completion counted on the
+// barrier at shared::cluster address `bar`, which may be the peer CTA's.
+__device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const void* desc, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(desc)), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+
+// Arrive (release, cluster scope) on the barrier at shared::cluster address `bar`.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_try_wait_acq_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// Abort flags: this CTA's, and (pairs) the shared::cluster address of the
+// peer's, so that a role that gives up stops both CTAs of the pair.
+struct AbortFlag {
+  volatile int* local;
+  uint32_t peer;  // 0: no peer
+};
+
+__device__ __forceinline__ void raise_abort(const AbortFlag& ab) {
+  *ab.local = 1;
+  if (ab.peer) asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(ab.peer), "r"(1u) : "memory");
+}
+
+// Bounded wait unless the pair already gave up; false means "stop".  With
+// `cluster_acq` the wait acquires at cluster scope (arrivals from the peer).
+__device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, const AbortFlag& ab, int* status,
+                                          bool cluster_acq = false) {
+  // fast path: the phase is already complete (no abort-flag load on the way)
+  if (cluster_acq ? mbar_try_wait_acq_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+  if (*ab.local) return false;
+  if (cluster_acq) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait_acq_cluster(bar, parity)) {
+      if (*ab.local) return false;
+      if (clock64() - t0 > kWaitCycles) {
+        set_status(status, ST_TIMEOUT);
+        raise_abort(ab);
+        return false;
+      }
+    }
+    return true;
+  }
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity)) {
+    if (*ab.local) return false;
+    if (clock64() - t0 > kWaitCycles) {
+      set_status(status, ST_TIMEOUT);
+      raise_abort(ab);
+      return false;
+    }
+  }
+  return true;
+}
+
+// 16 consecutive 32-bit TMEM columns of this thread's lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+// Tile order of the bf16 kernels: groups of 16 row tiles walk the columns
+// together, so that the operand tiles of a group are reused from L2.
+__device__ __forceinline__ void tile_coords16(int tile, int tiles_m, int tiles_n, int& tm, int& tn) {
+  constexpr int G = 16;  // row tiles per group of the tile order (16: 1-2 % faster than 8 at n = 8192-16384)
+  int per_group = G * tiles_n;
+  int g = tile / per_group;
+  int first = g * G;
+  int gsz = tiles_m - first < G ? tiles_m - first : G;
+  int in = tile - g * per_group;
+  tm = first + in % gsz;
+  tn = in / gsz;
+}
+
 }  // namespace emu
