@@ -58,9 +58,11 @@
  *  - Environment (read once per process; results do not depend on it):
  *    EMU_II_ENGINE=mma runs Scheme II on the INT8 mma.sync kernel instead of
  *    the bf16 tcgen05 one; EMU_F8_ENGINE=mma runs E4M3 slices on the warp
- *    level instead of tcgen05; EMU_II_CLUSTER=2 runs the bf16 Scheme II
- *    residue GEMM on CTA pairs (256 x 256 tiles, tcgen05.mma.cta_group::2)
- *    instead of single CTAs (128 x 256 tiles); EMU_FAULT=alloc makes every
+ *    level instead of tcgen05; EMU_I_ENGINE=mma runs INT8 slices on the
+ *    mma.sync kernel instead of as bf16 digit products (tcgen05);
+ *    EMU_II_CLUSTER=1 or 2 runs the bf16 Scheme II residue GEMM always on
+ *    single CTAs (128 x 256 tiles) or always on CTA pairs (256 x 256 tiles,
+ *    tcgen05.mma.cta_group::2) instead of choosing by size; EMU_FAULT=alloc makes every
  *    library-owned workspace allocation fail and EMU_FAULT=launch every
  *    fused GEMM launch of a product fail with EMU_ERR_CUDA (host-side fault
  *    injection; nothing is run on the device in its place).

@@ -860,7 +860,7 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   // rows (A) and 256 / cluster rows (B: a CTA pair loads half of each
   // 256-column tile per CTA); INT8: 32-byte boxes of 64 / 32 rows
   const uint64_t row_bytes = static_cast<uint64_t>(pl.cols) * (tc ? 2 : 1);
-  const int cluster = tc ? gemm_II_tc_cluster() : 1;
+  const int cluster = tc ? gemm_II_tc_cluster(v.M, k) : 1;
   if (!make_tmap_i8(&ta, resA, row_bytes, static_cast<uint64_t>(pl.rows_a) * nm * nsets,
                     tc ? static_cast<uint32_t>(gemm_II_tc_tile_m()) : 64, tc ? 128 : 32) ||
       !make_tmap_i8(&tb, resB, row_bytes, static_cast<uint64_t>(pl.rows_b) * nm * nsets,
@@ -871,6 +871,7 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   a.descB = &tb;
   a.M = static_cast<int>(v.M);
   a.N = static_cast<int>(v.N);
+  a.K = static_cast<int>(k);
   a.nk32 = static_cast<int>(pl.cols / 32);
   a.rowsA_pad = static_cast<int>(pl.rows_a);
   a.rowsB_pad = static_cast<int>(pl.rows_b);

@@ -184,7 +184,7 @@ cudaError_t launch_gemm_II_tc(int out_mode, const GemmIIArgs& a, const ModTables
 int gemm_II_tc_tile_m();
 int gemm_II_tc_tile_n();
 size_t gemm_II_tc_residue_bytes(int64_t M, int64_t N, int nm, bool is_complex, int cluster);
-int gemm_II_tc_cluster();
+int gemm_II_tc_cluster(int64_t M, int64_t K);
 
 // Tensor map for a row-major byte matrix [rows][cols] read in boxes of
 // box_bytes x box_rows: 32-byte boxes with 32-byte swizzling, or 128-byte

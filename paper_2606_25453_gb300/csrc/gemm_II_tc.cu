@@ -6,7 +6,7 @@
 // products of two of them (|r_a r_b| <= 2^14) are exact, and an FP32 sum of
 // up to 960 such products stays an exact integer (|sum| <= 960 * 2^14 <
 // 2^24).  So every per-modulus product of Eq. (6) runs as a bf16 GEMM on the
-// 5th-generation tensor cores in K segments of 960, and the result is
+// 5th-generation tensor cores in K segments of 896 (CTA pairs) or 960, and the result is
 // bit-identical to the INT8 kernel's.
 //
 // The work is modulus-major, as in the paper's Scheme II kernel (Sec. IV):
@@ -21,69 +21,31 @@
 // symmetric range, rounds it once to binary64, scales it back and applies
 // the BLAS update (3M combination of Eq. (16) for complex input).
 //
-// GEMM tile, PAIR form: 256 rows x 256 columns on a pair of CTAs
-// (a cluster of two on neighbouring SMs) with tcgen05.mma.cta_group::2: one
-// 256 x 256 x 16 MMA per K-step, issued by the even CTA, reads the 128 rows
-// of A that each CTA holds and the 256 columns of B of which each CTA holds
-// half, and leaves rows 0-127 of the product in the even CTA's TMEM and
-// rows 128-255 in the odd one's.  Each CTA's TMA fills only its own shared
-// memory (its A rows and its half of B) and counts the bytes on the even
-// CTA's stage barrier; the MMA commits release the stage in both CTAs.  Per
-// K-step an SM then reads 8 KB of operands from shared memory and receives
-// 8 KB by TMA, against 12 + 12 KB for a 128 x 256 tile on one CTA, whose
-// shared-memory traffic (192 B per clock at full tensor rate against 128 B
-// per clock of bandwidth) caps it near two thirds of the tensor peak; the
-// smaller stages also fit six deep instead of four.  Measured on GB300 the
-// pair form is nevertheless not faster than the single-CTA form (128 x 256
-// tile, tcgen05.mma.cta_group::1), which is the default; the pair form runs
-// with EMU_II_CLUSTER=2.
-//
-// Two FP32 accumulators take all 512 TMEM columns of each CTA and alternate
-// between K segments, so the MMAs of one segment overlap the reduction of
-// the last.  Roles (320 threads per CTA): warps 0-7 drain (warp w: TMEM
-// lanes = tile rows 32 (w % 4) .., columns 128 (w / 4) .. +127; each
-// finished segment is added to a running residue, four per register, with
-// FP32 arithmetic only), warp 8 lane 0 TMA, warp 9 TMEM allocation and
-// (lane 0 of the even CTA) MMAs.
-// All waits are bounded; a timeout sets the status word, raises the abort
-// flag of both CTAs of a pair for the other roles, and the TMEM is still
-// released.
+// The main loop and its two forms (CTA pairs, single CTAs): bf16_gemm.cuh.
 #include <cstdlib>
 #include <type_traits>
 
+#include "bf16_gemm.cuh"
 #include "crt_core.cuh"
-#include "emu_internal.h"
-#include "tc_core.cuh"
 
 namespace emu {
 namespace {
 
-constexpr int kBM = 128, kBN = 256;  // accumulator tile of one CTA: TMEM lanes x FP32 columns
-constexpr int kThreads = 320;
-constexpr int kDrainWarps = 8;
-constexpr int kProducerWarp = 8, kMmaWarp = 9;
-constexpr int kSegStages = 15;  // 64-wide K chunks per exact FP32 segment (960 * 2^14 < 2^24)
-static_assert(kSegStages * 64 * 16384 < (1 << 24), "segment sums must stay exact in FP32");
+using bf16g::kBM;
+using bf16g::kBN;
 
-template <bool PAIR>
-struct CfgII {
-  static constexpr int kRowsB = PAIR ? kBN / 2 : kBN;  // B rows (output columns) this CTA loads
-  static constexpr int kBlkA = kBM * 128;               // one K chunk: 128 rows x 64 bf16, 128-byte rows
-  static constexpr int kBlkB = kRowsB * 128;
-  static constexpr int kStageBytes = kBlkA + kBlkB;
-  static constexpr int kStages = PAIR ? 6 : 4;
-  static constexpr int kSmem = kStages * kStageBytes + 1024 + 256;
-  static_assert(kSmem <= 232448, "shared memory");
-  static_assert(kStageBytes % 1024 == 0, "stages keep the 1024-byte swizzle alignment");
-};
+// Residue GEMM, 14 moduli, single / pair in us: n = 2048, K = 512: 66 / 80,
+// 896: 94 / 87, 1024: 112 / 108, 2048: 177 / 161; n = 4096, K = 512: 228 /
+// 285, 896: 338 / 299, 3072: 916 / 813; n = 1024, K = 896: 31 / 31.
+constexpr int64_t kPairMinK = 896;
 
 struct KParamsIITC {
   CUtensorMap tA;  // bf16 planes as bytes: 128-byte x 128-row boxes, 128-byte swizzle
   CUtensorMap tB;  // 128-byte x (256 or 128)-row boxes
   int nst;         // 64-wide K chunks per plane
   int tiles_m;     // 128-row tiles of the residue matrices (even with CTA pairs)
-  int tiles_mu;    // row units of the work list: 256-row pair tiles or 128-row tiles
   int tiles_n;     // 256-column tiles
+  int N;
   int nplanes;     // NSET * nm residue planes (plane p = set * nm + l)
   int nm;
   int rowsA_pad, rowsB_pad;
@@ -97,273 +59,131 @@ struct KParamsIITC {
 // (p16: the symmetric residue of 2^16 mod m, |p16| <= 128).
 __device__ __forceinline__ int fold16(int x, int p16) { return (x >> 16) * p16 + (x & 0xFFFF); }
 
-// x mod m in [0, m) for |x| < 2^23: the quotient estimate floor(RN(x) *
-// RN(1/m)) errs by at most one (|x / m| < 2^16, relative error < 2^-22),
-// and one correction each way finishes.
-__device__ __forceinline__ int mod_small(int x, int m, float inv) {
-  const int q = __float2int_rd(__fmul_rn(__int2float_rn(x), inv));
-  int r = x - q * m;
-  if (r < 0) r += m;
-  if (r >= m) r -= m;
-  return r;
-}
-
-// Work item i: plane p = i / (tiles per plane), then the tile; tm is this
-// CTA's 128-row tile (a pair's rows 0-127 on the even CTA, 128-255 on the
-// odd one).
-template <bool PAIR>
-__device__ __forceinline__ void item_coords(const KParamsIITC& kp, int item, int crank, int& p, int& tm, int& tn) {
-  const int per_plane = kp.tiles_mu * kp.tiles_n;
-  p = item / per_plane;
-  int tu;
-  tile_coords16(item - p * per_plane, kp.tiles_mu, kp.tiles_n, tu, tn);
-  tm = PAIR ? 2 * tu + crank : tu;
-}
-
-template <bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1)
-    gemm_II_tc_kernel(const __grid_constant__ KParamsIITC kp, const __grid_constant__ ModTables mt) {
-  using Cfg = CfgII<PAIR>;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* smem = smem_raw + (base - raw);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Cfg::kStages * Cfg::kStageBytes);
-  uint64_t* empty = full + Cfg::kStages;
-  uint64_t* acc_full = empty + Cfg::kStages;  // two accumulators
-  uint64_t* acc_empty = acc_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
-  volatile int* abort_local = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t crank = PAIR ? cluster_ctarank() : 0u;  // 0: the pair's MMA-issuing CTA
-  const bool leader = crank == 0;
-  const int cid = PAIR ? static_cast<int>(cluster_id_x()) : static_cast<int>(blockIdx.x);
-  const int ncl = PAIR ? static_cast<int>(cluster_count_x()) : static_cast<int>(gridDim.x);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < Cfg::kStages; ++s) {
-      mbar_init(&full[s], 1);   // the even CTA's expect-tx arrival (+ the bytes of both CTAs)
-      mbar_init(&empty[s], 1);  // one MMA commit
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], PAIR ? 2 * kDrainWarps : kDrainWarps);  // one arrival per drain warp
-    }
-    *abort_local = 0;
-    fence_mbar_init();
-  }
-  if (warp == kMmaWarp) {  // the whole warp allocates the tensor memory (both CTAs of a pair)
-    tmem_alloc_all<PAIR>(tmem_slot);
-    tc_fence_before();
-  }
-  // barriers and flags initialised in both CTAs before either touches the peer's
-  if (PAIR)
-    cluster_sync_all();
-  else
-    __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  AbortFlag ab;
-  ab.local = abort_local;
-  ab.peer = PAIR ? cluster_addr(smem_u32(const_cast<int*>(abort_local)), crank ^ 1u) : 0u;
-
-  const int nitems = kp.nplanes * kp.tiles_mu * kp.tiles_n;
-  const int my_items = cid < nitems ? (nitems - 1 - cid) / ncl + 1 : 0;
-  const int nseg = (kp.nst + kSegStages - 1) / kSegStages;
-
-  if (warp == kProducerWarp) {
-    // ---------------------------------------------------------------- producer (both CTAs)
-    if (lane == 0) {
-      tma_prefetch_desc(&kp.tA);
-      tma_prefetch_desc(&kp.tB);
-      uint32_t j = 0;
-      bool stop = false;
-      for (int t = 0; t < my_items && !stop; ++t) {
-        int p, tm, tn;
-        item_coords<PAIR>(kp, cid + t * ncl, static_cast<int>(crank), p, tm, tn);
-        const int ya = p * kp.rowsA_pad + tm * kBM;
-        const int yb = p * kp.rowsB_pad + tn * kBN + static_cast<int>(crank) * Cfg::kRowsB;
-        for (int ks = 0; ks < kp.nst; ++ks, ++j) {
-          const uint32_t stage = j % Cfg::kStages;
-          if (j >= static_cast<uint32_t>(Cfg::kStages) &&
-              !wait_pair(&empty[stage], ((j / Cfg::kStages) & 1u) ^ 1u, ab, kp.status)) {
-            stop = true;
-            break;
-          }
-          uint8_t* sA = smem + stage * Cfg::kStageBytes;
-          if (PAIR) {
-            // both CTAs' bytes are counted on the even CTA's barrier
-            const uint32_t bar = cluster_addr(smem_u32(&full[stage]), 0u);
-            if (leader) mbar_arrive_expect_tx(&full[stage], 2 * Cfg::kStageBytes);
-            tma_load_2d_pair(sA, &kp.tA, bar, ks * 128, ya);
-            tma_load_2d_pair(sA + Cfg::kBlkA, &kp.tB, bar, ks * 128, yb);
-          } else {
-            mbar_arrive_expect_tx(&full[stage], Cfg::kStageBytes);
-            tma_load_2d(sA, &kp.tA, &full[stage], ks * 128, ya);
-            tma_load_2d(sA + Cfg::kBlkA, &kp.tB, &full[stage], ks * 128, yb);
-          }
-        }
-      }
-      // Drain: wait until the last MMA commits have arrived on this CTA's
-      // stage barriers (a pair's odd CTA gets them from the even one), so
-      // that none lands after the CTA exits.
-      if (!stop && PAIR) {
-        for (uint32_t jj = j; jj < j + Cfg::kStages; ++jj) {
-          if (jj < static_cast<uint32_t>(Cfg::kStages)) continue;
-          const uint32_t stage = jj % Cfg::kStages;
-          if (!wait_pair(&empty[stage], ((jj / Cfg::kStages) & 1u) ^ 1u, ab, kp.status)) break;
-        }
-      }
-    }
-    __syncwarp();
-  } else if (warp == kMmaWarp) {
-    // ---------------------------------------------------------------- MMA issuer (even CTA of a pair)
-    if (lane == 0 && leader) {
-      const uint32_t idesc = idesc_bf16(PAIR ? 2 * kBM : kBM, kBN);
-      const uint32_t peer = 1u;
-      const uint32_t total = static_cast<uint32_t>(my_items) * static_cast<uint32_t>(kp.nst);
-      uint32_t it = 0, seg = 0;
-      bool stop = false;
-      bool ready = false;  // the probe after the previous stage's MMAs already saw this stage's data
-      for (int t = 0; t < my_items && !stop; ++t)
-        for (int ks = 0; ks < kp.nst; ++ks, ++it) {
-          const bool first = ks % kSegStages == 0;
-          const uint32_t b = seg & 1u;
-          if (first && seg >= 2) {  // the drain warps must have read this accumulator's last segment
-            if (!wait_pair(&acc_empty[b], ((seg >> 1) - 1) & 1u, ab, kp.status, PAIR)) {
-              stop = true;
-              break;
-            }
-            tc_fence_after();
-          }
-          const uint32_t stage = it % Cfg::kStages;
-          if (!ready && !wait_pair(&full[stage], (it / Cfg::kStages) & 1u, ab, kp.status)) {
-            stop = true;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sA = base + stage * Cfg::kStageBytes;
+// Residues in [0, m) of four sums |x| <= 2^21.3 (fold16's output), one byte
+// each, in FP32 arithmetic without conversions or corrections: with x / m =
+// n + j / m, y = x / m + 1 / (2m) - 1/2 lies 1 / (2m) >= 0.0019 inside
+// (n - 1/2, n + 1/2), and its computed value errs by less than 2^-10 (inv by
+// 2^-25 of |x / m| < 2^13.9, the FMA by half an ulp, 2^-11), so rounding y to
+// an integer gives n and r = x - n m is exact.
+__device__ __forceinline__ uint32_t mod4(const int* x, float inv, float off, float negm) {
+  uint32_t r[4];
 #pragma unroll
-          for (int q = 0; q < 4; ++q)  // four K-steps of 16 inside the 128-byte rows
-            umma_bf16<PAIR>(tmem + b * kBN, smem_desc_k128(sA + 32 * q), smem_desc_k128(sA + Cfg::kBlkA + 32 * q),
-                            idesc, (first && q == 0) ? 0u : 1u);
-          // Probe (without blocking) the next stage's data while these MMAs
-          // are queued: when it has arrived, the next MMAs follow at once
-          // instead of after a blocking wait, which would let the tensor
-          // pipe run dry.
-          ready = it + 1 < total &&
-                  mbar_test_wait(&full[(it + 1) % Cfg::kStages], ((it + 1) / Cfg::kStages) & 1u);
-          // the stage is free (in both CTAs of a pair) once these MMAs finish
-          if (PAIR) {
-            umma_commit_pair(smem_u32(&empty[stage]));
-            umma_commit_pair(cluster_addr(smem_u32(&empty[stage]), peer));
-          } else {
-            umma_commit(&empty[stage]);
-          }
-          if ((ks + 1) % kSegStages == 0 || ks + 1 == kp.nst) {
-            if (PAIR) {
-              umma_commit_pair(smem_u32(&acc_full[b]));
-              umma_commit_pair(cluster_addr(smem_u32(&acc_full[b]), peer));
-            } else {
-              umma_commit(&acc_full[b]);
-            }
-            ++seg;
-          }
-        }
-    }
+  for (int k = 0; k < 4; ++k) {
+    // 1.5 2^23 + x has x in its low mantissa bits
+    const float xf = __uint_as_float(0x4B400000u + static_cast<uint32_t>(x[k])) - 12582912.0f;
+    const float q = __fadd_rn(__fadd_rn(__fmaf_rn(xf, inv, off), 12582912.0f), -12582912.0f);
+    r[k] = __float_as_uint(__fadd_rn(__fmaf_rn(q, negm, xf), 8388608.0f));
+  }
+  return __byte_perm(__byte_perm(r[0], r[1], 0x0040u), __byte_perm(r[2], r[3], 0x0040u), 0x5410u);
+}
+
+// Work item i: plane p = i / (tiles per plane), then the tile.
+template <bool PAIR>
+struct WorkII {
+  const KParamsIITC& kp;
+  __device__ __forceinline__ int nitems() const {
+    return kp.nplanes * (PAIR ? kp.tiles_m / 2 : kp.tiles_m) * kp.tiles_n;
+  }
+  __device__ __forceinline__ bf16g::Item item(int i) const {
+    const int tm_units = PAIR ? kp.tiles_m / 2 : kp.tiles_m, per_plane = tm_units * kp.tiles_n;
+    bf16g::Item t;
+    t.unit = i / per_plane;
+    tile_coords16(i - t.unit * per_plane, tm_units, kp.tiles_n, t.tm, t.tn);
+    if (PAIR) t.tm *= 2;
+    t.np = 1;
+    t.k0 = 0;
+    t.k1 = kp.nst;
+    t.seg = bf16g::Cfg<PAIR>::kSeg14;
+    t.aux = 0;
+    return t;
+  }
+  __device__ __forceinline__ int ya(const bf16g::Item& t, int) const { return t.unit * kp.rowsA_pad + t.tm * kBM; }
+  __device__ __forceinline__ int yb(const bf16g::Item& t, int) const { return t.unit * kp.rowsB_pad + t.tn * kBN; }
+  __device__ __forceinline__ int cols(const bf16g::Item& t) const {
+    const int n = kp.N - t.tn * kBN;
+    return n >= kBN ? kBN : (n + 31) & ~31;
+  }
+};
+
+template <bool PAIR>
+__global__ void __launch_bounds__(bf16g::kThreads, 1)
+    gemm_II_tc_kernel(const __grid_constant__ KParamsIITC kp, const __grid_constant__ ModTables mt) {
+  extern __shared__ uint8_t smem_raw[];
+  const bf16g::Ctx c = bf16g::setup<PAIR>(smem_raw);
+  const WorkII<PAIR> w{kp};
+  if (c.warp == bf16g::kProducerWarp) {
+    if (c.lane == 0) bf16g::produce<PAIR>(c, w, &kp.tA, &kp.tB, kp.status);
+    __syncwarp();
+  } else if (c.warp == bf16g::kMmaWarp) {
+    if (c.lane == 0 && c.crank == 0) bf16g::issue<PAIR>(c, w, kp.status);
     __syncwarp();
   } else {
-    // ---------------------------------------------------------------- drain (both CTAs)
-    const int hh = warp >> 2;
-    const int row_in_tile = (warp & 3) * 32 + lane;
-    const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + static_cast<uint32_t>(hh * 128);
-    // the accumulators are released to the even CTA's MMA thread
-    const uint32_t acc_empty0 = PAIR ? cluster_addr(smem_u32(&acc_empty[0]), 0u) : 0u;
-    const uint32_t acc_empty1 = PAIR ? cluster_addr(smem_u32(&acc_empty[1]), 0u) : 0u;
+    // drain: exact integer sums of this thread's columns over the segments;
+    // only the final sum is reduced mod m
+    constexpr int kC = bf16g::kDrainCols;
+    constexpr int kFold = 64;  // segments (|sum| < 2^24 each) per fold of the int32 sums
+    const int c0 = (c.warp >> 2) * kC, row = (c.warp & 3) * 32 + c.lane;
+    const uint32_t addr = bf16g::drain_addr(c);
+    const int nitems = w.nitems();
     uint32_t seg = 0;
     bool stop = false;
-    for (int t = 0; t < my_items && !stop; ++t) {
-      int p, tm, tn;
-      item_coords<PAIR>(kp, cid + t * ncl, static_cast<int>(crank), p, tm, tn);
-      const int l = p % kp.nm;
-      const int m = static_cast<int>(mt.mods[l]);
+    for (int rd = 0; rd * c.ncl < nitems && !stop; ++rd) {
+      const int i = bf16g::item_index(rd, c.cid, c.ncl);
+      if (i >= nitems) continue;
+      const bf16g::Item t = w.item(i);
+      const int nseg = (bf16g::stages_of<PAIR>(t) + t.seg - 1) / t.seg;
+      const int cols = w.cols(t) - c0;  // of this warp's kC columns
+      const int l = t.unit % kp.nm;
       const int p16 = mt.pow16[l][1];
-      const float inv = mt.inv[l];
-      // Exact integer sums of this thread's 128 columns over the segments so
-      // far: each segment adds one exact FP32 value per output, and only the
-      // final sum is reduced mod m -- two instructions per output and
-      // segment, because the drain competes for issue slots with the MMA
-      // thread, which must keep the tensor pipe fed.
-      int run[128];
+      int run[kC];
 #pragma unroll
-      for (int i = 0; i < 128; ++i) run[i] = 0;
+      for (int x = 0; x < kC; ++x) run[x] = 0;
       for (int s = 0; s < nseg; ++s, ++seg) {
-        const uint32_t b = seg & 1u;
-        // one lane per warp polls the barrier (256 polling threads slowed the
-        // other roles), the warp follows it
-        bool ok = true;
-        if (lane == 0) ok = wait_pair(&acc_full[b], (seg >> 1) & 1u, ab, kp.status);
-        ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-        __syncwarp();
-        if (!ok) {
+        if (!bf16g::wait_segment(c, seg, kp.status)) {
           stop = true;
           break;
         }
-        tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < kC / 16; ++q) {
           uint32_t v[16];
-          tmem_ld16(lane_addr + b * kBN + 16 * q, v);
-          tmem_wait_ld();
-          if (q == 7) {  // the MMAs may refill this accumulator now
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-              if (PAIR)
-                mbar_arrive_cluster(b ? acc_empty1 : acc_empty0);
-              else
-                mbar_arrive(&acc_empty[b]);
-            }
+          if (16 * q < cols) {
+            tmem_ld16(addr + (seg & 1u) * kBN + 16 * q, v);
+            tmem_wait_ld();
           }
+          if (q == kC / 16 - 1) bf16g::release_segment<PAIR>(c, seg);
+          if (16 * q < cols) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) run[16 * q + i] += __float2int_rn(__uint_as_float(v[i]));
+            for (int x = 0; x < 16; ++x) run[16 * q + x] += __float2int_rn(__uint_as_float(v[x]));
+          }
         }
-        // |segment sum| <= 960 * 2^14 < 2^24: fold every 64 segments so that
-        // the int32 sums never overflow, whatever K is
-        if ((s & 63) == 63) {
+        // fold every 64 segments, so that the int32 sums never overflow, whatever K is
+        if (s % kFold == kFold - 1) {
 #pragma unroll
-          for (int i = 0; i < 128; ++i) run[i] = fold16(run[i], p16);
+          for (int x = 0; x < kC; ++x) run[x] = fold16(run[x], p16);
         }
       }
       if (stop) break;
-      // Eq. (7): residues in [0, m), 128 bytes of this thread's row
+      // Eq. (7): residues in [0, m), kC bytes of this thread's row
+      const float m = mt.mf[l], inv = mt.inv[l];
+      const float off = __fadd_rn(__fmul_rn(0.5f, inv), -0.5f);
+      const int tm = t.tm + static_cast<int>(c.crank);
       uint4* dst = reinterpret_cast<uint4*>(
-          kp.R + (static_cast<int64_t>(p) * kp.tiles_m * kBM + tm * kBM + row_in_tile) * kp.ldr + tn * kBN + hh * 128);
+          kp.R + (static_cast<int64_t>(t.unit) * kp.tiles_m * kBM + tm * kBM + row) * kp.ldr + t.tn * kBN + c0);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int g = 0; g < kC / 16; ++g) {
         uint32_t wv[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          uint32_t o = 0;
+          int x[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            o |= static_cast<uint32_t>(mod_small(fold16(run[16 * i + 4 * e + k], p16), m, inv)) << (8 * k);
-          wv[e] = o;
+          for (int k = 0; k < 4; ++k) x[k] = fold16(run[16 * g + 4 * e + k], p16);
+          wv[e] = mod4(x, inv, off, -m);
         }
-        dst[i] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+        if (16 * g < cols) dst[g] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
       }
     }
   }
-  tc_fence_before();
-  // no CTA of a pair leaves while the other may still touch its shared or tensor memory
-  if (PAIR)
-    cluster_sync_all();
-  else
-    __syncthreads();
-  if (warp == kMmaWarp) {
-    tc_fence_after();
-    tmem_free_all<PAIR>(tmem);
-  }
+  bf16g::finish<PAIR>(c);
 }
 
 // ---------------------------------------------------------------- CRT
@@ -505,42 +325,16 @@ __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KPa
   }
 }
 
-// Largest number of co-resident CTA pairs of the GEMM kernel (0 if it cannot
-// run in clusters of two).
-int max_pairs() {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(2u * 64u);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = CfgII<true>::kSmem;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, gemm_II_tc_kernel<true>, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
-  return n;
-}
-
-template <bool PAIR>
-cudaError_t launch_residues_t(const GemmIIArgs& a, int nsets, const ModTables& mt, cudaStream_t st) {
-  using Cfg = CfgII<PAIR>;
-  cudaError_t e = cudaFuncSetAttribute(gemm_II_tc_kernel<PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg::kSmem);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_residues(const GemmIIArgs& a, int nsets, const ModTables& mt, cudaStream_t st) {
+  const bool pair = a.cluster == 2;
   KParamsIITC kp;
   kp.tA = *a.descA;
   kp.tB = *a.descB;
-  kp.nst = a.nk32 / 2;  // planes are padded to 128 K-elements
+  kp.nst = (a.K + 63) / 64;
   kp.tiles_m = (a.M + kBM - 1) / kBM;
-  if (PAIR) kp.tiles_m += kp.tiles_m & 1;  // whole pair tiles: the residue planes hold them
-  kp.tiles_mu = PAIR ? kp.tiles_m / 2 : kp.tiles_m;
+  if (pair) kp.tiles_m += kp.tiles_m & 1;  // whole pair tiles: the residue planes hold them
   kp.tiles_n = (a.N + kBN - 1) / kBN;
+  kp.N = a.N;
   kp.nplanes = nsets * a.nm;
   kp.nm = a.nm;
   kp.rowsA_pad = a.rowsA_pad;
@@ -548,36 +342,10 @@ cudaError_t launch_residues_t(const GemmIIArgs& a, int nsets, const ModTables& m
   kp.R = a.scratch;
   kp.ldr = static_cast<int64_t>(kp.tiles_n) * kBN;
   kp.status = a.status;
-  const int nitems = kp.nplanes * kp.tiles_mu * kp.tiles_n;
+  const int64_t nitems = static_cast<int64_t>(kp.nplanes) * (pair ? kp.tiles_m / 2 : kp.tiles_m) * kp.tiles_n;
   if (nitems == 0 || kp.nst == 0) return cudaSuccess;
-  if (!PAIR) {
-    const int grid = nitems < a.num_sms ? nitems : a.num_sms;
-    gemm_II_tc_kernel<false><<<grid, kThreads, Cfg::kSmem, st>>>(kp, mt);
-    return cudaGetLastError();
-  }
-  static int mc = -1;
-  if (mc < 0) mc = max_pairs();
-  if (mc <= 0) return cudaErrorInvalidConfiguration;
-  const int npairs = nitems < mc ? nitems : mc;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(static_cast<unsigned>(2 * npairs));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Cfg::kSmem;
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, gemm_II_tc_kernel<true>, kp, mt);
-}
-
-cudaError_t launch_residues(const GemmIIArgs& a, int nsets, const ModTables& mt, cudaStream_t st) {
-  if (a.cluster == 2) return launch_residues_t<true>(a, nsets, mt, st);
-  if (a.cluster == 1) return launch_residues_t<false>(a, nsets, mt, st);
-  return cudaErrorInvalidValue;
+  return pair ? bf16g::launch<true>(gemm_II_tc_kernel<true>, nitems, a.num_sms, st, kp, mt)
+              : bf16g::launch<false>(gemm_II_tc_kernel<false>, nitems, a.num_sms, st, kp, mt);
 }
 
 template <int MODE>
@@ -637,17 +405,24 @@ size_t gemm_II_tc_residue_bytes(int64_t M, int64_t N, int nm, bool is_complex, i
          static_cast<size_t>(tiles_n * kBN);
 }
 
-// CTAs per GEMM tile of the Scheme II tcgen05 kernel: 1 (one CTA on a
-// 128 x 256 tile; the default) or 2 (a CTA pair on one 256 x 256 tile,
-// tcgen05.mma.cta_group::2) with EMU_II_CLUSTER=2.  The B tensor map's box
-// is 256 / cluster rows.
-int gemm_II_tc_cluster() {
-  static int v = 0;
-  if (v == 0) {
+// Pairs need full 256-row tiles (an odd number of 128-row tiles leaves half a
+// pair idle, which costs more than pairs gain below 5) and long segments.
+static bool use_pairs(int64_t M, int64_t K) {
+  const int64_t t = (M + kBM - 1) / kBM;
+  return (t % 2 == 0 || t >= 5) && K >= kPairMinK;
+}
+
+// CTAs per GEMM tile of a product of M rows: 2 (a CTA pair on a 256 x 256
+// tile) or 1 (128 x 256), or always the one that EMU_II_CLUSTER names.  The B
+// tensor map's box is 256 / cluster rows.
+int gemm_II_tc_cluster(int64_t M, int64_t K) {
+  static int v = -1;
+  if (v < 0) {
     const char* e = std::getenv("EMU_II_CLUSTER");
-    v = (e && std::atoi(e) == 2) ? 2 : 1;
+    const int x = e ? std::atoi(e) : 0;
+    v = x == 1 || x == 2 ? x : 0;
   }
-  return v;
+  return v ? v : use_pairs(M, K) ? 2 : 1;
 }
 
 cudaError_t launch_gemm_II_tc(int out_mode, const GemmIIArgs& a, const ModTables& mt, const CrtTables& ct,

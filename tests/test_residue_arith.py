@@ -45,3 +45,19 @@ def test_quotient_exact_over_whole_range(orc, nd):
 def test_offset_half_is_needed(orc):
     # with c = RN(off/m) the exact multiples of m (j = 0) can come out one low
     assert sum(_mismatches(m, 4, half=False) for m in orc.moduli(20)) > 0
+
+
+def test_output_residue_rounding_exact_over_whole_range(orc):
+    # the residue GEMM's reduction: x mod m = x - m RN(RN(x inv + off)), off =
+    # RN(inv / 2 - 1/2), for every sum that its fold by 2^16 mod m can leave:
+    # |x| <= 128 (2^30 + 2^21.1) / 2^16 + 65535.  The FMA is exact in binary64
+    # before its one rounding (x and inv have at most 22 and 24 bits, off's
+    # last bit is above 2^-34).
+    bound = 128 * ((2 ** 30 + 2 ** 22) >> 16) + 65535
+    x = np.arange(-bound, bound + 1, dtype=np.int64)
+    for m in orc.moduli(20):
+        inv = np.float32(1) / np.float32(m)
+        off = np.float32(np.float32(0.5) * inv - np.float32(0.5))
+        y = np.float32(x * float(inv) + float(off))
+        n = np.float32(y.astype(np.float64) + 12582912.0).astype(np.float64) - 12582912.0
+        assert np.array_equal(x - n.astype(np.int64) * m, x % m), m
