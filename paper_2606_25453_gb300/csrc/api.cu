@@ -528,12 +528,16 @@ constexpr int64_t kTriMaxK = int64_t{1} << 20;
 constexpr int kTriSmallP = 8;
 constexpr int64_t kTriLargeWork = int64_t{1} << 33;
 
-int64_t tri_rows(int64_t m, int64_t n, int64_t k, int p) {
-  if (!i_engine_tc() || k < 1 || k > kTriMaxK) return 0;
+bool tri_takes(int64_t m, int64_t n, int64_t k, int p) {
+  if (!i_engine_tc() || k < 1 || k > kTriMaxK) return false;
   if (p > kTriSmallP && static_cast<double>(m) * static_cast<double>(n) * static_cast<double>(k) < kTriLargeWork)
-    return 0;
+    return false;
   // plane rows are TMA coordinates (int32)
-  if ((m > n ? m : n) > INT32_MAX / tri_num_planes(p) / 2) return 0;
+  return (m > n ? m : n) <= INT32_MAX / tri_num_planes(p) / 2;
+}
+
+int64_t tri_rows(int64_t m, int64_t n, int64_t k, int p) {
+  if (!tri_takes(m, n, k, p)) return 0;
   auto pass = [&](int64_t rows) {
     const TriLayout L = tri_layout(rows, n, k, p);
     return static_cast<int64_t>(L.Cs_bytes) + 2 * static_cast<int64_t>(tri_num_planes(p)) * rows * L.kpad;

@@ -34,12 +34,13 @@
 // pair for the other roles, and the TMEM is still released.
 //
 // Work: a policy W with
-//   int nitems();  int tiles_m() (row units), tiles_n();
-//   Item item(i): plane-pair count `np`, K stage range [k0, k1) in 64-deep
-//     chunks, row unit tm, column tile tn, and segment length `seg` in stages
-//   int ya(item, q), yb(item, q): first row of A's tile (PAIR: of this CTA's
-//     half) and of B's tile in the stacked planes, for plane pair q
-//   int cols(item): columns of the tile that the MMAs compute
+//   bool at(r, cid, ncl, item): the r-th item of CTA (pair) cid of ncl; false
+//     after the last one.  An item: plane-pair count `np`, K range [k0, k1) in
+//     64-deep chunks, first 128-row tile tm (of the even CTA), column tile tn,
+//     segment length `seg` in stages, columns `cols` that the MMAs compute
+//   int ya(item, q), yb(item, q): first row of A's tile (the even CTA's) and
+//     of B's tile in the stacked planes, for plane pair q
+//   const CUtensorMap* tA(item), tB(item); int bytes(item): of one chunk's boxes
 #pragma once
 #include "emu_internal.h"
 #include "tc_core.cuh"
@@ -73,7 +74,7 @@ struct Cfg {
 };
 
 struct Item {
-  int unit, np, k0, k1, seg, tm, tn, aux;
+  int unit, np, k0, k1, seg, tm, tn, cols, aux, prob;
 };
 
 // Stages of one item: every plane pair has its own, the last of each may
@@ -83,8 +84,8 @@ __device__ __forceinline__ int stages_of(const Item& t) {
   return t.np * ((t.k1 - t.k0 + Cfg<PAIR>::kKS - 1) / Cfg<PAIR>::kKS);
 }
 
-// Item of this CTA (pair) in round r: odd rounds run backwards, which evens
-// out the sums when the items are sorted by length.
+// Index of CTA (pair) cid's item in round r: odd rounds run backwards, which
+// evens out the sums when the items are sorted by length.
 __device__ __forceinline__ int item_index(int r, int cid, int ncl) {
   return r * ncl + ((r & 1) ? ncl - 1 - cid : cid);
 }
@@ -160,20 +161,18 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
 
 // The producer thread (one of each CTA).
 template <bool PAIR, class W>
-__device__ __forceinline__ void produce(const Ctx& c, const W& w, const CUtensorMap* tA, const CUtensorMap* tB,
-                                        int* status) {
+__device__ __forceinline__ void produce(const Ctx& c, const W& w, int* status) {
   using C = Cfg<PAIR>;
-  tma_prefetch_desc(tA);
-  tma_prefetch_desc(tB);
-  const int nitems = w.nitems();
   uint32_t j = 0;
   bool stop = false;
-  for (int r = 0; r * c.ncl < nitems && !stop; ++r) {
-    const int i = item_index(r, c.cid, c.ncl);
-    if (i >= nitems) continue;
-    const Item t = w.item(i);
+  Item t;
+  for (int r = 0; !stop && w.at(r, c.cid, c.ncl, t); ++r) {
+    const CUtensorMap *const tA = w.tA(t), *const tB = w.tB(t);
+    tma_prefetch_desc(tA);
+    tma_prefetch_desc(tB);
+    const int bytes = (PAIR ? 2 : 1) * w.bytes(t);
     // each CTA of a pair holds half of the columns the MMAs read
-    const int half = PAIR ? static_cast<int>(c.crank) * (w.cols(t) / 2) : 0;
+    const int half = PAIR ? static_cast<int>(c.crank) * (t.cols / 2) : 0;
     for (int q = 0; q < t.np && !stop; ++q) {
       const int ya = w.ya(t, q) + static_cast<int>(c.crank) * kBM, yb = w.yb(t, q) + half;
       for (int ks = t.k0; ks < t.k1; ks += C::kKS, ++j) {
@@ -185,7 +184,7 @@ __device__ __forceinline__ void produce(const Ctx& c, const W& w, const CUtensor
         }
         uint8_t* s = c.smem + stage * C::kStageBytes;
         const int parts = t.k1 - ks < C::kKS ? t.k1 - ks : C::kKS;
-        if (c.crank == 0) mbar_arrive_expect_tx(&c.full[stage], (PAIR ? 2 : 1) * parts * C::kChunkBytes);
+        if (c.crank == 0) mbar_arrive_expect_tx(&c.full[stage], parts * bytes);
         // both CTAs' bytes are counted on the even CTA's barrier
         const uint32_t bar = PAIR ? cluster_addr(smem_u32(&c.full[stage]), 0u) : 0u;
 #pragma unroll
@@ -220,15 +219,12 @@ __device__ __forceinline__ void produce(const Ctx& c, const W& w, const CUtensor
 template <bool PAIR, class W>
 __device__ __forceinline__ void issue(const Ctx& c, const W& w, int* status) {
   using C = Cfg<PAIR>;
-  const int nitems = w.nitems();
   uint32_t it = 0, seg = 0;
   bool stop = false;
   bool ready = false;  // the probe after the previous stage's MMAs already saw this stage's data
-  for (int r = 0; r * c.ncl < nitems && !stop; ++r) {
-    const int i = item_index(r, c.cid, c.ncl);
-    if (i >= nitems) continue;
-    const Item t = w.item(i);
-    const uint32_t idesc = idesc_bf16(PAIR ? 2 * kBM : kBM, w.cols(t));
+  Item t;
+  for (int r = 0; !stop && w.at(r, c.cid, c.ncl, t); ++r) {
+    const uint32_t idesc = idesc_bf16(PAIR ? 2 * kBM : kBM, t.cols);
     const int per = (t.k1 - t.k0 + C::kKS - 1) / C::kKS, n = t.np * per;
     const int last_parts = t.k1 - t.k0 - (per - 1) * C::kKS;  // chunks of a plane pair's last stage
     int left = 0, ks = 0;  // stages left in this segment; stage within the plane pair
@@ -317,6 +313,13 @@ __device__ __forceinline__ void finish(const Ctx& c) {
     tc_fence_after();
     tmem_free_all<PAIR>(c.tmem);
   }
+}
+
+// Columns of column tile tn that the MMAs compute: of the last tile only as
+// many as n needs, in steps of 32.
+__device__ __forceinline__ int tile_cols(int n, int tn) {
+  const int left = n - tn * kBN;
+  return left >= kBN ? kBN : (left + 31) & ~31;
 }
 
 // Launch `kernel` on nitems items: one CTA (pair) per SM (two SMs).

@@ -118,7 +118,10 @@ struct TriLayout {
   bool one;           // one plane pair per output plane, else one group of them
   size_t Cs_bytes;
 };
-TriLayout tri_layout(int64_t M, int64_t N, int64_t k, int p);
+// one: 1 or 0 fixes `one`, -1 leaves it to the product's size.
+TriLayout tri_layout(int64_t M, int64_t N, int64_t k, int p, int one = -1);
+// The products of the recentring constants alone (part of every S), 128 bits.
+void tri_const(int p, int64_t K, uint64_t* lo, uint64_t* hi);
 int tri_tile_m();
 int tri_tile_n();
 int tri_num_planes(int p);

@@ -81,12 +81,10 @@ __device__ __forceinline__ uint32_t mod4(const int* x, float inv, float off, flo
 template <bool PAIR>
 struct WorkII {
   const KParamsIITC& kp;
-  __device__ __forceinline__ int nitems() const {
-    return kp.nplanes * (PAIR ? kp.tiles_m / 2 : kp.tiles_m) * kp.tiles_n;
-  }
-  __device__ __forceinline__ bf16g::Item item(int i) const {
+  __device__ __forceinline__ bool at(int r, int cid, int ncl, bf16g::Item& t) const {
     const int tm_units = PAIR ? kp.tiles_m / 2 : kp.tiles_m, per_plane = tm_units * kp.tiles_n;
-    bf16g::Item t;
+    const int i = bf16g::item_index(r, cid, ncl);
+    if (i >= kp.nplanes * per_plane) return false;
     t.unit = i / per_plane;
     tile_coords16(i - t.unit * per_plane, tm_units, kp.tiles_n, t.tm, t.tn);
     if (PAIR) t.tm *= 2;
@@ -94,15 +92,14 @@ struct WorkII {
     t.k0 = 0;
     t.k1 = kp.nst;
     t.seg = bf16g::Cfg<PAIR>::kSeg14;
-    t.aux = 0;
-    return t;
+    t.cols = bf16g::tile_cols(kp.N, t.tn);
+    return true;
   }
   __device__ __forceinline__ int ya(const bf16g::Item& t, int) const { return t.unit * kp.rowsA_pad + t.tm * kBM; }
   __device__ __forceinline__ int yb(const bf16g::Item& t, int) const { return t.unit * kp.rowsB_pad + t.tn * kBN; }
-  __device__ __forceinline__ int cols(const bf16g::Item& t) const {
-    const int n = kp.N - t.tn * kBN;
-    return n >= kBN ? kBN : (n + 31) & ~31;
-  }
+  __device__ __forceinline__ const CUtensorMap* tA(const bf16g::Item&) const { return &kp.tA; }
+  __device__ __forceinline__ const CUtensorMap* tB(const bf16g::Item&) const { return &kp.tB; }
+  __device__ __forceinline__ int bytes(const bf16g::Item&) const { return bf16g::Cfg<PAIR>::kChunkBytes; }
 };
 
 template <bool PAIR>
@@ -112,7 +109,7 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1)
   const bf16g::Ctx c = bf16g::setup<PAIR>(smem_raw);
   const WorkII<PAIR> w{kp};
   if (c.warp == bf16g::kProducerWarp) {
-    if (c.lane == 0) bf16g::produce<PAIR>(c, w, &kp.tA, &kp.tB, kp.status);
+    if (c.lane == 0) bf16g::produce<PAIR>(c, w, kp.status);
     __syncwarp();
   } else if (c.warp == bf16g::kMmaWarp) {
     if (c.lane == 0 && c.crank == 0) bf16g::issue<PAIR>(c, w, kp.status);
@@ -124,15 +121,12 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1)
     constexpr int kFold = 64;  // segments (|sum| < 2^24 each) per fold of the int32 sums
     const int c0 = (c.warp >> 2) * kC, row = (c.warp & 3) * 32 + c.lane;
     const uint32_t addr = bf16g::drain_addr(c);
-    const int nitems = w.nitems();
     uint32_t seg = 0;
     bool stop = false;
-    for (int rd = 0; rd * c.ncl < nitems && !stop; ++rd) {
-      const int i = bf16g::item_index(rd, c.cid, c.ncl);
-      if (i >= nitems) continue;
-      const bf16g::Item t = w.item(i);
+    bf16g::Item t;
+    for (int rd = 0; !stop && w.at(rd, c.cid, c.ncl, t); ++rd) {
       const int nseg = (bf16g::stages_of<PAIR>(t) + t.seg - 1) / t.seg;
-      const int cols = w.cols(t) - c0;  // of this warp's kC columns
+      const int cols = t.cols - c0;  // of this warp's kC columns
       const int l = t.unit % kp.nm;
       const int p16 = mt.pow16[l][1];
       int run[kC];

@@ -28,6 +28,7 @@
 #include "emu_handle.h"
 #include "emu_internal.h"
 #include "gemm_I_core.cuh"
+#include "grouped_tri.h"
 #include "split_core.cuh"
 
 namespace emu {
@@ -385,6 +386,7 @@ struct GroupPlan {
   std::vector<int> pcfg;  // configuration of each product (caller's order)
   int p = 0, count = 0;
   int max_stages = kMaxStages;  // the setting the plan was built for
+  bool want_tri = false;        // built with the bf16 path allowed
   int nstages = 1;
   StagePlan stages[kMaxStages];
   std::vector<SubPlan> subs;
@@ -396,6 +398,7 @@ struct GroupPlan {
   size_t max_bytes = 0;
   cudaGraphExec_t exec = nullptr;
   cudaGraph_t graph = nullptr;
+  GroupTri* tri = nullptr;  // the whole batch on the bf16 tensor cores (then no subs and one stage)
 };
 
 constexpr int kMaxSubs = kMaxStages * kNumCfg;
@@ -413,6 +416,7 @@ void free_plan(GroupPlan* pl) {
   if (pl->exec) cudaGraphExecDestroy(pl->exec);
   if (pl->graph) cudaGraphDestroy(pl->graph);
   if (pl->dev) cudaFree(pl->dev);
+  group_tri_free(pl->tri);
   delete pl;
 }
 
@@ -422,8 +426,8 @@ GroupState* state_of(emu_handle_s* h) {
 }
 
 bool same_plan(const GroupPlan* pl, const emu_gemm_desc_t* b, int count, int p, const std::vector<int>& pcfg,
-               int stages) {
-  if (!pl || pl->p != p || pl->max_stages != stages || static_cast<int>(pl->descs.size()) != count ||
+               int stages, bool tri) {
+  if (!pl || pl->p != p || (pl->want_tri != tri) || pl->max_stages != stages || static_cast<int>(pl->descs.size()) != count ||
       pl->pcfg != pcfg)
     return false;
   return std::memcmp(pl->descs.data(), b, sizeof(emu_gemm_desc_t) * count) == 0;
@@ -517,6 +521,13 @@ int occupancy_of(int cfg) { return (kCfgBM[cfg] / 16) * (kCfgBN[cfg] / 16) >= 8 
 // split, so that stage 0's GEMMs overlap stage 1's scan and split; every
 // branch joins `st` before the end.
 cudaError_t launch_group(const GroupPlan& pl, GroupState* gs, int* status, cudaStream_t st) {
+  if (pl.tri) {
+    cudaMemsetAsync(pl.tri->zero, 0, pl.tri->zero_bytes, st);
+    const StagePlan& sg = pl.stages[0];
+    grouped_scan_kernel<<<sg.scan_blocks, 256, 0, st>>>(pl.d_probs, sg.count, sg.d_startA_scan, sg.d_startB_scan,
+                                                         status);
+    return group_tri_launch(*pl.tri, status, st);
+  }
   cudaMemsetAsync(pl.d_max, 0, pl.max_bytes, st);
   for (int s = 0; s < pl.nstages; ++s) {
     const StagePlan& sg = pl.stages[s];
@@ -784,6 +795,63 @@ emu_status_t build_plan(emu_handle_s* h, int count, const emu_gemm_desc_t* d_in,
   return EMU_OK;
 }
 
+// A plan of the bf16 path: its tables and workspace (grouped_tri.cu) and the
+// scan's product table.
+emu_status_t build_tri_plan(emu_handle_s* h, int count, const emu_gemm_desc_t* d, int p, const std::vector<int>& pcfg,
+                            int stages, GroupPlan** out) {
+  auto* pl = new GroupPlan();
+  pl->descs.assign(d, d + count);
+  pl->pcfg = pcfg;
+  pl->p = p;
+  pl->count = count;
+  pl->max_stages = stages;
+  pl->stages[0].count = count;
+  pl->tri = new GroupTri();
+  emu_status_t s = group_tri_build(h, count, d, p, pl->tri);
+  if (s != EMU_OK) {
+    free_plan(pl);
+    return s;
+  }
+  std::vector<GProb> probs(count);
+  std::vector<int> st(2 * (count + 1), 0);
+  int *sA = st.data(), *sB = sA + count + 1;
+  for (int i = 0; i < count; ++i) {
+    GProb& g = probs[i];
+    std::memset(&g, 0, sizeof(g));
+    g.A = d[i].A;
+    g.B = d[i].B;
+    g.lda = d[i].lda;
+    g.ldb = d[i].ldb;
+    g.M = static_cast<int>(d[i].m);
+    g.N = static_cast<int>(d[i].n);
+    g.K = static_cast<int>(d[i].k);
+    g.maxA = pl->tri->maxA[i];
+    g.maxB = pl->tri->maxB[i];
+    sA[i + 1] = sA[i] + static_cast<int>(((d[i].m + 7) / 8) * ((d[i].k + 2047) / 2048));
+    sB[i + 1] = sB[i] + static_cast<int>(((d[i].n + 31) / 32) * ((d[i].k + 255) / 256));
+  }
+  pl->stages[0].scan_blocks = sA[count] + sB[count];
+  const size_t o_st = al256(sizeof(GProb) * count);
+  pl->dev_bytes = o_st + al256(sizeof(int) * st.size());
+  if (cudaMalloc(&pl->dev, pl->dev_bytes) != cudaSuccess) {
+    pl->dev = nullptr;
+    cudaGetLastError();
+    free_plan(pl);
+    return EMU_ERR_ALLOC;
+  }
+  uint8_t* base = static_cast<uint8_t*>(pl->dev);
+  pl->d_probs = reinterpret_cast<GProb*>(base);
+  pl->stages[0].d_startA_scan = reinterpret_cast<int*>(base + o_st);
+  pl->stages[0].d_startB_scan = pl->stages[0].d_startA_scan + count + 1;
+  if (cudaMemcpy(base, probs.data(), sizeof(GProb) * count, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(base + o_st, st.data(), sizeof(int) * st.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+    free_plan(pl);
+    return EMU_ERR_CUDA;
+  }
+  *out = pl;
+  return EMU_OK;
+}
+
 // Capture the plan's launch sequence into a graph (on a private stream, with
 // private side streams for the parallel GEMM branches).
 emu_status_t capture_plan(emu_handle_s* h, GroupState* gs, GroupPlan* pl) {
@@ -797,7 +865,7 @@ emu_status_t capture_plan(emu_handle_s* h, GroupState* gs, GroupPlan* pl) {
           cudaEventCreateWithFlags(&gs->join[i], cudaEventDisableTiming) != cudaSuccess)
         return EMU_ERR_CUDA;
   }
-  if (prepare_attrs(*pl) != cudaSuccess) return EMU_ERR_CUDA;
+  if ((pl->tri ? group_tri_prepare() : prepare_attrs(*pl)) != cudaSuccess) return EMU_ERR_CUDA;
   if (cudaStreamBeginCapture(gs->capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return EMU_ERR_CUDA;
   cudaError_t le = launch_group(*pl, gs, h->status, gs->capture);
   cudaError_t ce = cudaStreamEndCapture(gs->capture, &pl->graph);
@@ -823,18 +891,22 @@ emu_status_t validate(emu_handle_s* h, int count, const emu_gemm_desc_t* d, int 
 
 // Run (building and capturing if the product list or the configurations
 // changed) with a tile configuration per product.
+// tri: the bf16 path may take the batch.
 emu_status_t run_group(emu_handle_s* h, int count, const emu_gemm_desc_t* d, int p, const std::vector<int>& pcfg,
-                       int stages, cudaStream_t st) {
+                       int stages, cudaStream_t st, bool tri = false) {
   GroupState* gs = state_of(h);
   GroupPlan* pl = gs->plan;
-  if (!same_plan(pl, d, count, p, pcfg, stages)) {
+  if (!same_plan(pl, d, count, p, pcfg, stages, tri)) {
     if (pl) {
       cudaDeviceSynchronize();
       free_plan(pl);
       gs->plan = nullptr;
     }
-    emu_status_t s = build_plan(h, count, d, p, pcfg, stages, &pl);
+    // memory too full for the planes: the mma.sync kernels (the same bits)
+    emu_status_t s = tri ? build_tri_plan(h, count, d, p, pcfg, stages, &pl) : EMU_ERR_ALLOC;
+    if (s == EMU_ERR_ALLOC) s = build_plan(h, count, d, p, pcfg, stages, &pl);
     if (s != EMU_OK) return s;
+    pl->want_tri = tri;
     s = capture_plan(h, gs, pl);
     if (s != EMU_OK) {
       free_plan(pl);
@@ -844,7 +916,8 @@ emu_status_t run_group(emu_handle_s* h, int count, const emu_gemm_desc_t* d, int
   }
   trace_begin(h, PH_GEMM, st);
   cudaError_t e = cudaGraphLaunch(pl->exec, st);
-  trace_end(h, PH_GEMM, st, 1 + 2 * pl->nstages + static_cast<int>(pl->subs.size()));
+  trace_end(h, PH_GEMM, st,
+            pl->tri ? 1 + kGroupTriKernels : 1 + 2 * pl->nstages + static_cast<int>(pl->subs.size()));
   return e == cudaSuccess ? EMU_OK : EMU_ERR_CUDA;
 }
 
@@ -975,8 +1048,10 @@ emu_status_t emu_dgemm_grouped(emu_handle_t h, int count, const emu_gemm_desc_t*
   if (s != EMU_OK || count == 0) return s;
   cudaSetDevice(h->device);
   GroupState* gs = state_of(h);
+  // up to eight slices the whole batch runs on the bf16 tensor cores; tile
+  // configurations (tuned or loaded) are those of the mma.sync kernels
   return run_group(h, count, descs, p, configs_of(gs, count, descs, p), stages_of(gs, p),
-                   static_cast<cudaStream_t>(stream));
+                   static_cast<cudaStream_t>(stream), p <= kGroupTriMaxP && group_tri_takes(count, descs, p));
 }
 
 emu_status_t emu_dgemm_grouped_loop(emu_handle_t h, int count, const emu_gemm_desc_t* d, int p, emu_stream_t stream) {

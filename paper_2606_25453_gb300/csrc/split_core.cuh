@@ -106,7 +106,7 @@ __device__ __forceinline__ void fill_tile_strided(uint64_t (*tile)[133], const T
 // True when 16-byte loads of the vectors of X (leading dimension ld) are
 // aligned: X on a 16-byte boundary and ld a multiple of 16 bytes.
 template <typename T>
-inline bool vec16_ok(const T* X, int64_t ld) {
+__host__ __device__ inline bool vec16_ok(const T* X, int64_t ld) {
   return (reinterpret_cast<uintptr_t>(X) & 15u) == 0 && (static_cast<uint64_t>(ld) * sizeof(T)) % 16 == 0;
 }
 
