@@ -188,10 +188,76 @@ void host_crt_tables(int nm, CrtTables* t) {
     int64_t q = inv_mod(pm, mods[l]);
     limbs_mul_small(Pl, static_cast<uint32_t>(q));
     for (int i = 0; i < kCrtLimbs && i < static_cast<int>(Pl.size()); ++i) t->w[l][i] = Pl[i];
-    double wd = 0.0;
-    for (int i = kCrtLimbs - 1; i >= 0; --i) wd = wd * 4294967296.0 + t->w[l][i];
-    t->wP[l] = static_cast<float>(wd / pd);
   }
+}
+
+void host_crt_pair_tables(int nm, CrtPairTables* t) {
+  std::memset(t, 0, sizeof(*t));
+  int32_t mods[kMaxModuli];
+  host_moduli(nm, mods);
+  t->nm = nm;
+  const Limbs P = limbs_P(nm);
+  const int bl = limbs_bitlen(P);
+  for (size_t i = 0; i < P.size() && i < kCrtLimbs; ++i) t->P[i] = P[i];
+  for (int i = 0; i < kCrtLimbs; ++i) t->Phalf[i] = (t->P[i] >> 1) | (i + 1 < kCrtLimbs ? (t->P[i + 1] << 31) : 0u);
+  t->limbs = std::max(2, (bl + 31) / 32);
+  const int e = std::max(0, bl - 32);
+  t->sh = e - 32 * (t->limbs - 2);
+  if (e == 0) t->sh = 0;
+  t->frac = bl - 1 - e;
+  {  // floor(2^(63 + bl) / P) by binary long division (64 quotient bits; P a power of two: all ones)
+    Limbs rem(P.size() + 1, 0u);
+    auto ge = [&] {
+      if (rem[P.size()]) return true;
+      for (size_t i = P.size(); i-- > 0;)
+        if (rem[i] != P[i]) return rem[i] > P[i];
+      return true;
+    };
+    uint64_t q = 0;
+    bool over = false;
+    for (int b = 63 + bl; b >= 0; --b) {
+      uint32_t carry = b == 63 + bl ? 1u : 0u;
+      for (auto& w : rem) {
+        const uint32_t top = w >> 31;
+        w = (w << 1) | carry;
+        carry = top;
+      }
+      over = over || (q >> 63) != 0;
+      q <<= 1;
+      if (ge()) {
+        uint64_t br = 0;
+        for (size_t i = 0; i < rem.size(); ++i) {
+          const uint64_t d = static_cast<uint64_t>(rem[i]) - (i < P.size() ? P[i] : 0u) - br;
+          rem[i] = static_cast<uint32_t>(d);
+          br = d >> 63;
+        }
+        q |= 1u;
+      }
+    }
+    t->recip = over ? ~uint64_t{0} : q;
+  }
+  for (int i = 0; 2 * i < nm; ++i) {
+    const int64_t m = mods[2 * i], m2 = 2 * i + 1 < nm ? mods[2 * i + 1] : 1, mm = m * m2;
+    const int64_t lo = m2 * inv_mod(m2 % m, m) % mm, hi = m2 > 1 ? m * inv_mod(m % m2, m2) % mm : 0;
+    t->c[i] = static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
+    t->off[i] = static_cast<uint32_t>(((int64_t{1} << 25) / mm + 1) * mm);
+    Limbs W{1u};
+    for (int j = 0; j < nm; ++j)
+      if (j / 2 != i) limbs_mul_small(W, static_cast<uint32_t>(mods[j]));
+    limbs_mul_small(W, static_cast<uint32_t>(inv_mod(limbs_mod_small(W, static_cast<uint32_t>(mm)), mm)));
+    for (size_t j = 0; j < W.size() && j < kCrtLimbs; ++j) t->w[i][j] = W[j];
+  }
+}
+
+const MethodTables& method_tables(int nm) {
+  static MethodTables tabs[kMaxModuli + 1];
+  static std::once_flag once[kMaxModuli + 1];
+  std::call_once(once[nm], [nm] {
+    host_mod_tables(nm, &tabs[nm].mod);
+    host_crt_tables(nm, &tabs[nm].crt);
+    host_crt_pair_tables(nm, &tabs[nm].pair);
+  });
+  return tabs[nm];
 }
 
 // ================================================================ tensor maps
@@ -831,10 +897,8 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   if (norm) host_norm_halves_II(nm, &bA, &bB);
   auto* nEA = reinterpret_cast<int32_t*>(ws + pl.off_nEA);
   auto* nEB = reinterpret_cast<int32_t*>(ws + pl.off_nEB);
-  ModTables mt;
-  host_mod_tables(nm, &mt);
-  CrtTables ct;
-  host_crt_tables(nm, &ct);
+  const MethodTables& tabs = method_tables(nm);
+  const ModTables& mt = tabs.mod;
   const bool do_a = phase != 1, do_b = phase != 2;
   trace_begin(h, PH_SCAN, st);
   const unsigned long long* mA = v.maxA ? v.maxA : maxA;
@@ -897,18 +961,18 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   if (!tc) {
     trace_begin(h, PH_GEMM, st);
     cudaError_t e = fault_launch();
-    if (e == cudaSuccess) e = launch_gemm_II(out_mode, a, mt, ct, st);
+    if (e == cudaSuccess) e = launch_gemm_II(out_mode, a, mt, tabs.crt, st);
     trace_end(h, PH_GEMM, st, 1);
     return cuda_err(e);
   }
   // the residue GEMM is the traced GEMM phase, the CRT kernel "other"
   trace_begin(h, PH_GEMM, st);
   cudaError_t e = fault_launch();
-  if (e == cudaSuccess) e = launch_gemm_II_tc(out_mode, a, mt, ct, st, 1);
+  if (e == cudaSuccess) e = launch_gemm_II_tc(out_mode, a, mt, tabs.pair, st, 1);
   trace_end(h, PH_GEMM, st, 1);
   if (e != cudaSuccess) return cuda_err(e);
   trace_begin(h, PH_OTHER, st);
-  e = launch_gemm_II_tc(out_mode, a, mt, ct, st, 2);
+  e = launch_gemm_II_tc(out_mode, a, mt, tabs.pair, st, 2);
   trace_end(h, PH_OTHER, st, 1);
   return cuda_err(e);
 }
@@ -1124,8 +1188,7 @@ emu_status_t emu_split_II(emu_handle_t h, emu_layout_t layout, int operand, int6
   emu_status_t s = handle_workspace(h, 8 * static_cast<size_t>(rows > 0 ? rows : 1), st, &ws);
   if (s != EMU_OK) return s;
   auto* mx = reinterpret_cast<unsigned long long*>(ws);
-  ModTables mt;
-  host_mod_tables(nm, &mt);
+  const ModTables& mt = method_tables(nm).mod;
   int b = host_scale_bits_II(nm, k_total, 0);
   launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
   launch_split_II<double>(X, ldx, kcontig, rows, k, nm, b, 1, mt, mx, res, E, st);

@@ -114,124 +114,109 @@ __device__ __forceinline__ double crt_finish(const uint32_t* S, const CrtTables&
   return limbs_to_double_rn(R);
 }
 
-// ---------------------------------------------------------------- lazy form
-// S = sum_l w_l r_l kept as one 64-bit sum per 32-bit limb of w (each below
-// nm * 3 * 256 * 2^32 < 2^46 for residues r_l < 3 m_l, so no carries until
-// the end), next to the binary32 estimate t = sum_l r_l (w_l / P) of S / P.
-// Residues may exceed m_l (the complex modes add m_l or 2 m_l instead of
-// reducing): w_l m_l is a multiple of P, so S mod P is unchanged.
-struct CrtLazy {
-  uint64_t s[kCrtLimbs];
-  float t;
+// ---------------------------------------------------------------- pair form
+// S = sum over pairs of moduli of W x, with x the residue modulo m m' of one
+// pair (not reduced) and W < P its CRT weight, kept as one 64-bit sum per
+// 32-bit limb of W: at most ten x < 2^27, so no carries until the end.  Half
+// the multi-word products of a sum over single moduli.
+template <int L>
+struct CrtPair {
+  uint64_t s[L];
 };
 
-__device__ __forceinline__ void crt_lazy_init(CrtLazy& a) {
+// Finish: x = S - k P with k = round(S / P) from the top 64 bits of S and a
+// 64-bit reciprocal of P (k is exact unless S / P lies within 8 units of its
+// fixed-point form from a half, which the exact comparison below settles),
+// |x| <= P / 2, rounded once to binary64.  L 32-bit limbs of P.
+template <int L>
+__device__ __forceinline__ double crt_finish_pair(const CrtPair<L>& a, const CrtPairTables& ct) {
+  static_assert(L >= 2 && L <= kCrtLimbs, "limb count");
+  uint32_t S[L + 1];
+  uint64_t c = 0;
 #pragma unroll
-  for (int i = 0; i < kCrtLimbs; ++i) a.s[i] = 0;
-  a.t = 0.0f;
-}
-
-// a += w_l r_l, r in [0, 3 m_l).  L: the number of 32-bit limbs of P (and so
-// of every w_l < P); the limbs above stay zero, their products are skipped.
-template <int L = kCrtLimbs>
-__device__ __forceinline__ void crt_lazy_acc(CrtLazy& a, const CrtTables& ct, int l, uint32_t r) {
-  static_assert(L >= 1 && L <= kCrtLimbs, "limb count");
-#pragma unroll
-  for (int i = 0; i < L; ++i) a.s[i] += static_cast<uint64_t>(ct.w[l][i]) * r;
-  // r as binary32 without a conversion instruction: 2^23 + r has r in its low mantissa bits
-  a.t = __fmaf_rn(__uint_as_float(0x4B000000u | r) - 8388608.0f, ct.wP[l], a.t);
-}
-
-// Six-limb (192-bit) helpers on 32-bit carry chains (PTX add/sub/mad with
-// carry; one instruction per limb).  Outputs are early-clobber: they are
-// written while later inputs are still to be read.
-// d = a - b (mod 2^192); returns 1 if a < b (unsigned).
-__device__ __forceinline__ uint32_t sub6(const uint32_t* a, const uint32_t* b, uint32_t* d) {
-  uint32_t br;
-  asm("sub.cc.u32 %0, %7, %13;\n\t"
-      "subc.cc.u32 %1, %8, %14;\n\t"
-      "subc.cc.u32 %2, %9, %15;\n\t"
-      "subc.cc.u32 %3, %10, %16;\n\t"
-      "subc.cc.u32 %4, %11, %17;\n\t"
-      "subc.cc.u32 %5, %12, %18;\n\t"
-      "subc.u32 %6, 0, 0;"
-      : "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(br)
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(b[0]), "r"(b[1]), "r"(b[2]),
-        "r"(b[3]), "r"(b[4]), "r"(b[5]));
-  return br & 1u;
-}
-
-// d = k * P for a five-limb P and k < 2^32 (six limbs).  h0..h3 are scratch
-// outputs of the multiply chain (hence the front-end note suppressed here).
-#pragma nv_diag_suppress 550
-__device__ __forceinline__ void mul6(const uint32_t* P, uint32_t k, uint32_t* d) {
-  uint32_t h0, h1, h2, h3;
-  asm("mul.lo.u32 %0, %10, %15;\n\t"
-      "mul.hi.u32 %6, %10, %15;\n\t"
-      "mul.hi.u32 %7, %11, %15;\n\t"
-      "mul.hi.u32 %8, %12, %15;\n\t"
-      "mul.hi.u32 %9, %13, %15;\n\t"
-      "mad.lo.cc.u32 %1, %11, %15, %6;\n\t"
-      "madc.lo.cc.u32 %2, %12, %15, %7;\n\t"
-      "madc.lo.cc.u32 %3, %13, %15, %8;\n\t"
-      "madc.lo.cc.u32 %4, %14, %15, %9;\n\t"
-      "madc.hi.u32 %5, %14, %15, 0;"
-      : "=&r"(d[0]), "=&r"(d[1]), "=&r"(d[2]), "=&r"(d[3]), "=&r"(d[4]), "=&r"(d[5]), "=&r"(h0), "=&r"(h1),
-        "=&r"(h2), "=&r"(h3)
-      : "r"(P[0]), "r"(P[1]), "r"(P[2]), "r"(P[3]), "r"(P[4]), "r"(k));
-}
-#pragma nv_diag_default 550
-
-// Eq. (8) finish from the lazy form: x = S - kP with k = rint(t) (below
-// 3 * 20 * 256), which is round(S / P) or one off (t errs by less than 0.02
-// for up to 20 moduli), then
-// one exact correction each way into the symmetric range (-P/2, P/2] (the
-// lift of S mod P: above floor(P/2) it becomes negative), rounded once to
-// binary64.  All limb arithmetic is exact; only the choice of k is estimated.
-__device__ __forceinline__ double crt_finish_lazy(const CrtLazy& a, const CrtTables& ct) {
-  // S in six 32-bit limbs: the 64-bit lazy sums (each < 2^46) overlap by 32 bits
-  uint32_t S[kSL];
+  for (int i = 0; i < L; ++i) {
+    c += a.s[i] & 0xFFFFFFFFull;  // two 32-bit halves of each 64-bit sum
+    S[i] = static_cast<uint32_t>(c);
+    c = (c >> 32) + (a.s[i] >> 32);
+  }
+  S[L] = static_cast<uint32_t>(c);
+  // S / 2^e, e = 32 (L - 2) + sh, in 64 bits (S < 2^31 P)
+  const uint64_t hi = (static_cast<uint64_t>(S[L]) << 32) | S[L - 1];
+  const uint64_t sn = ct.sh == 32 ? hi : (hi << (32 - ct.sh)) | (S[L - 2] >> ct.sh);
+  const uint64_t q = __umul64hi(sn, ct.recip);  // (S / P) 2^frac, at most 2 low
+  const uint32_t half = 1u << (ct.frac - 1);
+  const uint32_t k = static_cast<uint32_t>((q + half) >> ct.frac);
+  uint32_t R[L];  // S - k P modulo 2^(32 L), which holds |x| <= P / 2 with its sign
   {
-    uint32_t l[kCrtLimbs], h[kCrtLimbs];
+    uint64_t m = 0;
+    uint32_t br = 0;
 #pragma unroll
-    for (int i = 0; i < kCrtLimbs; ++i) {
-      l[i] = static_cast<uint32_t>(a.s[i]);
-      h[i] = static_cast<uint32_t>(a.s[i] >> 32);
+    for (int i = 0; i < L; ++i) {
+      m += static_cast<uint64_t>(ct.P[i]) * k;
+      const uint64_t d = static_cast<uint64_t>(S[i]) - static_cast<uint32_t>(m) - br;
+      R[i] = static_cast<uint32_t>(d);
+      br = static_cast<uint32_t>(d >> 63);
+      m >>= 32;
     }
-    S[0] = l[0];
-    asm("add.cc.u32 %0, %5, %10;\n\t"
-        "addc.cc.u32 %1, %6, %11;\n\t"
-        "addc.cc.u32 %2, %7, %12;\n\t"
-        "addc.cc.u32 %3, %8, %13;\n\t"
-        "addc.u32 %4, %9, 0;"
-        : "=&r"(S[1]), "=&r"(S[2]), "=&r"(S[3]), "=&r"(S[4]), "=&r"(S[5])
-        : "r"(l[1]), "r"(l[2]), "r"(l[3]), "r"(l[4]), "r"(h[4]), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]));
   }
-  const uint32_t k = static_cast<uint32_t>(__float2int_rn(a.t));
-  uint32_t kP[kSL], R[kSL];
-  mul6(ct.P, k, kP);
-  sub6(S, kP, R);  // S - kP, two's complement
-  bool neg = static_cast<int32_t>(R[kSL - 1]) < 0;
-  uint32_t mag[kSL];
-  {
-    const uint32_t zero[kSL] = {0, 0, 0, 0, 0, 0};
-    uint32_t nr[kSL];
-    sub6(zero, R, nr);
+  bool neg = static_cast<int32_t>(R[L - 1]) < 0;
+  const uint32_t f = static_cast<uint32_t>(q) & (2u * half - 1u);
+  if (f - (half - 8u) <= 16u) {
+    // S / P next to a half: the fraction of k is not certain.  With k as
+    // floor(S / P + 1/2) or one off, x lies in (-P, P); lift it into
+    // (-P / 2, P / 2] exactly.  (P is below 2^(32 L); the sign of x comes from
+    // comparing S with k P over L + 1 limbs.)
+    uint64_t m = 0;
+    int64_t top = 0;
+    uint32_t br = 0;
 #pragma unroll
-    for (int i = 0; i < kSL; ++i) mag[i] = neg ? nr[i] : R[i];
+    for (int i = 0; i <= L; ++i) {
+      m += i < L ? static_cast<uint64_t>(ct.P[i < L ? i : 0]) * k : 0ull;
+      const uint64_t d = static_cast<uint64_t>(S[i]) - static_cast<uint32_t>(m) - br;
+      if (i < L) R[i] = static_cast<uint32_t>(d);
+      top = static_cast<int64_t>(d);
+      br = static_cast<uint32_t>(d >> 63);
+      m >>= 32;
+    }
+    neg = top < 0;
+    // |x| against P / 2 by halves: x > P / 2 -> x - P, x <= -P / 2 -> x + P
+    uint32_t mag[L];
+    uint64_t cy = neg ? 1 : 0;
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      cy += neg ? ~R[i] : R[i];
+      mag[i] = static_cast<uint32_t>(cy);
+      cy >>= 32;
+    }
+    int cmp = 0;  // sign of mag - P / 2
+#pragma unroll
+    for (int i = L - 1; i >= 0; --i)
+      if (cmp == 0 && mag[i] != ct.Phalf[i]) cmp = mag[i] > ct.Phalf[i] ? 1 : -1;
+    if (neg ? cmp >= 0 : cmp > 0) {
+      uint32_t b2 = 0;
+#pragma unroll
+      for (int i = 0; i < L; ++i) {
+        const uint64_t d = static_cast<uint64_t>(ct.P[i]) - mag[i] - b2;
+        mag[i] = static_cast<uint32_t>(d);
+        b2 = static_cast<uint32_t>(d >> 63);
+      }
+      neg = !neg;
+    }
+    uint32_t m5[kCrtLimbs] = {0, 0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < L; ++i) m5[i] = mag[i];
+    const double v = limbs_to_double_rn(m5);
+    return neg ? bitsd(dbits(v) ^ 0x8000000000000000ull) : v;
   }
-  // |R| against floor(P/2) = P/2 (P is even: 256 is always a modulus)
-  const uint32_t half[kSL] = {ct.Phalf[0], ct.Phalf[1], ct.Phalf[2], ct.Phalf[3], ct.Phalf[4], 0};
-  uint32_t diff[kSL];
-  const bool below = sub6(mag, half, diff) != 0;  // |R| < P/2
-  const bool equal = !below && (diff[0] | diff[1] | diff[2] | diff[3] | diff[4] | diff[5]) == 0;
-  // R > P/2: R - P (negative, magnitude P - R); R <= -P/2: R + P (magnitude P - |R|)
-  if ((!neg && !below && !equal) || (neg && !below)) {
-    const uint32_t P6[kSL] = {ct.P[0], ct.P[1], ct.P[2], ct.P[3], ct.P[4], 0};
-    sub6(P6, mag, mag);
-    neg = !neg;
+  uint32_t mag[kCrtLimbs] = {0, 0, 0, 0, 0};
+  uint64_t cy = neg ? 1 : 0;
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    cy += neg ? ~R[i] : R[i];
+    mag[i] = static_cast<uint32_t>(cy);
+    cy >>= 32;
   }
-  const double v = limbs_to_double_rn(mag);  // |x| <= P/2 < 2^159: five limbs
+  const double v = limbs_to_double_rn(mag);
   return neg ? bitsd(dbits(v) ^ 0x8000000000000000ull) : v;  // sign flip without an FP64 instruction
 }
 

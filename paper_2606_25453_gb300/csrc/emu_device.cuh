@@ -193,28 +193,22 @@ __device__ __forceinline__ ScaledInt scaled_trunc_bits(uint64_t bits, int shift)
   return r;
 }
 
-// Round an unsigned 128-bit integer to binary64, nearest-even, from its bits.
+// Round an unsigned 128-bit integer to binary64, nearest-even, from its bits:
+// normalise it, keep the top 64 bits with a sticky bit for the rest, round
+// the 53 leading ones, and let the carry run into the exponent.  Straight-
+// line integer code (no FP64 instruction).
 __device__ __forceinline__ double u128_to_double_rn(unsigned __int128 u) {
-  uint64_t hi = static_cast<uint64_t>(u >> 64), lo = static_cast<uint64_t>(u);
-  if (hi == 0 && lo < (1ull << 53)) {  // exact: built from the bits (no FP64 instruction)
-    if (lo == 0) return 0.0;
-    const int Ls = 64 - __clzll(static_cast<long long>(lo));  // 1 .. 53 significant bits
-    const uint64_t m = lo << (53 - Ls);                       // in [2^52, 2^53)
-    return bitsd((static_cast<uint64_t>(Ls - 1 + 1023) << 52) | (m & 0x000FFFFFFFFFFFFFull));
-  }
-  int L = hi ? 128 - __clzll(static_cast<long long>(hi)) : 64 - __clzll(static_cast<long long>(lo));
-  int drop = L - 53;  // >= 1
-  uint64_t top = static_cast<uint64_t>(u >> drop);
-  unsigned __int128 rest = u - (static_cast<unsigned __int128>(top) << drop);
-  unsigned __int128 half = static_cast<unsigned __int128>(1) << (drop - 1);
-  if (rest > half || (rest == half && (top & 1))) top += 1;
-  int exp = drop;  // value = top * 2^exp, top in [2^52, 2^53]
-  if (top == (1ull << 53)) {
-    top >>= 1;
-    exp += 1;
-  }
-  uint64_t bits = (static_cast<uint64_t>(exp + 52 + 1023) << 52) | (top & 0x000FFFFFFFFFFFFFull);
-  return bitsd(bits);
+  const uint64_t hi = static_cast<uint64_t>(u >> 64), lo = static_cast<uint64_t>(u);
+  const uint64_t top = hi ? hi : lo, next = hi ? lo : 0ull;
+  if (top == 0) return 0.0;
+  const int n = __clzll(static_cast<long long>(top));
+  const uint64_t t = (top << n) | (n ? next >> (64 - n) : 0ull);
+  const uint64_t T = t | ((next << n) != 0 ? 1ull : 0ull);
+  const uint64_t mant = T >> 11;  // 53 bits, the leading one included
+  const uint32_t rest = static_cast<uint32_t>(T) & 0x7FFu;
+  const uint64_t up = rest + (static_cast<uint32_t>(mant) & 1u) > 0x400u ? 1u : 0u;
+  // the leading one adds 1 to the exponent field
+  return bitsd((static_cast<uint64_t>((hi ? 1149 : 1085) - n) << 52) + mant + up);
 }
 
 // Signed 128-bit integer to binary64, nearest-even.

@@ -42,8 +42,20 @@ struct CrtTables {
   uint32_t P[kCrtLimbs];
   uint32_t Phalf[kCrtLimbs];          // floor(P/2)
   double invP;                        // 1/P rounded (quotient estimate only)
-  float wP[kMaxModuli];               // w_l / P rounded to binary32 (quotient estimate only)
   int nm;
+};
+
+// The same by pairs of moduli (2 i, 2 i + 1) for crt_finish_pair.
+constexpr int kMaxPairs = kMaxModuli / 2;
+struct CrtPairTables {
+  uint32_t c[kMaxPairs];              // x = r c_lo + r' c_hi is congruent to both residues: 16-bit halves c_lo | c_hi << 16
+  uint32_t off[kMaxPairs];            // a multiple of m m' above any x
+  uint32_t w[kMaxPairs][kCrtLimbs];   // (P / (m m')) times its inverse modulo m m'
+  uint32_t P[kCrtLimbs], Phalf[kCrtLimbs];
+  uint64_t recip;                     // floor(2^(63 + bitlen(P)) / P)
+  int sh;                             // S is shifted right by e = max(0, bitlen(P) - 32) = 32 (limbs - 2) + sh
+  int frac;                           // fraction bits of (S / 2^e) recip / 2^64
+  int limbs, nm;                      // 32-bit limbs of P (at least 2)
 };
 
 // Host-side method constants (api.cu).
@@ -53,6 +65,14 @@ int64_t host_chunk_len_F8(int p);
 int host_scale_bits_II(int nm, int64_t k, int is_complex);
 void host_mod_tables(int nm, ModTables* t);
 void host_crt_tables(int nm, CrtTables* t);
+void host_crt_pair_tables(int nm, CrtPairTables* t);
+// The tables of nm moduli, built once per process.
+struct MethodTables {
+  ModTables mod;
+  CrtTables crt;
+  CrtPairTables pair;
+};
+const MethodTables& method_tables(int nm);
 
 // ---------------------------------------------------------------- launchers
 // Zero `bytes` (rounded up to 16) at the 16-byte aligned p.
@@ -183,7 +203,7 @@ cudaError_t launch_gemm_II(int out_mode, const GemmIIArgs& a, const ModTables& m
 // the residue GEMM, 2 the CRT kernel (after the residue GEMM on the same
 // stream), 3 both.
 cudaError_t launch_gemm_II_tc(int out_mode, const GemmIIArgs& a, const ModTables& mt,
-                              const CrtTables& ct, cudaStream_t st, int part = 3);
+                              const CrtPairTables& ct, cudaStream_t st, int part = 3);
 int gemm_II_tc_tile_m();
 int gemm_II_tc_tile_n();
 size_t gemm_II_tc_residue_bytes(int64_t M, int64_t N, int nm, bool is_complex, int cluster);
