@@ -57,17 +57,6 @@ __device__ __forceinline__ bool a16(const double* X, int64_t ld) {
   return ((reinterpret_cast<uintptr_t>(X) & 15u) | static_cast<uintptr_t>(ld & 1)) == 0;
 }
 
-// index of the problem owning block `blk` in a prefix array start[0..count]
-__device__ __forceinline__ int find_prob(const int* start, int count, int blk) {
-  int lo = 0, hi = count - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (start[mid] <= blk) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 // ---------------------------------------------------------------- scan
 // Blocks [0, startA[count]) scan rows of A (one warp per row, K segments of
 // 2048); the rest scan columns of B (32 columns x 8 K-lanes, segments of 256).

@@ -32,62 +32,50 @@ struct GTriProb {
 
 namespace {
 
-__device__ __forceinline__ int owner(const int* start, int count, int blk) {
-  int lo = 0, hi = count - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(start + mid) <= blk)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
+constexpr int kSplitRun = 8;  // groups of 128 elements along K per split block
 
-// Blocks [0, startA[count]): eight rows of A x 128 elements; the rest: 32
-// columns of B x 128 elements through shared memory.
+// Blocks [0, startA[count]): eight rows of A x kSplitRun groups of 128
+// elements, one row per warp; the rest: 32 columns of B x as many through
+// shared memory.  HBM bound in principle (2 bytes per plane written); what
+// costs is each block's chain of dependent loads (product, table entry,
+// exponent, elements), hence several groups per block: the batch above took
+// 4.59 ms with one group per block and a binary search for the product, 4.01
+// with this and the search by whole warps.
 template <int P>
-__global__ void __launch_bounds__(256) grouped_split_tri_kernel(const GTriProb* __restrict__ probs, int count,
-                                                                const int* __restrict__ startA,
-                                                                const int* __restrict__ startB) {
+__global__ void __launch_bounds__(256, P <= 4 ? 4 : P <= 6 ? 3 : 2) grouped_split_tri_kernel(const GTriProb* __restrict__ probs, int count,
+                                                                   const int* __restrict__ startA,
+                                                                   const int* __restrict__ startB) {
   __shared__ uint64_t tile[32][133];
+  __shared__ int ssum[32][P], sE[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int blk = blockIdx.x;
   const int totA = startA[count];
   const bool first = blk < totA;
   if (!first) blk -= totA;
-  const int pi = owner(first ? startA : startB, count, blk);
+  const int* const start = first ? startA : startB;
+  const int pi = find_prob(start, count, blk);
   const GTriProb& pr = probs[pi];
-  const int64_t rows = first ? pr.M : pr.N, ngroups = (pr.kpad + 127) / 128;
-  const int local = blk - (first ? startA : startB)[pi];
-  const int64_t hbase = (local % ngroups) * 128, h0 = hbase + lane * 4;
-  const int64_t r0 = (local / ngroups) * (first ? 8 : 32);
-  const bool vec = vec16_ok(first ? pr.A : pr.B, first ? pr.lda : pr.ldb);
-  if (!first) {
-    fill_tile_strided(tile, pr.B, pr.ldb, rows, pr.K, r0, hbase, vec);
-    __syncthreads();
-  }
-  const unsigned long long* const maxbits = first ? pr.maxA : pr.maxB;
-  uint16_t* const planes = first ? pr.planesA : pr.planesB;
-  int32_t* const sums = first ? pr.sumA : pr.sumB;
-#pragma unroll 1
-  for (int rl = warp; rl < (first ? 8 : 32); rl += 8) {
-    const int64_t r = r0 + rl;
-    if (r >= rows) break;
+  const int64_t rows = first ? pr.M : pr.N, kpad = pr.kpad, K = pr.K;
+  const int nrun = (static_cast<int>((kpad + 127) / 128) + kSplitRun - 1) / kSplitRun;
+  const int local = blk - start[pi];
+  const int64_t r0 = static_cast<int64_t>(local / nrun) * (first ? 8 : 32), hb = (local % nrun) * (kSplitRun * 128);
+  const int64_t hend = min(hb + kSplitRun * 128, kpad);
+  const int64_t plane = rows * kpad;
+  if (first) {
+    const int64_t r = r0 + warp;
+    if (r >= rows) return;
+    const double* const X = pr.A + r * pr.lda;
+    const bool vec = vec16_ok(pr.A, pr.lda);
+    uint16_t* const dst = pr.planesA + r * kpad;
+    const int E = exp_from_maxbits(pr.maxA, r, rows);
+    if (hb == 0 && lane == 0) pr.EA[r] = E;
     int sum[P];
 #pragma unroll
     for (int t = 0; t < P; ++t) sum[t] = 0;
-    if (h0 < pr.kpad) {
-      const int E = exp_from_maxbits(maxbits, r, rows);
+    for (int64_t h0 = hb + lane * 4; h0 < hend; h0 += 128) {
       uint64_t bits[4];
-      if (first) {
-        load4_kcontig(pr.A + r * pr.lda, h0, pr.K, true, vec, bits);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) bits[q] = tile[rl][q * 33 + lane];
-      }
-      digits4<P>(bits, E, live_count(h0, pr.K), planes + r * pr.kpad + h0, rows * pr.kpad, sum);
-      if (h0 == 0) (first ? pr.EA : pr.FB)[r] = E;
+      load4_kcontig(X, h0, K, true, vec, bits);
+      digits4<P>(bits, E, live_count(h0, K), dst + h0, plane, sum);
     }
     __syncwarp();
     int mine = 0;
@@ -96,7 +84,48 @@ __global__ void __launch_bounds__(256) grouped_split_tri_kernel(const GTriProb* 
       const int s = __reduce_add_sync(0xFFFFFFFFu, sum[t]);
       if (lane == t) mine = s;
     }
-    if (lane < P) atomicAdd(sums + lane * rows + r, mine);
+    if (lane < P) atomicAdd(pr.sumA + lane * rows + r, mine);
+    return;
+  }
+  const bool vec = vec16_ok(pr.B, pr.ldb);
+  const double* const X = pr.B;
+  const int64_t ld = pr.ldb;
+  for (int i = threadIdx.x; i < 32 * P; i += 256) (&ssum[0][0])[i] = 0;
+  if (threadIdx.x < 32 && r0 + threadIdx.x < rows) {
+    const int E = exp_from_maxbits(pr.maxB, r0 + threadIdx.x, rows);
+    sE[threadIdx.x] = E;
+    if (hb == 0) pr.FB[r0 + threadIdx.x] = E;
+  }
+  for (int64_t hbase = hb; hbase < hend; hbase += 128) {
+    __syncthreads();  // the previous group is done with the tile
+    fill_tile_strided(tile, X, ld, rows, K, r0, hbase, vec);
+    __syncthreads();
+    const int64_t h0 = hbase + lane * 4;
+#pragma unroll 1
+    for (int rl = warp; rl < 32; rl += 8) {
+      const int64_t r = r0 + rl;
+      if (r >= rows) break;
+      int sum[P];
+#pragma unroll
+      for (int t = 0; t < P; ++t) sum[t] = 0;
+      if (h0 < kpad) {
+        uint64_t bits[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bits[q] = tile[rl][q * 33 + lane];
+        digits4<P>(bits, sE[rl], live_count(h0, K), pr.planesB + r * kpad + h0, plane, sum);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < P; ++t) {
+        const int s = __reduce_add_sync(0xFFFFFFFFu, sum[t]);
+        if (lane == t) ssum[rl][t] += s;  // only this warp, this lane touches it
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 32 * P; i += 256) {
+    const int rl = i % 32, t = i / 32;
+    if (r0 + rl < rows) atomicAdd(pr.sumB + t * rows + r0 + rl, ssum[rl][t]);
   }
 }
 
@@ -151,9 +180,9 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1) gemm_I_grouped_tc_kernel(c
 }
 
 template <int P, bool ONE>
-__global__ void __launch_bounds__(256) grouped_combine_kernel(const GTriProb* __restrict__ probs, int count,
+__global__ void __launch_bounds__(256, P == 8 && !ONE ? 2 : 0) grouped_combine_kernel(const GTriProb* __restrict__ probs, int count,
                                                               const int* __restrict__ startC) {
-  const int pi = owner(startC, count, blockIdx.x);
+  const int pi = find_prob(startC, count, blockIdx.x);
   const GTriProb& pr = probs[pi];
   KParamsTriComb kp;
   kp.Cs = pr.Cs;
@@ -246,9 +275,9 @@ emu_status_t group_tri_build(emu_handle_s* h, int count, const emu_gemm_desc_t* 
     zero += sh[i].zero;
     rest += sh[i].rest;
     const TriLayout& L = sh[i].L;
-    const int64_t ng = (L.kpad + 127) / 128;
-    sA[i + 1] = sA[i] + static_cast<int>((d[i].m + 7) / 8 * ng);
-    sB[i + 1] = sB[i] + static_cast<int>((d[i].n + 31) / 32 * ng);
+    const int64_t nrun = ((L.kpad + 127) / 128 + kSplitRun - 1) / kSplitRun;
+    sA[i + 1] = sA[i] + static_cast<int>((d[i].m + 7) / 8 * nrun);
+    sB[i + 1] = sB[i] + static_cast<int>((d[i].n + 31) / 32 * nrun);
     sC[i + 1] = sC[i] + static_cast<int>(L.tiles_m * L.tiles_n * kPatches);
     for (int u = 0; u < tp.nunits; ++u) {
       const int64_t cols = std::min<int64_t>((d[i].n + 31) / 32 * 32, kBN);

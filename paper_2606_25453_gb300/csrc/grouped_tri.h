@@ -10,6 +10,21 @@ namespace emu {
 
 constexpr int kGroupTriMaxP = 8;
 
+// Last product whose first block is not beyond blk, by the whole warp: 32
+// starts per step, so two dependent loads for up to 1024 products.
+__device__ __forceinline__ int find_prob(const int* start, int count, int blk) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = count;
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const unsigned in = __ballot_sync(0xFFFFFFFFu, lane * step < n && __ldg(start + lo + min(lane * step, n - 1)) <= blk);
+    const int j = max(__popc(in) - 1, 0) * step;
+    lo += j;
+    n = min(step, n - j);
+  }
+  return lo;
+}
+
 struct GTriProb;  // device table entry of one product
 
 struct GroupTri {

@@ -201,6 +201,7 @@ template <int P, bool ONE>
 __device__ __forceinline__ void combine_patch(const KParamsTriComb& kp, int block) {
   using O = TriOut<P, ONE>;
   __shared__ __int128 sR[kCombRows], sQ[kCombCols];
+  __shared__ int sE[kCombRows], sF[kCombCols];
   constexpr int kPC = kBN / kCombCols, kPR = kBM / kCombRows;
   const int tile = block / (kPC * kPR), part = block % (kPC * kPR);
   const int tm = tile % kp.tiles_m, tn = tile / kp.tiles_m;
@@ -223,10 +224,12 @@ __device__ __forceinline__ void combine_patch(const KParamsTriComb& kp, int bloc
     if (kc == 0) {  // the row and column terms while the planes are on their way
       if (threadIdx.x < kCombRows) {
         const int rr = row0 + threadIdx.x;
+        sE[threadIdx.x] = rr < kp.M ? kp.EA[rr] + kp.escale : 0;
         sR[threadIdx.x] = rr < kp.M ? digit_sum_term<P>(kp.sumA + rr, kp.M) : 0;
       } else if (threadIdx.x < kCombRows + kCombCols) {
         const int c = col0 + threadIdx.x - kCombRows;
         const __int128 k0 = static_cast<__int128>((static_cast<unsigned __int128>(kp.const_hi) << 64) | kp.const_lo);
+        sF[threadIdx.x - kCombRows] = c < kp.N ? kp.FB[c] : 0;
         sQ[threadIdx.x - kCombRows] = (c < kp.N ? digit_sum_term<P>(kp.sumB + c, kp.N) : 0) + k0;
       }
     }
@@ -265,12 +268,12 @@ __device__ __forceinline__ void combine_patch(const KParamsTriComb& kp, int bloc
   }
   __syncthreads();
   if (!live) return;
-  const int erow = kp.EA[row] + kp.escale;
+  const int erow = sE[r];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (col + q >= kp.N) break;
     const __int128 t = S[q] + sR[r] + sQ[cl + q];
-    const double x = scale2_fast(i128_to_double_rn(t), erow + kp.FB[col + q]);
+    const double x = scale2_fast(i128_to_double_rn(t), erow + sF[cl + q]);
     if (!kp.f32) {
       double* cp = static_cast<double*>(kp.C) + static_cast<int64_t>(row) * kp.ldc + col + q;
       *cp = kp.plain ? x : blas_update(kp.alpha, x, kp.beta, kp.beta != 0.0 ? *cp : 0.0);
