@@ -605,14 +605,14 @@ __global__ void split_II_kcontig(const T* __restrict__ X, int64_t ld, int64_t ro
   if (h0 == 0 && r < rows && E_out) E_out[r] = E;
 }
 
-template <typename T, int CW, bool BF, int ND>
+template <typename T, int CW, bool BF, int ND, bool SMALL>
 __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                          int64_t rows_pad, int64_t kpad, int nm, int b,
                                                          const __grid_constant__ ModTables mt,
                                                          const unsigned long long* __restrict__ maxbits,
                                                          const int32_t* __restrict__ Ein, int8_t* __restrict__ res,
                                                          int32_t* __restrict__ E_out, bool vec) {
-  constexpr int TR = CW == 2 ? 16 : 32;  // vectors per tile (two tiles for complex)
+  constexpr int TR = SMALL ? 8 : CW == 2 ? 16 : 32;  // vectors per tile (two tiles for complex)
   __shared__ uint64_t tre[TR][133];
   __shared__ uint64_t tim[CW == 2 ? TR : 1][CW == 2 ? 133 : 1];
   const int64_t hbase = static_cast<int64_t>(blockIdx.x) * 128;
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X
        r0 += static_cast<int64_t>(gridDim.y) * TR) {
     __syncthreads();  // the previous row block is done with the tiles
     if constexpr (CW == 1) {
-      fill_tile_strided(tre, X, ld, rows, k, r0, hbase, vec);
+      fill_tile_strided<TR>(tre, X, ld, rows, k, r0, hbase, vec);
     } else {
       for (int i = threadIdx.x; i < TR * 128; i += 256) {
         const int rl = i % TR, hl = i / TR;
@@ -773,12 +773,26 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
     else
       EMU_SPLIT_II(split_II_kcontig, blocks, 1);
   } else {
-    const int64_t rb = rows_pad / (cw == 2 ? 16 : 32);
+    // Eight vectors per block while more would leave SMs without a block: a
+    // warp then packs one vector instead of two or four in turn.  14 moduli,
+    // whole call: n = 512 32.9 -> 27.9 us; n = 1000 (256 blocks of 32) was 73.6
+    // and took 74.6 with 8, so the line lies at one block per SM.
+    const bool small = bf16 && rows_pad / (cw == 2 ? 16 : 32) * (kpad / 128) < 152;
+    const int64_t rb = rows_pad / (small ? 8 : cw == 2 ? 16 : 32);
     dim3 grid(static_cast<unsigned>(kpad / 128), static_cast<unsigned>(rb < 65535 ? rb : 65535));
-    if (cw == 2)
-      EMU_SPLIT_II(split_II_kstrided, grid, 2);
+#define EMU_STRIDED(CW, ND, SMALL) split_II_kstrided<T, CW, true, ND, SMALL><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS)
+#define EMU_STRIDED_ND(CW, SMALL) \
+  (nd == 2 ? EMU_STRIDED(CW, 2, SMALL) : nd == 4 ? EMU_STRIDED(CW, 4, SMALL) : EMU_STRIDED(CW, 6, SMALL))
+    if (!bf16 && cw == 2)
+      split_II_kstrided<T, 2, false, 6, false><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS);
+    else if (!bf16)
+      split_II_kstrided<T, 1, false, 6, false><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS);
+    else if (cw == 2)
+      small ? EMU_STRIDED_ND(2, true) : EMU_STRIDED_ND(2, false);
     else
-      EMU_SPLIT_II(split_II_kstrided, grid, 1);
+      small ? EMU_STRIDED_ND(1, true) : EMU_STRIDED_ND(1, false);
+#undef EMU_STRIDED_ND
+#undef EMU_STRIDED
   }
 #undef EMU_SPLIT_II
 #undef EMU_SPLIT_II_ARGS

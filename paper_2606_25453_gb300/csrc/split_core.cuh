@@ -67,19 +67,19 @@ __device__ __forceinline__ void load4_kcontig(const T* row, int64_t h0, int64_t 
   for (int q = 0; q < 4; ++q) bits[q] = (live && h0 + q < k) ? elem_bits(__ldg(row + h0 + q)) : 0ull;
 }
 
-// Fill tile[32][133] with 32 K-strided vectors r0 .. r0+31 x 128 elements
+// Fill tile[TR][133] with TR K-strided vectors r0 .. r0+TR-1 x 128 elements
 // hbase .. hbase+127 (element (r, h) at X[h ld + r]; zero outside rows x k),
 // element hl of vector rl at column (hl mod 4) 33 + hl / 4, by all 256
 // threads of the block.  With `vec` (X on a 16-byte boundary, ld a multiple
 // of 16 bytes) each thread reads 16 contiguous bytes: 16 / sizeof(T)
 // consecutive vectors of one K row.
-template <typename T>
+template <int TR = 32, typename T>
 __device__ __forceinline__ void fill_tile_strided(uint64_t (*tile)[133], const T* X, int64_t ld, int64_t rows,
                                                   int64_t k, int64_t r0, int64_t hbase, bool vec) {
   constexpr int V = 16 / static_cast<int>(sizeof(T));  // vectors per 16-byte load
-  constexpr int LPR = 32 / V;                           // threads per K row
+  constexpr int LPR = TR / V;                           // threads per K row
 #pragma unroll 4
-  for (int it = 0; it < 32 * 128 / V / 256; ++it) {
+  for (int it = 0; it < TR * 128 / V / 256; ++it) {
     const int i = threadIdx.x + it * 256;
     const int rl = (i % LPR) * V, hl = i / LPR;
     const int64_t r = r0 + rl, h = hbase + hl;

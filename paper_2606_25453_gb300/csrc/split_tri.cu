@@ -48,23 +48,23 @@ __global__ void __launch_bounds__(256) split_tri_kcontig(const T* __restrict__ X
   if (g0 == 0 && lane == 0) E_out[r] = E;
 }
 
-// K-strided source: a block takes 32 vectors x `per` groups of 128 elements
+// K-strided source: a block takes TR vectors x `per` groups of 128 elements
 // through a shared-memory tile; warp w packs vectors w, w + 8, ..  The
 // exponents are read once per block and one vector is packed at a time, so
 // that four blocks fit an SM (two when the compiler interleaved vectors): both
 // splits of n = 8192, p = 8 took 1.35 ms before, 1.19 after (bytes: 1.06).
-template <typename T, int P>
+template <typename T, int P, int TR>
 __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                           int64_t kpad, int per,
                                                           const unsigned long long* __restrict__ maxbits,
                                                           uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
                                                           int32_t* __restrict__ sums, bool vec) {
-  __shared__ uint64_t tile[32][133];
-  __shared__ int ssum[32][P], sE[32];
+  __shared__ uint64_t tile[TR][133];
+  __shared__ int ssum[TR][P], sE[TR];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * 32;
-  for (int i = threadIdx.x; i < 32 * P; i += 256) (&ssum[0][0])[i] = 0;
-  if (threadIdx.x < 32 && r0 + threadIdx.x < rows) {
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * TR;
+  for (int i = threadIdx.x; i < TR * P; i += 256) (&ssum[0][0])[i] = 0;
+  if (threadIdx.x < TR && r0 + threadIdx.x < rows) {
     const int E = exp_from_maxbits(maxbits, r0 + threadIdx.x, rows);
     sE[threadIdx.x] = E;
     if (blockIdx.y == 0) E_out[r0 + threadIdx.x] = E;
@@ -73,11 +73,11 @@ __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const 
     const int64_t hbase = g * 128;
     if (hbase >= kpad) break;
     __syncthreads();  // the previous group is done with the tile
-    fill_tile_strided(tile, X, ld, rows, k, r0, hbase, vec);
+    fill_tile_strided<TR>(tile, X, ld, rows, k, r0, hbase, vec);
     __syncthreads();
     const int64_t h0 = hbase + lane * 4;
 #pragma unroll 1
-    for (int rl = warp; rl < 32; rl += 8) {
+    for (int rl = warp; rl < TR; rl += 8) {
       const int64_t r = r0 + rl;
       if (r >= rows) break;
       int sum[P];
@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const 
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 32 * P; i += 256) {
-    const int rl = i % 32, t = i / 32;
+  for (int i = threadIdx.x; i < TR * P; i += 256) {
+    const int rl = i % TR, t = i / TR;
     if (r0 + rl < rows) atomicAdd(sums + t * rows + r0 + rl, ssum[rl][t]);
   }
 }
@@ -124,8 +124,16 @@ void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, con
       per *= 2;
       nseg = (ngroups + per - 1) / per;
     }
-    const dim3 grid(static_cast<unsigned>((rows + 31) / 32), static_cast<unsigned>(nseg));
-    split_tri_kstrided<T, P><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+    // Eight vectors per block (64 contiguous bytes per K row of binary64) while
+    // 32 would leave SMs without two blocks: a warp then packs one vector
+    // instead of four in turn.  p = 7, whole call: n = 256 25.2 -> 21.1 us, n =
+    // 1024 94.4 -> 92.4; with enough blocks the shorter rows only cost.
+    const bool small = units * nseg < 2 * static_cast<int64_t>(num_sms);
+    const dim3 grid(static_cast<unsigned>(small ? (rows + 7) / 8 : units), static_cast<unsigned>(nseg));
+    if (small)
+      split_tri_kstrided<T, P, 8><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+    else
+      split_tri_kstrided<T, P, 32><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
   }
 }
 
@@ -133,7 +141,8 @@ template <int P>
 void preload_p() {
   cudaFuncAttributes a;
   cudaFuncGetAttributes(&a, split_tri_kcontig<double, P>);
-  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P>);
+  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P, 8>);
+  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P, 32>);
   if constexpr (P < kTriMaxP) preload_p<P + 1>();
 }
 
