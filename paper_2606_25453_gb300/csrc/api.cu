@@ -635,15 +635,13 @@ Plan plan_II(int64_t m, int64_t n, int64_t k, int nm, int nsets, int es) {
   size_t off = 0;
   pl.off_maxA = off; off += al256(8 * static_cast<size_t>(m > 0 ? m : 1));
   pl.off_maxB = off; off += al256(8 * static_cast<size_t>(n > 0 ? n : 1));
+  // norm-based scaling: 128-bit sums of squares, zeroed with the maxima
+  pl.off_accA = off; off += al256(16 * static_cast<size_t>(m > 0 ? m : 1));
+  pl.off_accB = off; off += al256(16 * static_cast<size_t>(n > 0 ? n : 1));
   pl.off_EA = off; off += al256(4 * static_cast<size_t>(m > 0 ? m : 1));
   pl.off_FB = off; off += al256(4 * static_cast<size_t>(n > 0 ? n : 1));
   pl.off_hatA = off; off += al256(static_cast<size_t>(es) * nsets * nm * pl.rows_a * pl.cols);
   pl.off_hatB = off; off += al256(static_cast<size_t>(es) * nsets * nm * pl.rows_b * pl.cols);
-  // norm-based scaling: 128-bit sums of squares and the exponents
-  pl.off_accA = off; off += al256(16 * static_cast<size_t>(m > 0 ? m : 1));
-  pl.off_accB = off; off += al256(16 * static_cast<size_t>(n > 0 ? n : 1));
-  pl.off_nEA = off; off += al256(4 * static_cast<size_t>(m > 0 ? m : 1));
-  pl.off_nEB = off; off += al256(4 * static_cast<size_t>(n > 0 ? n : 1));
   // tcgen05 kernel: the residue planes (one byte per output and modulus; row
   // tiles rounded to whole CTA-pair tiles)
   pl.off_scratch = off; off += es == 2 ? al256(gemm_II_tc_residue_bytes(m, n, nm, nsets == 3, 2)) : 0;
@@ -895,32 +893,37 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   // maxima) or norm-based scaling (hA, hB, exponents of the 2-norms)
   int bA = host_scale_bits_II(nm, k, cw == 2), bB = bA;
   if (norm) host_norm_halves_II(nm, &bA, &bB);
-  auto* nEA = reinterpret_cast<int32_t*>(ws + pl.off_nEA);
-  auto* nEB = reinterpret_cast<int32_t*>(ws + pl.off_nEB);
+  auto* accA = reinterpret_cast<unsigned long long*>(ws + pl.off_accA);
+  auto* accB = reinterpret_cast<unsigned long long*>(ws + pl.off_accB);
   const MethodTables& tabs = method_tables(nm);
   const ModTables& mt = tabs.mod;
   const bool do_a = phase != 1, do_b = phase != 2;
   trace_begin(h, PH_SCAN, st);
   const unsigned long long* mA = v.maxA ? v.maxA : maxA;
   const unsigned long long* mB = v.maxB ? v.maxB : maxB;
+  const bool both = do_a && do_b;
   if (!v.maxA) {
-    const bool both = do_a && do_b;
-    if (both) launch_zero(ws + pl.off_maxA, pl.off_maxB + sizeof(*maxB) * v.N - pl.off_maxA, st);
+    if (both) {  // maxima, and the sums of squares behind them, in one launch
+      const size_t end = norm ? pl.off_accB + 2 * sizeof(*accB) * v.N : pl.off_maxB + sizeof(*maxB) * v.N;
+      launch_zero(ws + pl.off_maxA, end - pl.off_maxA, st);
+    }
     launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, do_a ? maxA : nullptr, B, v.ldB, v.b_kcontig, v.N,
                    do_b ? maxB : nullptr, k, cw, both, h->status, st);
   }
-  if (norm && do_a)
-    launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, k, cw, mA, reinterpret_cast<unsigned long long*>(ws + pl.off_accA),
-                   nEA, st);
-  if (norm && do_b)
-    launch_norm<T>(B, v.ldB, v.b_kcontig, v.N, k, cw, mB, reinterpret_cast<unsigned long long*>(ws + pl.off_accB),
-                   nEB, st);
-  trace_end(h, PH_SCAN, st, (do_a + do_b) * (norm ? 3 : 1));
+  if (norm) {
+    if (v.maxA || !both) {
+      if (do_a) launch_zero(accA, 2 * sizeof(*accA) * v.M, st);
+      if (do_b) launch_zero(accB, 2 * sizeof(*accB) * v.N, st);
+    }
+    launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, mA, do_a ? accA : nullptr, B, v.ldB, v.b_kcontig, v.N, mB,
+                   do_b ? accB : nullptr, k, cw, st);
+  }
+  trace_end(h, PH_SCAN, st, norm ? 3 : do_a + do_b);
   trace_begin(h, PH_SPLIT, st);
   if (do_a)
-    launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, mA, resA, EA, st, norm ? nEA : nullptr, tc);
+    launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, mA, resA, EA, st, norm ? accA : nullptr, tc);
   if (do_b)
-    launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, mB, resB, FB, st, norm ? nEB : nullptr, tc);
+    launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, mB, resB, FB, st, norm ? accB : nullptr, tc);
   trace_end(h, PH_SPLIT, st, do_a + do_b);
   if (phase == 1) return cuda_err(cudaGetLastError());
   CUtensorMap ta, tb;

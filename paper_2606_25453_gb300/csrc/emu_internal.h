@@ -98,12 +98,14 @@ void launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t 
 template <typename T>
 void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
                      int cw, const ModTables& tabs, const unsigned long long* maxbits, int8_t* res,
-                     int32_t* E, cudaStream_t st, const int32_t* Ein = nullptr, bool bf16 = false);
-// Norm-based Scheme II scaling: E[r] with ||x_r||_2 < 2^E[r], computed
-// exactly (maxbits from launch_scan; acc: 2 rows words of scratch).
+                     int32_t* E, cudaStream_t st, const unsigned long long* acc = nullptr, bool bf16 = false);
+// Norm-based Scheme II scaling: the sums of squares of both operands' vectors
+// in one launch, exact in any order (maxima from launch_scan; acc: two words
+// per vector, zeroed; null: that operand is left out).
 template <typename T>
-void launch_norm(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
-                 const unsigned long long* maxbits, unsigned long long* acc, int32_t* E, cudaStream_t st);
+void launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
+                 unsigned long long* accA, const T* B, int64_t ldB, bool b_kcontig, int64_t N,
+                 const unsigned long long* maxB, unsigned long long* accB, int64_t k, int cw, cudaStream_t st);
 void host_norm_halves_II(int nm, int* hA, int* hB);
 
 // Output modes of the Scheme I kernel.

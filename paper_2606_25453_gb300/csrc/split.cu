@@ -252,59 +252,77 @@ __device__ __forceinline__ unsigned __int128 shfl_add_u128(unsigned __int128 v) 
   return v;
 }
 
-// Same launch shapes as scan_kernel; acc: 2 words per row, zeroed first.
-template <typename T, bool KCONTIG>
-__global__ void norm_kernel(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int cw, int64_t seg,
-                            const unsigned long long* __restrict__ maxbits, unsigned long long* __restrict__ acc) {
-  if (KCONTIG) {
-    const int lane = threadIdx.x & 31;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= rows) return;
-    const uint64_t mb = maxbits[r];
-    if (mb == 0 || mb >= 0x7FF0000000000000ull) return;  // zero row / non-finite (flagged by the scan)
-    const int Emax = frexp_exp_bits(mb);
-    const int64_t len = k * cw;
-    const int64_t h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    const int64_t h1 = h0 + seg < len ? h0 + seg : len;
-    const T* row = X + r * ld * cw;
-    unsigned __int128 sum = 0;
+// One launch sums both operands (two memsets, two sums and two finishing
+// launches before: 300 x 200 x 300, 14 moduli, as a graph 39.8 -> 28.5 us; 2905
+// x 1777 x 803 297 -> 278 us; the splits read the exponent off the sum): the
+// blocks of the first, then those of the
+// second), with the shapes of scan_kernel's scalar loads; acc: 2 words per
+// vector, zeroed first.
+template <typename T>
+struct NormOperand {
+  const T* X;
+  int64_t ld, rows, k, seg;
+  int64_t vb, blocks;  // blocks per K segment; all blocks
+  const unsigned long long* maxbits;
+  unsigned long long* acc;
+  int cw;
+  bool kcontig;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ NormOperand<T> a,
+                                                   const __grid_constant__ NormOperand<T> b) {
+  __shared__ unsigned __int128 red[8][32];
+  const bool first = blockIdx.x < a.blocks;
+  const NormOperand<T>& op = first ? a : b;
+  const int64_t blk = first ? blockIdx.x : blockIdx.x - a.blocks;
+  const int64_t bx = blk % op.vb, by = blk / op.vb;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cw = op.cw;
+  const int64_t r = op.kcontig ? bx * 8 + warp : bx * 32 + lane;
+  // a zero vector adds nothing; a non-finite one was flagged by the scan
+  const uint64_t mb = r < op.rows ? op.maxbits[r] : 0ull;
+  const bool live = mb != 0 && mb < 0x7FF0000000000000ull;
+  const int Emax = live ? frexp_exp_bits(mb) : 0;
+  unsigned __int128 sum = 0;
+  if (op.kcontig) {
+    if (!live) return;
+    const int64_t len = op.k * cw, h0 = by * op.seg;
+    const int64_t h1 = h0 + op.seg < len ? h0 + op.seg : len;
+    const T* row = op.X + r * op.ld * cw;
 #pragma unroll 4
     for (int64_t h = h0 + lane; h < h1; h += 32) sum += sq_ceil64(load_bits(row + h), Emax);
     sum = shfl_add_u128(sum);
-    if (lane == 0 && sum) atomic_add_u128(acc + 2 * r, sum);
-  } else {
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
-    const int64_t h0 = static_cast<int64_t>(blockIdx.y) * seg;
-    const int64_t h1 = h0 + seg < k ? h0 + seg : k;
-    if (r >= rows) return;
-    const uint64_t mb = maxbits[r];
-    if (mb == 0 || mb >= 0x7FF0000000000000ull) return;
-    const int Emax = frexp_exp_bits(mb);
-    unsigned __int128 sum = 0;
+    if (lane == 0 && sum) atomic_add_u128(op.acc + 2 * r, sum);
+    return;
+  }
+  if (live) {
+    const int64_t h0 = by * op.seg, h1 = h0 + op.seg < op.k ? h0 + op.seg : op.k;
 #pragma unroll 4
-    for (int64_t h = h0 + threadIdx.y; h < h1; h += blockDim.y) {
-      const T* p = X + (h * ld + r) * cw;
+    for (int64_t h = h0 + warp; h < h1; h += 8) {
+      const T* p = op.X + (h * op.ld + r) * cw;
       sum += sq_ceil64(load_bits(p), Emax);
       if (cw == 2) sum += sq_ceil64(load_bits(p + 1), Emax);
     }
-    if (sum) atomic_add_u128(acc + 2 * r, sum);
+  }
+  red[warp][lane] = sum;
+  __syncthreads();
+  if (warp == 0 && live) {
+    for (int q = 1; q < 8; ++q) sum += red[q][lane];
+    if (sum) atomic_add_u128(op.acc + 2 * r, sum);
   }
 }
 
-__global__ void norm_finish_kernel(int64_t rows, const unsigned long long* __restrict__ maxbits,
-                                   const unsigned long long* __restrict__ acc, int32_t* __restrict__ E) {
-  const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
+// Exponent e of vector r with ||x||_2 < 2^e from its sum of squares.
+__device__ __forceinline__ int exp_from_norm(const unsigned long long* acc, const unsigned long long* maxbits,
+                                             int64_t r, int64_t rows) {
+  if (r >= rows) return 0;
   const unsigned long long lo = acc[2 * r], hi = acc[2 * r + 1];
   const uint64_t mb = maxbits[r];
-  if ((lo | hi) == 0 || mb >= 0x7FF0000000000000ull) {
-    E[r] = 0;
-    return;
-  }
+  if ((lo | hi) == 0 || mb >= 0x7FF0000000000000ull) return 0;
   const int L = hi ? 128 - __clzll(static_cast<long long>(hi)) : 64 - __clzll(static_cast<long long>(lo));
   const int d = L - 64;
   const int ep = d >= 0 ? (d + 1) / 2 : -((-d) / 2);  // ceil(d / 2)
-  E[r] = frexp_exp_bits(mb) + ep;
+  return frexp_exp_bits(mb) + ep;
 }
 
 // ------------------------------------------------------------------ split I
@@ -572,21 +590,21 @@ __device__ __forceinline__ void residues4(const ModTables& mt, int nm, int shift
 // ((q*nm + l)*rows_pad + r)*kpad + h of `res` (set = 0 for real; 0, 1, 2 =
 // re, im, re + im for complex); elements are INT8, or bf16 (BF) for the
 // tcgen05 kernel.  Row exponent: of the maximum (worst-case
-// scaling) or of the 2-norm (Ein).  K-contiguous sources: one warp per
+// scaling) or of the 2-norm (acc).  K-contiguous sources: one warp per
 // (vector, 128 K-elements), lane l takes elements 4l .. 4l+3 and writes one
 // word per plane; strided sources go through a shared-memory tile of 32
 // vectors (16 for complex) x 128 elements as in the Scheme I split.
 template <typename T, int CW, bool BF, int ND>
 __global__ void split_II_kcontig(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int64_t rows_pad,
                                  int64_t kpad, int nm, int b, const __grid_constant__ ModTables mt,
-                                 const unsigned long long* __restrict__ maxbits, const int32_t* __restrict__ Ein,
+                                 const unsigned long long* __restrict__ maxbits, const unsigned long long* __restrict__ acc,
                                  int8_t* __restrict__ res, int32_t* __restrict__ E_out, bool vec) {
   const int lane = threadIdx.x & 31;
   const int64_t ngroups = kpad / 128;
   const int64_t w = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (w >= rows_pad * ngroups) return;
   const int64_t r = w / ngroups, h0 = (w % ngroups) * 128 + lane * 4;
-  const int E = Ein ? (r < rows ? Ein[r] : 0) : exp_from_maxbits(maxbits, r, rows);
+  const int E = acc ? exp_from_norm(acc, maxbits, r, rows) : exp_from_maxbits(maxbits, r, rows);
   uint64_t re[4], im[4];
   if constexpr (CW == 1) {
     load4_kcontig(X + (r < rows ? r : 0) * ld, h0, k, r < rows, vec, re);
@@ -610,7 +628,7 @@ __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X
                                                          int64_t rows_pad, int64_t kpad, int nm, int b,
                                                          const __grid_constant__ ModTables mt,
                                                          const unsigned long long* __restrict__ maxbits,
-                                                         const int32_t* __restrict__ Ein, int8_t* __restrict__ res,
+                                                         const unsigned long long* __restrict__ acc, int8_t* __restrict__ res,
                                                          int32_t* __restrict__ E_out, bool vec) {
   constexpr int TR = SMALL ? 8 : CW == 2 ? 16 : 32;  // vectors per tile (two tiles for complex)
   __shared__ uint64_t tre[TR][133];
@@ -637,7 +655,7 @@ __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X
     for (int rl = warp; rl < TR; rl += 8) {
       const int64_t r = r0 + rl;
       if (r >= rows_pad) continue;
-      const int E = Ein ? (r < rows ? Ein[r] : 0) : exp_from_maxbits(maxbits, r, rows);
+      const int E = acc ? exp_from_norm(acc, maxbits, r, rows) : exp_from_maxbits(maxbits, r, rows);
       uint64_t re[4], im[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -753,13 +771,13 @@ template void launch_split_I<float>(const float*, int64_t, bool, int64_t, int64_
 template <typename T>
 void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
                      int cw, const ModTables& tabs, const unsigned long long* maxbits, int8_t* res,
-                     int32_t* E, cudaStream_t st, const int32_t* Ein, bool bf16) {
+                     int32_t* E, cudaStream_t st, const unsigned long long* acc, bool bf16) {
   const int64_t rows_pad = split_rows(rows), kpad = split_cols_II(k);
   if (rows_pad == 0 || kpad == 0) return;
   // 14-bit digits that hold |a'| < 2^b (bf16 planes; the INT8 form has its own)
   const int nd = b <= 28 ? 2 : b <= 56 ? 4 : 6;
   const bool vec = cw == 1 && vec16_ok(X, ld);
-#define EMU_SPLIT_II_ARGS X, ld, rows, k, rows_pad, kpad, nm, b, tabs, maxbits, Ein, res, E, vec
+#define EMU_SPLIT_II_ARGS X, ld, rows, k, rows_pad, kpad, nm, b, tabs, maxbits, acc, res, E, vec
 #define EMU_SPLIT_II(KERNEL, GRID, CW)                                             \
   (!bf16      ? KERNEL<T, CW, false, 6><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS) \
    : nd == 2 ? KERNEL<T, CW, true, 2><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS)  \
@@ -799,33 +817,38 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
 }
 
 template <typename T>
-void launch_norm(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
-                 const unsigned long long* maxbits, unsigned long long* acc, int32_t* E, cudaStream_t st) {
-  if (rows == 0) return;
-  cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 2 * rows, st);
-  if (k > 0) {
-    if (kcontig) {
-      const int64_t len = k * cw, rb = (rows + 7) / 8, seg = scan_seg(rb, len, 2048, 256);
-      dim3 grid(static_cast<unsigned>(rb), static_cast<unsigned>((len + seg - 1) / seg));
-      norm_kernel<T, true><<<grid, 256, 0, st>>>(X, ld, rows, k, cw, seg, maxbits, acc);
-    } else {
-      const int64_t rb = (rows + 31) / 32, seg = scan_seg(rb, k, 256, 32);
-      dim3 grid(static_cast<unsigned>(rb), static_cast<unsigned>((k + seg - 1) / seg));
-      norm_kernel<T, false><<<grid, dim3(32, 8), 0, st>>>(X, ld, rows, k, cw, seg, maxbits, acc);
-    }
-  }
-  norm_finish_kernel<<<static_cast<unsigned>((rows + 255) / 256), 256, 0, st>>>(rows, maxbits, acc, E);
+static NormOperand<T> norm_operand(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
+                                   const unsigned long long* maxbits, unsigned long long* acc) {
+  NormOperand<T> op{X, ld, rows, k, 0, 1, 0, maxbits, acc, cw, kcontig};
+  if (rows == 0 || k == 0) return op;
+  const int64_t len = kcontig ? k * cw : k;
+  op.vb = (rows + (kcontig ? 7 : 31)) / (kcontig ? 8 : 32);
+  op.seg = kcontig ? scan_seg(op.vb, len, 2048, 256) : scan_seg(op.vb, len, 256, 32);
+  op.blocks = op.vb * ((len + op.seg - 1) / op.seg);
+  return op;
 }
-template void launch_norm<double>(const double*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
-                                  unsigned long long*, int32_t*, cudaStream_t);
-template void launch_norm<float>(const float*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
-                                 unsigned long long*, int32_t*, cudaStream_t);
+
+template <typename T>
+void launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
+                 unsigned long long* accA, const T* B, int64_t ldB, bool b_kcontig, int64_t N,
+                 const unsigned long long* maxB, unsigned long long* accB, int64_t k, int cw, cudaStream_t st) {
+  const NormOperand<T> a = norm_operand(A, ldA, a_kcontig, accA ? M : 0, k, cw, maxA, accA);
+  const NormOperand<T> b = norm_operand(B, ldB, b_kcontig, accB ? N : 0, k, cw, maxB, accB);
+  if (a.blocks + b.blocks == 0) return;
+  norm_kernel<T><<<static_cast<unsigned>(a.blocks + b.blocks), 256, 0, st>>>(a, b);
+}
+template void launch_norm<double>(const double*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
+                                  const double*, int64_t, bool, int64_t, const unsigned long long*,
+                                  unsigned long long*, int64_t, int, cudaStream_t);
+template void launch_norm<float>(const float*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
+                                 const float*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
+                                 int64_t, int, cudaStream_t);
 
 template void launch_split_II<double>(const double*, int64_t, bool, int64_t, int64_t, int, int, int,
                                       const ModTables&, const unsigned long long*, int8_t*, int32_t*,
-                                      cudaStream_t, const int32_t*, bool);
+                                      cudaStream_t, const unsigned long long*, bool);
 template void launch_split_II<float>(const float*, int64_t, bool, int64_t, int64_t, int, int, int,
                                      const ModTables&, const unsigned long long*, int8_t*, int32_t*,
-                                     cudaStream_t, const int32_t*, bool);
+                                     cudaStream_t, const unsigned long long*, bool);
 
 }  // namespace emu
