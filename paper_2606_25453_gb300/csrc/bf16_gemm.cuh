@@ -140,6 +140,7 @@ __device__ __forceinline__ Ctx setup(uint8_t* smem_raw) {
   else
     __syncthreads();
   tc_fence_after();
+  grid_begin();  // barriers and tensor memory were set up while the kernel before ended
   c.tmem = *slot;
   c.ab.local = abort_local;
   c.ab.peer = PAIR ? cluster_addr(smem_u32(const_cast<int*>(abort_local)), c.crank ^ 1u) : 0u;
@@ -330,17 +331,19 @@ cudaError_t launch(K kernel, int64_t nitems, int num_sms, cudaStream_t st, const
   const int64_t most = PAIR ? num_sms / 2 : num_sms;
   const int64_t n = nitems < most ? nitems : most;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 2;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3(static_cast<unsigned>(PAIR ? 2 * n : n));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = Cfg<PAIR>::kSmem;
   cfg.stream = st;
   cfg.attrs = at;
-  cfg.numAttrs = PAIR ? 1 : 0;
+  cfg.numAttrs = PAIR ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

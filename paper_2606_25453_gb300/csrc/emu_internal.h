@@ -9,6 +9,25 @@
 
 namespace emu {
 
+// Launch a kernel that begins with grid_begin() so that its launch and the end
+// of the kernel before it overlap: a small product is six or seven short
+// kernels, and what passed between them was a third of its time.  256^3, p = 7:
+// 32.8 -> 21.9 us per call; 2905 x 1777 x 803, 14 moduli, norm scaling: 278 ->
+// 260; 3001 x 2047 x 2500 complex64: 755 -> 742.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int kMaxModuli = 20;  // Scheme II moduli supported
 constexpr int kCrtLimbs = 5;     // P < 2^160 for up to 20 moduli
 constexpr int kSplitRowAlign = 128;

@@ -233,6 +233,7 @@ __device__ __forceinline__ void load_pairs(const uint8_t* p, int64_t plane, int 
 template <int MODE, int L>
 __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KParamsCRT kp,
                                                      const __grid_constant__ CrtPairTables ct) {
+  grid_begin();
   constexpr bool CPLX = MODE == II_Z3M || MODE == II_C3M;
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int ncq = (kp.N + kCrtCols - 1) / kCrtCols;
@@ -364,12 +365,11 @@ cudaError_t launch_crt(const GemmIIArgs& a, const CrtPairTables& ct, cudaStream_
   if (threads == 0) return cudaSuccess;
   const unsigned grid = static_cast<unsigned>((threads + 255) / 256);
   switch (ct.limbs) {
-    case 2: crt_II_kernel<MODE, 2><<<grid, 256, 0, st>>>(kp, ct); break;
-    case 3: crt_II_kernel<MODE, 3><<<grid, 256, 0, st>>>(kp, ct); break;
-    case 4: crt_II_kernel<MODE, 4><<<grid, 256, 0, st>>>(kp, ct); break;
-    default: crt_II_kernel<MODE, 5><<<grid, 256, 0, st>>>(kp, ct); break;
+    case 2: return launch_after(crt_II_kernel<MODE, 2>, grid, 256, st, kp, ct);
+    case 3: return launch_after(crt_II_kernel<MODE, 3>, grid, 256, st, kp, ct);
+    case 4: return launch_after(crt_II_kernel<MODE, 4>, grid, 256, st, kp, ct);
+    default: return launch_after(crt_II_kernel<MODE, 5>, grid, 256, st, kp, ct);
   }
-  return cudaGetLastError();
 }
 
 // part: 1 = the residue GEMM, 2 = the CRT kernel, 3 = both.

@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1) gemm_I_tc_kernel(const __g
 // A block combines a 32 x 32 patch (combine_patch).
 template <int P, bool ONE>
 __global__ void __launch_bounds__(256) combine_I_kernel(const __grid_constant__ KParamsTriComb kp) {
+  grid_begin();
   combine_patch<P, ONE>(kp, static_cast<int>(blockIdx.x));
 }
 
@@ -87,11 +88,8 @@ template <int P>
 cudaError_t launch_combine(const KParamsTriComb& kp, bool one, cudaStream_t st) {
   const unsigned grid =
       static_cast<unsigned>(kp.tiles_m * kp.tiles_n * (kBN / kCombCols) * (kBM / kCombRows));
-  if (one)
-    combine_I_kernel<P, true><<<grid, 256, 0, st>>>(kp);
-  else
-    combine_I_kernel<P, false><<<grid, 256, 0, st>>>(kp);
-  return cudaGetLastError();
+  return one ? launch_after(combine_I_kernel<P, true>, grid, 256, st, kp)
+             : launch_after(combine_I_kernel<P, false>, grid, 256, st, kp);
 }
 
 template <int P>

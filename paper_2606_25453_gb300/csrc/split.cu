@@ -186,6 +186,7 @@ __device__ __forceinline__ void scan_kstrided(const ScanOperand<T>& op, int64_t 
 template <typename T>
 __global__ void __launch_bounds__(256) scan_kernel(const __grid_constant__ ScanOperand<T> a,
                                                    const __grid_constant__ ScanOperand<T> b, int* status) {
+  grid_begin();
   __shared__ uint64_t red[8][32 * 4];
   const bool first = blockIdx.x < a.blocks;
   const ScanOperand<T>& op = first ? a : b;
@@ -252,12 +253,11 @@ __device__ __forceinline__ unsigned __int128 shfl_add_u128(unsigned __int128 v) 
   return v;
 }
 
-// One launch sums both operands (two memsets, two sums and two finishing
-// launches before: 300 x 200 x 300, 14 moduli, as a graph 39.8 -> 28.5 us; 2905
-// x 1777 x 803 297 -> 278 us; the splits read the exponent off the sum): the
-// blocks of the first, then those of the
-// second), with the shapes of scan_kernel's scalar loads; acc: 2 words per
-// vector, zeroed first.
+// One launch sums both operands, the blocks of the first, then those of the
+// second, with the shapes of scan_kernel's scalar loads; acc: 2 words per
+// vector, zeroed first.  The splits read the exponent off the sum.  Two
+// memsets, two sums and two finishing launches before: 300 x 200 x 300, 14
+// moduli, as a graph 39.8 -> 28.5 us; 2905 x 1777 x 803 297 -> 278 us.
 template <typename T>
 struct NormOperand {
   const T* X;
@@ -272,6 +272,7 @@ struct NormOperand {
 template <typename T>
 __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ NormOperand<T> a,
                                                    const __grid_constant__ NormOperand<T> b) {
+  grid_begin();
   __shared__ unsigned __int128 red[8][32];
   const bool first = blockIdx.x < a.blocks;
   const NormOperand<T>& op = first ? a : b;
@@ -599,6 +600,7 @@ __global__ void split_II_kcontig(const T* __restrict__ X, int64_t ld, int64_t ro
                                  int64_t kpad, int nm, int b, const __grid_constant__ ModTables mt,
                                  const unsigned long long* __restrict__ maxbits, const unsigned long long* __restrict__ acc,
                                  int8_t* __restrict__ res, int32_t* __restrict__ E_out, bool vec) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const int64_t ngroups = kpad / 128;
   const int64_t w = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -630,6 +632,7 @@ __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X
                                                          const unsigned long long* __restrict__ maxbits,
                                                          const unsigned long long* __restrict__ acc, int8_t* __restrict__ res,
                                                          int32_t* __restrict__ E_out, bool vec) {
+  grid_begin();
   constexpr int TR = SMALL ? 8 : CW == 2 ? 16 : 32;  // vectors per tile (two tiles for complex)
   __shared__ uint64_t tre[TR][133];
   __shared__ uint64_t tim[CW == 2 ? TR : 1][CW == 2 ? 133 : 1];
@@ -684,13 +687,14 @@ static int64_t scan_seg(int64_t vec_blocks, int64_t len, int64_t seg0, int64_t s
 }
 
 __global__ void zero_kernel(uint4* p, int64_t n) {
+  grid_begin();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) p[i] = make_uint4(0, 0, 0, 0);
 }
 
 void launch_zero(void* p, size_t bytes, cudaStream_t st) {
   const int64_t n = static_cast<int64_t>((bytes + 15) / 16);
-  if (n > 0) zero_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(static_cast<uint4*>(p), n);
+  if (n > 0) launch_after(zero_kernel, static_cast<unsigned>((n + 255) / 256), 256, st, static_cast<uint4*>(p), n);
 }
 
 template <typename T>
@@ -718,7 +722,7 @@ void launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned lo
   const ScanOperand<T> a = scan_operand(A, ldA, a_kcontig, maxA ? M : 0, k, cw, maxA);
   const ScanOperand<T> b = scan_operand(B, ldB, b_kcontig, maxB ? N : 0, k, cw, maxB);
   if (a.blocks + b.blocks == 0) return;
-  scan_kernel<T><<<static_cast<unsigned>(a.blocks + b.blocks), 256, 0, st>>>(a, b, status);
+  launch_after(scan_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b, status);
 }
 template void launch_scan<double>(const double*, int64_t, bool, int64_t, unsigned long long*, const double*, int64_t,
                                   bool, int64_t, unsigned long long*, int64_t, int, bool, int*, cudaStream_t);
@@ -779,10 +783,10 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
   const bool vec = cw == 1 && vec16_ok(X, ld);
 #define EMU_SPLIT_II_ARGS X, ld, rows, k, rows_pad, kpad, nm, b, tabs, maxbits, acc, res, E, vec
 #define EMU_SPLIT_II(KERNEL, GRID, CW)                                             \
-  (!bf16      ? KERNEL<T, CW, false, 6><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS) \
-   : nd == 2 ? KERNEL<T, CW, true, 2><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS)  \
-   : nd == 4 ? KERNEL<T, CW, true, 4><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS)  \
-             : KERNEL<T, CW, true, 6><<<GRID, 256, 0, st>>>(EMU_SPLIT_II_ARGS))
+  (!bf16     ? launch_after(KERNEL<T, CW, false, 6>, GRID, 256, st, EMU_SPLIT_II_ARGS) \
+   : nd == 2 ? launch_after(KERNEL<T, CW, true, 2>, GRID, 256, st, EMU_SPLIT_II_ARGS)  \
+   : nd == 4 ? launch_after(KERNEL<T, CW, true, 4>, GRID, 256, st, EMU_SPLIT_II_ARGS)  \
+             : launch_after(KERNEL<T, CW, true, 6>, GRID, 256, st, EMU_SPLIT_II_ARGS))
   if (kcontig) {
     const int64_t warps = rows_pad * (kpad / 128);
     const unsigned blocks = static_cast<unsigned>((warps + 7) / 8);
@@ -798,13 +802,13 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
     const bool small = bf16 && rows_pad / (cw == 2 ? 16 : 32) * (kpad / 128) < 152;
     const int64_t rb = rows_pad / (small ? 8 : cw == 2 ? 16 : 32);
     dim3 grid(static_cast<unsigned>(kpad / 128), static_cast<unsigned>(rb < 65535 ? rb : 65535));
-#define EMU_STRIDED(CW, ND, SMALL) split_II_kstrided<T, CW, true, ND, SMALL><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS)
+#define EMU_STRIDED(CW, ND, SMALL) launch_after(split_II_kstrided<T, CW, true, ND, SMALL>, grid, 256, st, EMU_SPLIT_II_ARGS)
 #define EMU_STRIDED_ND(CW, SMALL) \
   (nd == 2 ? EMU_STRIDED(CW, 2, SMALL) : nd == 4 ? EMU_STRIDED(CW, 4, SMALL) : EMU_STRIDED(CW, 6, SMALL))
     if (!bf16 && cw == 2)
-      split_II_kstrided<T, 2, false, 6, false><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS);
+      launch_after(split_II_kstrided<T, 2, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS);
     else if (!bf16)
-      split_II_kstrided<T, 1, false, 6, false><<<grid, 256, 0, st>>>(EMU_SPLIT_II_ARGS);
+      launch_after(split_II_kstrided<T, 1, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS);
     else if (cw == 2)
       small ? EMU_STRIDED_ND(2, true) : EMU_STRIDED_ND(2, false);
     else
@@ -835,7 +839,7 @@ void launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsig
   const NormOperand<T> a = norm_operand(A, ldA, a_kcontig, accA ? M : 0, k, cw, maxA, accA);
   const NormOperand<T> b = norm_operand(B, ldB, b_kcontig, accB ? N : 0, k, cw, maxB, accB);
   if (a.blocks + b.blocks == 0) return;
-  norm_kernel<T><<<static_cast<unsigned>(a.blocks + b.blocks), 256, 0, st>>>(a, b);
+  launch_after(norm_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b);
 }
 template void launch_norm<double>(const double*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
                                   const double*, int64_t, bool, int64_t, const unsigned long long*,

@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(256) split_tri_kcontig(const T* __restrict__ X
                                                          const unsigned long long* __restrict__ maxbits,
                                                          uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
                                                          int32_t* __restrict__ sums, bool vec) {
+  grid_begin();
   const int lane = threadIdx.x & 31;
   const int64_t w = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (w >= rows * nseg) return;
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const 
                                                           const unsigned long long* __restrict__ maxbits,
                                                           uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
                                                           int32_t* __restrict__ sums, bool vec) {
+  grid_begin();
   __shared__ uint64_t tile[TR][133];
   __shared__ int ssum[TR][P], sE[TR];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -117,7 +119,7 @@ void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, con
   int64_t nseg = (ngroups + per - 1) / per;
   if (kcontig) {
     const int64_t blocks = (rows * nseg + 7) / 8;
-    split_tri_kcontig<T, P><<<static_cast<unsigned>(blocks), 256, 0, st>>>(X, ld, rows, k, kpad, per, nseg, maxbits,
+    launch_after(split_tri_kcontig<T, P>, static_cast<unsigned>(blocks), 256, st, X, ld, rows, k, kpad, per, nseg, maxbits,
                                                                            planes, E, sums, vec);
   } else {
     while (nseg > 65535) {
@@ -131,9 +133,9 @@ void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, con
     const bool small = units * nseg < 2 * static_cast<int64_t>(num_sms);
     const dim3 grid(static_cast<unsigned>(small ? (rows + 7) / 8 : units), static_cast<unsigned>(nseg));
     if (small)
-      split_tri_kstrided<T, P, 8><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+      launch_after(split_tri_kstrided<T, P, 8>, grid, 256, st, X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
     else
-      split_tri_kstrided<T, P, 32><<<grid, 256, 0, st>>>(X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+      launch_after(split_tri_kstrided<T, P, 32>, grid, 256, st, X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
   }
 }
 
