@@ -1,14 +1,17 @@
-"""Benchmark: emulated FP64 GEMM on the INT8 tensor cores of one GB300.
+"""Benchmark: emulated FP64 GEMM on the tensor cores of one GB300.
 
 Workload (one "step"): Scheme I emulated DGEMM C = A @ B, M = N = K = 8192,
 row-major float64, A and B drawn by the paper's test-matrix generator
-(Eq. 19) with phi = 0.5, p = 8 INT8 slices: exponent scan, split into
-interleaved slices, fused INT8 GEMM with the exact shift-reduce epilogue.
+(Eq. 19) with phi = 0.5, p = 8 slices of 8 bits: exponent scan, split into
+digits and digit sums (exact bf16 planes), the exact integer products of the
+digit triangle on the bf16 tensor cores, and their exact combination with one
+rounding (EMU_I_ENGINE=mma: the fused INT8 mma.sync kernel; same result).
 Inputs (512 MiB each) are larger than L2 (129 MB), so no L2 flush is needed.
 
 Printed: one JSON line with the effective FP64 TFLOP/s (2 M N K / t), the
-INT8 tensor rate and its fraction of the measured INT8 peak, the roofline
-of the fused GEMM kernel, an end-to-end number through host buffers, cuBLAS
+rate of the p(p+1)/2 8-bit slice products it stands for and that rate over the
+measured INT8 peak (above 1: the bf16 tensor cores form them from fewer
+products), the roofline of the GEMM kernel, an end-to-end number through host buffers, cuBLAS
 DGEMM on the same GPU at its own accuracy, the error of both against a
 double-double reference on sampled entries, the CPU oracle baseline, and the
 SM clocks seen during the timed region.
@@ -36,7 +39,7 @@ sys.path.insert(0, ROOT)
 
 import synth  # noqa: E402
 
-METRIC = "emulated FP64 TFLOP/s (Scheme I DGEMM on INT8 tensor cores)"
+METRIC = "emulated FP64 TFLOP/s (Scheme I DGEMM, 8-bit slices)"
 UNIT = "TFLOP/s"
 
 
@@ -97,13 +100,14 @@ class ClockSampler:
     def __init__(self, index: int):
         self.index = index
         self.proc = None
+        self.first = 0
         self.lines = []
 
     def __enter__(self):
         try:
             self.proc = subprocess.Popen(
                 ["nvidia-smi", "-i", str(self.index), "--query-gpu=" + self.FIELDS, "--format=csv,noheader,nounits",
-                 "-lms", "200"], stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
+                 "-lms", "20"], stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
             self.thread = threading.Thread(target=self._read, daemon=True)
             self.thread.start()
         except OSError:
@@ -122,10 +126,14 @@ class ClockSampler:
             except subprocess.TimeoutExpired:
                 self.proc.kill()
 
+    def mark(self):
+        """The samples from here on are the ones reported."""
+        self.first = len(self.lines)
+
     def summary(self):
         sm, mx, reasons = [], [], set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
-        for ln in self.lines:
+        for ln in self.lines[self.first:]:
             parts = [x.strip() for x in ln.split(",")]
             if len(parts) < 7:
                 continue
@@ -264,7 +272,7 @@ def scheme_II_leg(emu, h, Ad, Bd, Cd, n, stream, ri, ci, hi, lo, den, cublas_tfl
                             "bf16_peak_tflops": bf16,
                             "err_max_rel_absAB": err,
                             "speedup_vs_cublas_dgemm": 2.0 * n ** 3 / (ms * 1e-3) / 1e12 / cublas_tflops,
-                            "kernel": "gemm_II_tc_kernel (tcgen05 bf16, 128 x 256 tiles)"}
+                            "kernel": "gemm_II_tc_kernel (tcgen05 bf16, CTA pairs on 256 x 256 tiles)"}
     return out
 
 
@@ -370,13 +378,19 @@ def run_ours(args, rank, world, local_rank):
         raise RuntimeError("device status %d after warm-up" % h.status())
 
     # ---------------- timed region: inputs resident in HBM
-    h.trace(True)
-    h.trace_read()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    if dist:
-        dist.barrier()
-    torch.cuda.synchronize()
     with ClockSampler(local_rank) as clk:
+        # a step takes tens of milliseconds: more untimed ones until the sampler runs
+        t_end = time.perf_counter() + 3.0
+        while clk.proc and len(clk.lines) < 2 and time.perf_counter() < t_end:
+            step()
+            torch.cuda.synchronize()
+        h.trace(True)
+        h.trace_read()
+        if dist:
+            dist.barrier()
+        torch.cuda.synchronize()
+        clk.mark()
         e0.record(stream)
         for _ in range(args.steps):
             step()
@@ -485,7 +499,14 @@ def run_ours(args, rank, world, local_rank):
         achieved = int8_ops / (gemm_ms * 1e-3) / 1e12
         peak, peak_src = int8_peak, "measured live: cuBLASLt INT8 GEMM 8192^3 on this GPU"
         ii_tc = args.scheme == "II" and os.environ.get("EMU_II_ENGINE") != "mma"
-        if ii_tc:
+        # Scheme I on the bf16 tensor cores (the default): one product per digit
+        # (but the last), two for the outermost pair, one per other pair i < j, i + j < p
+        i_tc = args.scheme == "I" and os.environ.get("EMU_I_ENGINE") != "mma"
+        if i_tc:
+            nprod = max(p - 1, 1) + (2 if p > 1 else 0) + sum(
+                1 for i in range(p) for j in range(i + 1, p - i) if (i, j) != (0, p - 1))
+            achieved = 2.0 * nprod * n ** 3 / (gemm_ms * 1e-3) / 1e12
+        if ii_tc or i_tc:
             bf16 = measured_peaks().get("bf16_tflops")
             peak = bf16 if bf16 else 1900.0
             peak_src = ("measured dense bf16 peak (MEASURED_PEAKS.json)" if bf16 else
@@ -495,15 +516,18 @@ def run_ours(args, rank, world, local_rank):
             peak = 2.0 * bf16 if bf16 else 2.0 * 1900.0
             peak_src = ("FP8 dense peak = measured bf16 %s x nominal FP8/bf16 ratio 2 (4.5 / 2.25 PFLOP/s)"
                         % ("(MEASURED_PEAKS.json)" if bf16 else "(fallback 1.9 PFLOP/s)"))
-        traffic = (load_traffic("gemm_I", "p%d_n%d" % (p, n)) if args.scheme == "I" else
+        traffic = (load_traffic("gemm_I_tc", "p%d_n%d" % (p, n)) if i_tc else
+                   load_traffic("gemm_I", "p%d_n%d" % (p, n)) if args.scheme == "I" else
                    load_traffic("gemm_f8tc", "p%d_n%d" % (p, n)) if args.scheme == "I_F8" else
                    load_traffic("gemm_II_tc", "nm%d_n%d" % (p, n)) if ii_tc else None)
         kname = ("gemm_II_tc_kernel (tcgen05 bf16 residue GEMM; the CRT kernel is timed apart)" if ii_tc else "gemm_II_kernel (mma.sync INT8)" if args.scheme == "II" else
                  "gemm_f8tc_kernel<%d, OUT_F64> (tcgen05)" % p if args.scheme == "I_F8" else
+                 "gemm_I_tc_kernel (tcgen05 bf16 digit products; the combine kernel is timed apart)" if i_tc else
                  "gemm_I_kernel<%d, OUT_F64> (mma.sync INT8)" % p)
         ops_desc = ("bf16 tensor ops 2 N_m M N K (residue products)" if ii_tc else
                     "INT8 ops 2 N_m M N K" if args.scheme == "II" else
                     "exact E4M3 products p(p+1) M N K (multiply+add = 2)" if args.scheme == "I_F8" else
+                    "bf16 tensor ops 2 x %d M N K (exact products of digits and digit sums)" % nprod if i_tc else
                     "INT8 ops p(p+1) M N K (multiply+add = 2)")
         metric = METRIC if args.scheme == "I" else (
             "emulated FP64 TFLOP/s (Scheme II DGEMM on %s tensor cores)" % ("bf16" if ii_tc else "INT8")
@@ -512,7 +536,7 @@ def run_ours(args, rank, world, local_rank):
                 "warmup": max(args.warmup, 3), "ms_per_step": ms_step, "higher_is_better": True,
                 "scaling": "weak", "vs_baseline": None,
                 "dtype": ("e4m3->fp32 (f64 in/out)" if args.scheme == "I_F8" else
-                          "bf16->fp32 (f64 in/out)" if ii_tc else "int8->int32 (f64 in/out)"),
+                          "bf16->fp32 (f64 in/out)" if ii_tc or i_tc else "int8->int32 (f64 in/out)"),
                 "data": "synthetic",
                 "config": config(args, world),
                 "int8_tops": (int8_ops * args.steps * world / (ms * 1e-3) / 1e12) if not ii_tc else None,
@@ -525,7 +549,7 @@ def run_ours(args, rank, world, local_rank):
                              "traffic": traffic,
                              "ops": ops_desc,
                              "peak_source": peak_src},
-                "phase_ms_per_step": {k2: tr[k2] / args.steps for k2 in ("ms_scan", "ms_split", "ms_gemm")},
+                "phase_ms_per_step": {k2: tr[k2] / args.steps for k2 in ("ms_scan", "ms_split", "ms_gemm", "ms_other")},
                 "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 2 * 8 * n * n,
                         "d2h_bytes_per_step": 8 * n * n},
                 "gpu_launches": tr["kernel_launches"],
@@ -589,8 +613,8 @@ def suite_markdown(paths):
             t = d.get("tflops", d.get("tflops_8mnk"))
             unit = " (8MNK)" if "tflops_8mnk" in d else ""
             o.append(f"| {d['path']} | {d['n']} | {t:.3f}{unit} | {bits(d.get('err'))} |")
-    o.append("\n## Scheme I emulated DGEMM / SGEMM, INT8 slices (mma.sync)\n")
-    o.append("| path | n | phi | p | TFLOP/s | INT8 TOP/s | bits |\n|---|---|---|---|---|---|---|")
+    o.append("\n## Scheme I emulated DGEMM / SGEMM, 8-bit slices\n")
+    o.append("| path | n | phi | p | TFLOP/s | 8-bit slice products, TOP/s | bits |\n|---|---|---|---|---|---|---|")
     for d in rows:
         if d["path"] in ("emu_dgemm_I", "emu_sgemm_I"):
             o.append(f"| {d['path']} | {d['n']} | {d['phi']:g} | {d['p']} | {d['tflops']:.3f} | {d['int8_tops']:.1f} | {bits(d['err'])} |")

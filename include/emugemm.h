@@ -2,7 +2,7 @@
  * emugemm.h -- C ABI of the GB300 (sm_103a) emulated-GEMM library.
  *
  * The library computes C = alpha * A * B + beta * C for FP64, FP32 and
- * complex128 matrices on the INT8 tensor cores, with the two Ozaki schemes
+ * complex128 matrices on low-precision tensor cores, with the two Ozaki schemes
  * of the EmuGEMM paper (Lu, Maeder, Luisier, Ziogas):
  *
  *   Scheme I  (Sec. II-C-1, Eqs. 1-3; fused kernel of Algorithm 1, Sec. III)
@@ -11,7 +11,13 @@
  *     unsigned tails, beta = 8 bits each).  All p(p+1)/2 slice products with
  *     i + j < p are formed exactly in INT32 and combined by the shift-reduce
  *     of Eq. (3).  Here the shift-reduce is exact: the partial sums are
- *     combined as integers and rounded once to binary64.
+ *     combined as integers and rounded once to binary64.  On sm_103a the
+ *     products run by default on the bf16 tensor cores (tcgen05): recentred
+ *     digits and sums of two of them are exact bf16 values, their FP32 sums
+ *     stay exact integers, and the triangle needs one product per pair i < j
+ *     and per digit (24 instead of 36 at p = 8).  The INT8 mma.sync kernel
+ *     gives the same result and serves p > 8 below 2^33 multiply-adds,
+ *     workspaces that only hold its slices, and EMU_I_ENGINE=mma.
  *
  *   Scheme II (Sec. II-C-2, Eqs. 4-8; fused kernel of Sec. IV-A)
  *     A and B are scaled to integers, reduced modulo N pairwise-coprime
@@ -155,7 +161,9 @@ const char *emu_last_cuda_error(void);
 
 /* Bytes of device workspace one call needs (is_complex selects the complex
  * layouts: three residue sets per operand for the Scheme II 3M method, the
- * real embedding plus the slices of the 2K-deep product for Scheme I 4M). */
+ * real embedding plus the slices of the 2K-deep product for Scheme I 4M).
+ * For Scheme I this is what the bf16 engine uses; a smaller workspace that
+ * still holds the INT8 slices makes the call run on the INT8 kernel. */
 emu_status_t emu_workspace_size(emu_scheme_t scheme, int64_t m, int64_t n, int64_t k, int p_or_nm,
                                 int is_complex, size_t *bytes_host);
 
@@ -280,8 +288,8 @@ emu_status_t emu_dgemm_host(emu_handle_t h, emu_layout_t layout, int64_t m, int6
  *    stream capture on that device.  A call in a different context (for
  *    example after cudaDeviceReset re-created the primary context) looks the
  *    address up again, so that call, too, belongs outside a capture.
- *  - Products whose workspace (emu_workspace_size for Scheme I) exceeds
- *    EMU_NOALLOC_SCRATCH_BYTES are rejected with EMU_ERR_UNSUPPORTED
+ *  - Products whose INT8 slices exceed EMU_NOALLOC_SCRATCH_BYTES (m p k + n p k
+ *    bytes and a little more) are rejected with EMU_ERR_UNSUPPORTED
  *    (e.g. m = n = k = 2048 fits for p <= 7).
  *  - All calls share the array and it keeps the last call's contents; each
  *    call clears what must start at zero.  Calls whose work overlaps on the
