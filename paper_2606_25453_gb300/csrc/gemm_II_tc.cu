@@ -211,13 +211,14 @@ __device__ __forceinline__ void pair_acc(CrtPair<L>& a, const CrtPairTables& ct,
 
 // The residue words (four columns each) of one plane set, interleaved by
 // pairs of moduli.  All loads are issued first (independent, predicated).
+template <int MAXP>
 __device__ __forceinline__ void load_pairs(const uint8_t* p, int64_t plane, int nm, uint32_t* t01, uint32_t* t23) {
-  uint32_t w[kMaxModuli];
+  uint32_t w[2 * MAXP];
 #pragma unroll
-  for (int l = 0; l < kMaxModuli; ++l)
+  for (int l = 0; l < 2 * MAXP; ++l)
     w[l] = l < nm ? __ldg(reinterpret_cast<const uint32_t*>(p + static_cast<int64_t>(l) * plane)) : 0u;
 #pragma unroll
-  for (int i = 0; i < kMaxPairs; ++i) {
+  for (int i = 0; i < MAXP; ++i) {
     t01[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5140u);
     t23[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7362u);
   }
@@ -230,19 +231,23 @@ __device__ __forceinline__ void load_pairs(const uint8_t* p, int64_t plane, int 
 // two residues with 16-bit coefficients and L wide multiply-adds, half of what
 // a weight per modulus took.  n = 8192, 16 moduli: 1.08 -> 0.75 ms (the bytes
 // alone take 0.27), 3M 2.80 -> 1.92 ms; 2905 x 1777, 14 moduli: 82 -> 50 us.
+// Loops bounded by the 4 L moduli that L limbs hold, not by 20, need 52
+// registers instead of 110 at L = 2 (3M, 8 moduli, 3001 x 2047: 115 -> 80 us;
+// 16 moduli, n = 8192: 1.92 -> 1.72 ms).
 template <int MODE, int L>
 __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KParamsCRT kp,
                                                      const __grid_constant__ CrtPairTables ct) {
   grid_begin();
   constexpr bool CPLX = MODE == II_Z3M || MODE == II_C3M;
+  constexpr int kP = 2 * L;  // P of L limbs has at most 4 L moduli
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int ncq = (kp.N + kCrtCols - 1) / kCrtCols;
   if (idx >= static_cast<int64_t>(kp.M) * ncq) return;
   const int row = static_cast<int>(idx / ncq), c0 = static_cast<int>(idx % ncq) * kCrtCols;
   const uint8_t* const p = kp.R + static_cast<int64_t>(row) * kp.ldr + c0;
   const int erow = kp.EA[row] + kp.escale;
-  uint32_t a01[kMaxPairs], a23[kMaxPairs];
-  load_pairs(p, kp.plane, kp.nm, a01, a23);
+  uint32_t a01[kP], a23[kP];
+  load_pairs<kP>(p, kp.plane, kp.nm, a01, a23);
   if constexpr (!CPLX) {
 #pragma unroll
     for (int c = 0; c < kCrtCols; ++c) {
@@ -252,7 +257,7 @@ __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KPa
 #pragma unroll
       for (int j = 0; j < L; ++j) acc.s[j] = 0;
 #pragma unroll
-      for (int i = 0; i < kMaxPairs; ++i) {
+      for (int i = 0; i < kP; ++i) {
         if (2 * i >= kp.nm) break;
         pair_acc<L>(acc, ct, i, pair_x(ct.c[i], a01[i], a23[i], c));
       }
@@ -273,9 +278,9 @@ __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KPa
     }
   } else {
     const int64_t set = static_cast<int64_t>(kp.nm) * kp.plane;
-    uint32_t b01[kMaxPairs], b23[kMaxPairs], d01[kMaxPairs], d23[kMaxPairs];
-    load_pairs(p + set, kp.plane, kp.nm, b01, b23);
-    load_pairs(p + 2 * set, kp.plane, kp.nm, d01, d23);
+    uint32_t b01[kP], b23[kP], d01[kP], d23[kP];
+    load_pairs<kP>(p + set, kp.plane, kp.nm, b01, b23);
+    load_pairs<kP>(p + 2 * set, kp.plane, kp.nm, d01, d23);
 #pragma unroll
     for (int c = 0; c < kCrtCols; ++c) {
       const int cidx = c0 + c;
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(256) crt_II_kernel(const __grid_constant__ KPa
 #pragma unroll
       for (int j = 0; j < L; ++j) are.s[j] = aim.s[j] = 0;
 #pragma unroll
-      for (int i = 0; i < kMaxPairs; ++i) {
+      for (int i = 0; i < kP; ++i) {
         if (2 * i >= kp.nm) break;
         // T1 - T2 and T3 - T1 - T2 modulo m m', kept non-negative by a
         // multiple of it: the pair's weight times m m' is a multiple of P
