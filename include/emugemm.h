@@ -148,7 +148,9 @@ emu_status_t emu_get_status(emu_handle_t h, emu_stream_t stream);
  * every library-owned workspace allocation fails with EMU_ERR_ALLOC; with
  * EMU_FAULT=launch the fused GEMM launch of every emu_dgemm / emu_sgemm /
  * emu_zgemm / emu_cgemm call fails with EMU_ERR_CUDA ("unspecified launch
- * failure") after the scan and split were enqueued, and C is not written. */
+ * failure") after the scan and split were enqueued, and C is not written;
+ * with EMU_FAULT=zero, scan, norm or split the call ends the same way at the
+ * first launch of that step. */
 emu_status_t emu_selftest_wait(emu_handle_t h, int64_t limit_cycles, emu_stream_t stream);
 
 /* Human-readable name of a status code (static string). */

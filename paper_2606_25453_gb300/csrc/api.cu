@@ -343,9 +343,10 @@ using namespace emu;
 // ================================================================ handle
 // What was behind this thread's last EMU_ERR_CUDA (emu_last_cuda_error).
 static thread_local const char* g_last_cuda_error = "no error";
-static emu_status_t cuda_err(cudaError_t e) {
+emu_status_t emu::cuda_err(cudaError_t e) {
   if (e == cudaSuccess) return EMU_OK;
   g_last_cuda_error = cudaGetErrorString(e);
+  cudaGetLastError();  // reported here: not left for the thread's next query
   return EMU_ERR_CUDA;
 }
 static emu_status_t tmap_err() {
@@ -354,21 +355,26 @@ static emu_status_t tmap_err() {
 }
 
 namespace emu {
-// EMU_FAULT=alloc / EMU_FAULT=launch: host-side fault injection (read once).
+// EMU_FAULT: host-side fault injection (read once).  alloc: every
+// library-owned workspace allocation fails; launch: the fused GEMM launch of
+// every product, zero, scan, norm or split: every launch of that step before
+// it.  A launch fails as a launch would (cudaErrorLaunchFailure); nothing runs
+// on the device that could fault.
 static int fault_mode() {
   static int v = -1;
   if (v < 0) {
+    static const char* const names[] = {"", "alloc", "launch", "zero", "scan", "norm", "split"};
     const char* e = std::getenv("EMU_FAULT");
-    v = !e ? 0 : std::strcmp(e, "alloc") == 0 ? 1 : std::strcmp(e, "launch") == 0 ? 2 : 0;
+    int x = 0;
+    for (int i = FAULT_ALLOC; e && i <= FAULT_SPLIT; ++i)
+      if (std::strcmp(e, names[i]) == 0) x = i;
+    v = x;
   }
   return v;
 }
-// alloc: every library-owned workspace allocation fails.
-static bool fault_alloc() { return fault_mode() == 1; }
-// launch: the fused GEMM launch of every product fails as a launch would
-// (cudaErrorLaunchFailure, after the scan and split were enqueued); nothing
-// runs on the device that could fault.
-static cudaError_t fault_launch() { return fault_mode() == 2 ? cudaErrorLaunchFailure : cudaSuccess; }
+static bool fault_alloc() { return fault_mode() == FAULT_ALLOC; }
+cudaError_t fault_step(FaultStep step) { return fault_mode() == step ? cudaErrorLaunchFailure : cudaSuccess; }
+static cudaError_t fault_launch() { return fault_step(FAULT_GEMM); }
 
 emu_status_t handle_workspace(emu_handle_s* h, size_t bytes, cudaStream_t st, uint8_t** out) {
   if (bytes == 0) bytes = 256;
@@ -700,6 +706,7 @@ emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double al
   // maxima and digit sums start at zero; in a first pass over A with B one
   // memset and one scan serve both operands
   const bool both = phase == 0;
+  cudaError_t e = cudaSuccess;
   if (phase != 2) {
     trace_begin(h, PH_SCAN, st);
     if (both) {
@@ -707,35 +714,40 @@ emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double al
         sumA = v.sums;
         sumB = v.sums + static_cast<int64_t>(p) * v.M;
       } else {
-        launch_zero(ws, pl.zero_bytes, st);
+        e = launch_zero(ws, pl.zero_bytes, st);
       }
-      if (!v.maxA)
-        launch_scan<T>(A, v.ldA, v.a_kcontig, std::min(rows, v.M), maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1, true,
-                       h->status, st);
+      if (e == cudaSuccess && !v.maxA)
+        e = launch_scan<T>(A, v.ldA, v.a_kcontig, std::min(rows, v.M), maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1,
+                           true, h->status, st);
     } else {
-      cudaMemsetAsync(sumB, 0, sizeof(*sumB) * p * v.N, st);
-      if (!v.maxB) launch_scan_one<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
+      e = cudaMemsetAsync(sumB, 0, sizeof(*sumB) * p * v.N, st);
+      if (e == cudaSuccess && !v.maxB) e = launch_scan_one<T>(B, v.ldB, v.b_kcontig, v.N, k, 1, maxB, h->status, st);
     }
     trace_end(h, PH_SCAN, st, both ? 2 : 1);
+    if (e != cudaSuccess) return cuda_err(e);
     trace_begin(h, PH_SPLIT, st);
-    launch_split_tri<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, planesB, FB, sumB, h->num_sms, st);
+    e = launch_split_tri<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, planesB, FB, sumB, h->num_sms,
+                            st);
     trace_end(h, PH_SPLIT, st, 1);
+    if (e != cudaSuccess) return cuda_err(e);
   }
-  if (phase == 1) return cuda_err(cudaGetLastError());
+  if (phase == 1) return EMU_OK;
   const int np = tri_num_planes(p);
   for (int64_t r0 = 0; r0 < v.M; r0 += rows) {
     const int64_t m = std::min(rows, v.M - r0);
     const T* Ar = A + (v.a_kcontig ? r0 * v.ldA : r0);
     if (!both || r0 > 0) {
       trace_begin(h, PH_SCAN, st);
-      cudaMemsetAsync(sumA, 0, sizeof(*sumA) * p * m, st);
-      if (!v.maxA) launch_scan_one<T>(Ar, v.ldA, v.a_kcontig, m, k, 1, maxA, h->status, st);
+      e = cudaMemsetAsync(sumA, 0, sizeof(*sumA) * p * m, st);
+      if (e == cudaSuccess && !v.maxA) e = launch_scan_one<T>(Ar, v.ldA, v.a_kcontig, m, k, 1, maxA, h->status, st);
       trace_end(h, PH_SCAN, st, 1);
+      if (e != cudaSuccess) return cuda_err(e);
     }
     trace_begin(h, PH_SPLIT, st);
-    launch_split_tri<T>(Ar, v.ldA, v.a_kcontig, m, k, p, v.maxA ? v.maxA + r0 : maxA, planesA, EA, sumA, h->num_sms,
-                        st);
+    e = launch_split_tri<T>(Ar, v.ldA, v.a_kcontig, m, k, p, v.maxA ? v.maxA + r0 : maxA, planesA, EA, sumA,
+                            h->num_sms, st);
     trace_end(h, PH_SPLIT, st, 1);
+    if (e != cudaSuccess) return cuda_err(e);
     GemmTriArgs a{};
     a.L = tri_layout(rows, v.N, k, p);  // the workspace's layout, for fewer rows in the last pass
     a.L.tiles_m = (m + tri_tile_m() - 1) / tri_tile_m();
@@ -763,7 +775,7 @@ emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double al
     a.status = h->status;
     a.num_sms = h->num_sms;
     trace_begin(h, PH_GEMM, st);
-    cudaError_t e = fault_launch();
+    e = fault_launch();
     if (e == cudaSuccess) e = launch_gemm_I_tc(p, out_mode, a, st, 1);
     trace_end(h, PH_GEMM, st, 1);
     if (e != cudaSuccess) return cuda_err(e);
@@ -808,16 +820,21 @@ emu_status_t run_scheme_I(emu_handle_s* h, const View& v, int64_t k, int p, doub
   auto* hatB = reinterpret_cast<int8_t*>(ws + pl.off_hatB);
   const T* A = static_cast<const T*>(v.A);
   const T* B = static_cast<const T*>(v.B);
+  cudaError_t e = cudaSuccess;
   if (!v.maxA) {
     trace_begin(h, PH_SCAN, st);
-    launch_zero(ws + pl.off_maxA, pl.off_maxB + sizeof(*maxB) * v.N - pl.off_maxA, st);
-    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
+    e = launch_zero(ws + pl.off_maxA, pl.off_maxB + sizeof(*maxB) * v.N - pl.off_maxA, st);
+    if (e == cudaSuccess)
+      e = launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, maxA, B, v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
     trace_end(h, PH_SCAN, st, 2);
+    if (e != cudaSuccess) return cuda_err(e);
   }
   trace_begin(h, PH_SPLIT, st);
-  launch_split_I<T>(A, v.ldA, v.a_kcontig, v.M, k, p, v.maxA ? v.maxA : maxA, hatA, EA, st, f8);
-  launch_split_I<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, hatB, FB, st, f8);
+  e = launch_split_I<T>(A, v.ldA, v.a_kcontig, v.M, k, p, v.maxA ? v.maxA : maxA, hatA, EA, st, f8);
+  if (e == cudaSuccess)
+    e = launch_split_I<T>(B, v.ldB, v.b_kcontig, v.N, k, p, v.maxB ? v.maxB : maxB, hatB, FB, st, f8);
   trace_end(h, PH_SPLIT, st, 2);
+  if (e != cudaSuccess) return cuda_err(e);
   return scheme_I_gemm(h, hatA, pl.rows_a, hatB, pl.rows_b, pl.cols, v.M, v.N, k, p, EA, FB, alpha, beta, C, ldc,
                        out_mode, partials, st, f8);
 }
@@ -902,30 +919,35 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   const unsigned long long* mA = v.maxA ? v.maxA : maxA;
   const unsigned long long* mB = v.maxB ? v.maxB : maxB;
   const bool both = do_a && do_b;
+  cudaError_t e = cudaSuccess;
   if (!v.maxA) {
     if (both) {  // maxima, and the sums of squares behind them, in one launch
       const size_t end = norm ? pl.off_accB + 2 * sizeof(*accB) * v.N : pl.off_maxB + sizeof(*maxB) * v.N;
-      launch_zero(ws + pl.off_maxA, end - pl.off_maxA, st);
+      e = launch_zero(ws + pl.off_maxA, end - pl.off_maxA, st);
     }
-    launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, do_a ? maxA : nullptr, B, v.ldB, v.b_kcontig, v.N,
-                   do_b ? maxB : nullptr, k, cw, both, h->status, st);
+    if (e == cudaSuccess)
+      e = launch_scan<T>(A, v.ldA, v.a_kcontig, v.M, do_a ? maxA : nullptr, B, v.ldB, v.b_kcontig, v.N,
+                         do_b ? maxB : nullptr, k, cw, both, h->status, st);
   }
   if (norm) {
     if (v.maxA || !both) {
-      if (do_a) launch_zero(accA, 2 * sizeof(*accA) * v.M, st);
-      if (do_b) launch_zero(accB, 2 * sizeof(*accB) * v.N, st);
+      if (e == cudaSuccess && do_a) e = launch_zero(accA, 2 * sizeof(*accA) * v.M, st);
+      if (e == cudaSuccess && do_b) e = launch_zero(accB, 2 * sizeof(*accB) * v.N, st);
     }
-    launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, mA, do_a ? accA : nullptr, B, v.ldB, v.b_kcontig, v.N, mB,
-                   do_b ? accB : nullptr, k, cw, st);
+    if (e == cudaSuccess)
+      e = launch_norm<T>(A, v.ldA, v.a_kcontig, v.M, mA, do_a ? accA : nullptr, B, v.ldB, v.b_kcontig, v.N, mB,
+                         do_b ? accB : nullptr, k, cw, st);
   }
   trace_end(h, PH_SCAN, st, norm ? 3 : do_a + do_b);
+  if (e != cudaSuccess) return cuda_err(e);
   trace_begin(h, PH_SPLIT, st);
   if (do_a)
-    launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, mA, resA, EA, st, norm ? accA : nullptr, tc);
-  if (do_b)
-    launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, mB, resB, FB, st, norm ? accB : nullptr, tc);
+    e = launch_split_II<T>(A, v.ldA, v.a_kcontig, v.M, k, nm, bA, cw, mt, mA, resA, EA, st, norm ? accA : nullptr, tc);
+  if (e == cudaSuccess && do_b)
+    e = launch_split_II<T>(B, v.ldB, v.b_kcontig, v.N, k, nm, bB, cw, mt, mB, resB, FB, st, norm ? accB : nullptr, tc);
   trace_end(h, PH_SPLIT, st, do_a + do_b);
-  if (phase == 1) return cuda_err(cudaGetLastError());
+  if (e != cudaSuccess) return cuda_err(e);
+  if (phase == 1) return EMU_OK;
   CUtensorMap ta, tb;
   // tcgen05: the bf16 planes as bytes, 128-byte (64-element) boxes of 128
   // rows (A) and 256 / cluster rows (B: a CTA pair loads half of each
@@ -963,14 +985,14 @@ emu_status_t run_scheme_II(emu_handle_s* h, const View& v, int64_t k, int nm, in
   a.scratch = ws + pl.off_scratch;
   if (!tc) {
     trace_begin(h, PH_GEMM, st);
-    cudaError_t e = fault_launch();
+    e = fault_launch();
     if (e == cudaSuccess) e = launch_gemm_II(out_mode, a, mt, tabs.crt, st);
     trace_end(h, PH_GEMM, st, 1);
     return cuda_err(e);
   }
   // the residue GEMM is the traced GEMM phase, the CRT kernel "other"
   trace_begin(h, PH_GEMM, st);
-  cudaError_t e = fault_launch();
+  e = fault_launch();
   if (e == cudaSuccess) e = launch_gemm_II_tc(out_mode, a, mt, tabs.pair, st, 1);
   trace_end(h, PH_GEMM, st, 1);
   if (e != cudaSuccess) return cuda_err(e);
@@ -1170,9 +1192,9 @@ static emu_status_t split_slices(emu_handle_t h, emu_layout_t layout, int operan
   emu_status_t s = handle_workspace(h, 8 * static_cast<size_t>(rows > 0 ? rows : 1), st, &ws);
   if (s != EMU_OK) return s;
   auto* mx = reinterpret_cast<unsigned long long*>(ws);
-  launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
-  launch_split_I<double>(X, ldx, kcontig, rows, k, p, mx, hat, E, st, f8);
-  return cuda_err(cudaGetLastError());
+  cudaError_t e = launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
+  if (e == cudaSuccess) e = launch_split_I<double>(X, ldx, kcontig, rows, k, p, mx, hat, E, st, f8);
+  return cuda_err(e);
 }
 
 extern "C" {
@@ -1193,9 +1215,9 @@ emu_status_t emu_split_II(emu_handle_t h, emu_layout_t layout, int operand, int6
   auto* mx = reinterpret_cast<unsigned long long*>(ws);
   const ModTables& mt = method_tables(nm).mod;
   int b = host_scale_bits_II(nm, k_total, 0);
-  launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
-  launch_split_II<double>(X, ldx, kcontig, rows, k, nm, b, 1, mt, mx, res, E, st);
-  return cuda_err(cudaGetLastError());
+  cudaError_t e = launch_scan_one<double>(X, ldx, kcontig, rows, k, 1, mx, h->status, st);
+  if (e == cudaSuccess) e = launch_split_II<double>(X, ldx, kcontig, rows, k, nm, b, 1, mt, mx, res, E, st);
+  return cuda_err(e);
 }
 
 emu_status_t emu_partials_I(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n, int64_t k,

@@ -93,6 +93,9 @@ template <typename T>
 emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double alpha, double beta, void* C,
                      int64_t ldc, int out_mode, cudaStream_t st, uint8_t* ws, int64_t rows, int phase);
 
+// EMU_OK, or EMU_ERR_CUDA with the error's text for emu_last_cuda_error (api.cu).
+emu_status_t cuda_err(cudaError_t e);
+
 // The fused Scheme I GEMM on operands already split (api.cu).
 emu_status_t scheme_I_gemm(emu_handle_s* h, const int8_t* hatA, int64_t rows_a, const int8_t* hatB, int64_t rows_b,
                            int64_t cols, int64_t M, int64_t N, int64_t k, int p, const int32_t* EA,

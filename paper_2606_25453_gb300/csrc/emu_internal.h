@@ -93,36 +93,43 @@ struct MethodTables {
 };
 const MethodTables& method_tables(int nm);
 
+// Host-side fault injection (EMU_FAULT, api.cu): the error with which a
+// launch of this step fails in place of running, normally none.
+enum FaultStep : int { FAULT_ALLOC = 1, FAULT_GEMM, FAULT_ZERO, FAULT_SCAN, FAULT_NORM, FAULT_SPLIT };
+cudaError_t fault_step(FaultStep step);
+
 // ---------------------------------------------------------------- launchers
+// Each returns its own launch error: launch_after reports it there, and the
+// kernels after it would run on what an earlier call left in the workspace.
 // Zero `bytes` (rounded up to 16) at the 16-byte aligned p.
-void launch_zero(void* p, size_t bytes, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
 // The largest |x| (IEEE bits) of every row of A (M vectors) and column of B
 // (N), in one launch; a null maxA or maxB leaves that operand out.  zeroed:
 // the outputs are zero already.
 template <typename T>
-void launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
+[[nodiscard]] cudaError_t launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
                  int64_t ldB, bool b_kcontig, int64_t N, unsigned long long* maxB, int64_t k, int cw, bool zeroed,
                  int* status, cudaStream_t st);
 // One operand, zeroed here.
 template <typename T>
-inline void launch_scan_one(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
+[[nodiscard]] inline cudaError_t launch_scan_one(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int cw,
                             unsigned long long* maxbits, int* status, cudaStream_t st) {
-  launch_scan<T>(X, ld, kcontig, rows, maxbits, static_cast<const T*>(nullptr), 1, false, 0, nullptr, k, cw, false,
-                 status, st);
+  return launch_scan<T>(X, ld, kcontig, rows, maxbits, static_cast<const T*>(nullptr), 1, false, 0, nullptr, k, cw,
+                        false, status, st);
 }
 template <typename T>
-void launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+[[nodiscard]] cudaError_t launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
                     const unsigned long long* maxbits, int8_t* hat, int32_t* E, cudaStream_t st,
                     bool f8 = false);
 template <typename T>
-void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
+[[nodiscard]] cudaError_t launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
                      int cw, const ModTables& tabs, const unsigned long long* maxbits, int8_t* res,
                      int32_t* E, cudaStream_t st, const unsigned long long* acc = nullptr, bool bf16 = false);
 // Norm-based Scheme II scaling: the sums of squares of both operands' vectors
 // in one launch, exact in any order (maxima from launch_scan; acc: two words
 // per vector, zeroed; null: that operand is left out).
 template <typename T>
-void launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
+[[nodiscard]] cudaError_t launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
                  unsigned long long* accA, const T* B, int64_t ldB, bool b_kcontig, int64_t N,
                  const unsigned long long* maxB, unsigned long long* accB, int64_t k, int cw, cudaStream_t st);
 void host_norm_halves_II(int nm, int* hA, int* hB);
@@ -189,7 +196,7 @@ void preload_tri();
 void preload_split_tri();
 cudaError_t launch_gemm_I_tc(int p, int out_mode, const GemmTriArgs& a, cudaStream_t st, int part);
 template <typename T>
-void launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+[[nodiscard]] cudaError_t launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
                       const unsigned long long* maxbits, uint16_t* planes, int32_t* E, int32_t* sums, int num_sms,
                       cudaStream_t st);
 

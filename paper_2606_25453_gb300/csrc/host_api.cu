@@ -200,13 +200,16 @@ emu_status_t host_gemm(emu_handle_s* h, HostIO* io, const View& v, int64_t k, do
     auto* hatA = reinterpret_cast<int8_t*>(ws + pl.off_hatA);
     auto* hatB = reinterpret_cast<int8_t*>(ws + pl.off_hatB);
     if (cudaStreamWaitEvent(st, io->ev_b, 0) != cudaSuccess) return EMU_ERR_CUDA;
-    launch_scan_one<double>(dB, N, false, N, k, 1, maxB, h->status, st);
-    launch_split_I<double>(dB, N, false, N, k, p, maxB, hatB, FB, st, f8);
+    cudaError_t e = launch_scan_one<double>(dB, N, false, N, k, 1, maxB, h->status, st);
+    if (e == cudaSuccess) e = launch_split_I<double>(dB, N, false, N, k, p, maxB, hatB, FB, st, f8);
+    if (e != cudaSuccess) return cuda_err(e);
     for (int c = 0; c < nch; ++c) {
       const int64_t r0 = c * R, rows = std::min(R, M - r0);
       if (cudaStreamWaitEvent(st, io->ev_a[c], 0) != cudaSuccess) return EMU_ERR_CUDA;
-      launch_scan_one<double>(dA + r0 * k, k, true, rows, k, 1, maxA + r0, h->status, st);
-      launch_split_I<double>(dA + r0 * k, k, true, rows, k, p, maxA + r0, hatA + r0 * pl.cols, EA + r0, st, f8);
+      e = launch_scan_one<double>(dA + r0 * k, k, true, rows, k, 1, maxA + r0, h->status, st);
+      if (e == cudaSuccess)
+        e = launch_split_I<double>(dA + r0 * k, k, true, rows, k, p, maxA + r0, hatA + r0 * pl.cols, EA + r0, st, f8);
+      if (e != cudaSuccess) return cuda_err(e);
       s = scheme_I_gemm(h, hatA + r0 * pl.cols, split_rows(rows), hatB, pl.rows_b, pl.cols, rows, N, k, p, EA + r0,
                         FB, alpha, beta, dC + r0 * N, N, OUT_F64, nullptr, st, f8);
       if (s != EMU_OK) return s;

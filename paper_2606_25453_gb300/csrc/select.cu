@@ -719,9 +719,11 @@ emu_status_t auto_impl(emu_handle_t h, emu_layout_t layout, int64_t m, int64_t n
   if (s != EMU_OK) return s;
   if (cudaEventRecord(ss->ev_decide, st) != cudaSuccess) return EMU_ERR_CUDA;
   trace_begin(h, PH_SCAN, st);
-  launch_scan<double>(static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, maxA,
-                      static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
+  const cudaError_t es =
+      launch_scan<double>(static_cast<const double*>(v.A), v.ldA, v.a_kcontig, v.M, maxA,
+                          static_cast<const double*>(v.B), v.ldB, v.b_kcontig, v.N, maxB, k, 1, true, h->status, st);
   trace_end(h, PH_SCAN, st, 2);
+  if (es != cudaSuccess) return cuda_err(es);
   // the probe's side stream starts after the caller's earlier work
   if (probe > 0 && (cudaEventRecord(ss->ev_fork, st) != cudaSuccess ||
                     cudaStreamWaitEvent(ss->side, ss->ev_fork, 0) != cudaSuccess))

@@ -692,9 +692,11 @@ __global__ void zero_kernel(uint4* p, int64_t n) {
   if (i < n) p[i] = make_uint4(0, 0, 0, 0);
 }
 
-void launch_zero(void* p, size_t bytes, cudaStream_t st) {
+cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st) {
+  if (const cudaError_t e = fault_step(FAULT_ZERO); e != cudaSuccess) return e;
   const int64_t n = static_cast<int64_t>((bytes + 15) / 16);
-  if (n > 0) launch_after(zero_kernel, static_cast<unsigned>((n + 255) / 256), 256, st, static_cast<uint4*>(p), n);
+  if (n == 0) return cudaSuccess;
+  return launch_after(zero_kernel, static_cast<unsigned>((n + 255) / 256), 256, st, static_cast<uint4*>(p), n);
 }
 
 template <typename T>
@@ -712,29 +714,31 @@ static ScanOperand<T> scan_operand(const T* X, int64_t ld, bool kcontig, int64_t
 }
 
 template <typename T>
-void launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
+cudaError_t launch_scan(const T* A, int64_t ldA, bool a_kcontig, int64_t M, unsigned long long* maxA, const T* B,
                  int64_t ldB, bool b_kcontig, int64_t N, unsigned long long* maxB, int64_t k, int cw, bool zeroed,
                  int* status, cudaStream_t st) {
+  cudaError_t e = fault_step(FAULT_SCAN);
   if (!zeroed) {
-    if (maxA) cudaMemsetAsync(maxA, 0, sizeof(*maxA) * M, st);
-    if (maxB) cudaMemsetAsync(maxB, 0, sizeof(*maxB) * N, st);
+    if (e == cudaSuccess && maxA) e = cudaMemsetAsync(maxA, 0, sizeof(*maxA) * M, st);
+    if (e == cudaSuccess && maxB) e = cudaMemsetAsync(maxB, 0, sizeof(*maxB) * N, st);
   }
+  if (e != cudaSuccess) return e;
   const ScanOperand<T> a = scan_operand(A, ldA, a_kcontig, maxA ? M : 0, k, cw, maxA);
   const ScanOperand<T> b = scan_operand(B, ldB, b_kcontig, maxB ? N : 0, k, cw, maxB);
-  if (a.blocks + b.blocks == 0) return;
-  launch_after(scan_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b, status);
+  if (a.blocks + b.blocks == 0) return cudaSuccess;
+  return launch_after(scan_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b, status);
 }
-template void launch_scan<double>(const double*, int64_t, bool, int64_t, unsigned long long*, const double*, int64_t,
+template cudaError_t launch_scan<double>(const double*, int64_t, bool, int64_t, unsigned long long*, const double*, int64_t,
                                   bool, int64_t, unsigned long long*, int64_t, int, bool, int*, cudaStream_t);
-template void launch_scan<float>(const float*, int64_t, bool, int64_t, unsigned long long*, const float*, int64_t,
+template cudaError_t launch_scan<float>(const float*, int64_t, bool, int64_t, unsigned long long*, const float*, int64_t,
                                  bool, int64_t, unsigned long long*, int64_t, int, bool, int*, cudaStream_t);
 
 template <typename T, int P, bool F8>
-static void launch_split_I_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k,
+static cudaError_t launch_split_I_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k,
                              const unsigned long long* maxbits, int8_t* hat, int32_t* E,
                              cudaStream_t st) {
   int64_t rows_pad = split_rows(rows), nchunks = split_cols_I(k, 1) / 32;
-  if (rows_pad == 0 || nchunks == 0) return;
+  if (rows_pad == 0 || nchunks == 0) return cudaSuccess;
   if (kcontig) {
     int64_t warps = rows_pad * ((nchunks + 3) / 4);
     int64_t blocks = (warps + 7) / 8;
@@ -747,37 +751,37 @@ static void launch_split_I_p(const T* X, int64_t ld, bool kcontig, int64_t rows,
     split_I_kstrided<T, P, F8><<<grid, 256, 0, st>>>(X, ld, rows, k, rows_pad, nchunks, maxbits, hat, E,
                                                      vec16_ok(X, ld));
   }
+  return cudaGetLastError();
 }
 
 template <typename T>
-void launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+cudaError_t launch_split_I(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
                     const unsigned long long* maxbits, int8_t* hat, int32_t* E, cudaStream_t st, bool f8) {
+  if (const cudaError_t e = fault_step(FAULT_SPLIT); e != cudaSuccess) return e;
   switch (p) {
 #define EMU_CASE(PP)                                                                         \
   case PP:                                                                                   \
-    if (f8)                                                                                  \
-      launch_split_I_p<T, PP, true>(X, ld, kcontig, rows, k, maxbits, hat, E, st);          \
-    else                                                                                     \
-      launch_split_I_p<T, PP, false>(X, ld, kcontig, rows, k, maxbits, hat, E, st);         \
-    break;
+    return f8 ? launch_split_I_p<T, PP, true>(X, ld, kcontig, rows, k, maxbits, hat, E, st)  \
+              : launch_split_I_p<T, PP, false>(X, ld, kcontig, rows, k, maxbits, hat, E, st);
     EMU_CASE(1) EMU_CASE(2) EMU_CASE(3) EMU_CASE(4) EMU_CASE(5) EMU_CASE(6)
     EMU_CASE(7) EMU_CASE(8) EMU_CASE(9) EMU_CASE(10) EMU_CASE(11) EMU_CASE(12)
 #undef EMU_CASE
     default:
-      break;
+      return cudaErrorInvalidValue;
   }
 }
-template void launch_split_I<double>(const double*, int64_t, bool, int64_t, int64_t, int,
+template cudaError_t launch_split_I<double>(const double*, int64_t, bool, int64_t, int64_t, int,
                                      const unsigned long long*, int8_t*, int32_t*, cudaStream_t, bool);
-template void launch_split_I<float>(const float*, int64_t, bool, int64_t, int64_t, int,
+template cudaError_t launch_split_I<float>(const float*, int64_t, bool, int64_t, int64_t, int,
                                     const unsigned long long*, int8_t*, int32_t*, cudaStream_t, bool);
 
 template <typename T>
-void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
+cudaError_t launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int nm, int b,
                      int cw, const ModTables& tabs, const unsigned long long* maxbits, int8_t* res,
                      int32_t* E, cudaStream_t st, const unsigned long long* acc, bool bf16) {
   const int64_t rows_pad = split_rows(rows), kpad = split_cols_II(k);
-  if (rows_pad == 0 || kpad == 0) return;
+  if (rows_pad == 0 || kpad == 0) return cudaSuccess;
+  if (const cudaError_t e = fault_step(FAULT_SPLIT); e != cudaSuccess) return e;
   // 14-bit digits that hold |a'| < 2^b (bf16 planes; the INT8 form has its own)
   const int nd = b <= 28 ? 2 : b <= 56 ? 4 : 6;
   const bool vec = cw == 1 && vec16_ok(X, ld);
@@ -790,10 +794,7 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
   if (kcontig) {
     const int64_t warps = rows_pad * (kpad / 128);
     const unsigned blocks = static_cast<unsigned>((warps + 7) / 8);
-    if (cw == 2)
-      EMU_SPLIT_II(split_II_kcontig, blocks, 2);
-    else
-      EMU_SPLIT_II(split_II_kcontig, blocks, 1);
+    return cw == 2 ? EMU_SPLIT_II(split_II_kcontig, blocks, 2) : EMU_SPLIT_II(split_II_kcontig, blocks, 1);
   } else {
     // Eight vectors per block while more would leave SMs without a block: a
     // warp then packs one vector instead of two or four in turn.  14 moduli,
@@ -805,14 +806,11 @@ void launch_split_II(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
 #define EMU_STRIDED(CW, ND, SMALL) launch_after(split_II_kstrided<T, CW, true, ND, SMALL>, grid, 256, st, EMU_SPLIT_II_ARGS)
 #define EMU_STRIDED_ND(CW, SMALL) \
   (nd == 2 ? EMU_STRIDED(CW, 2, SMALL) : nd == 4 ? EMU_STRIDED(CW, 4, SMALL) : EMU_STRIDED(CW, 6, SMALL))
-    if (!bf16 && cw == 2)
-      launch_after(split_II_kstrided<T, 2, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS);
-    else if (!bf16)
-      launch_after(split_II_kstrided<T, 1, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS);
-    else if (cw == 2)
-      small ? EMU_STRIDED_ND(2, true) : EMU_STRIDED_ND(2, false);
-    else
-      small ? EMU_STRIDED_ND(1, true) : EMU_STRIDED_ND(1, false);
+    if (!bf16)
+      return cw == 2 ? launch_after(split_II_kstrided<T, 2, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS)
+                     : launch_after(split_II_kstrided<T, 1, false, 6, false>, grid, 256, st, EMU_SPLIT_II_ARGS);
+    if (cw == 2) return small ? EMU_STRIDED_ND(2, true) : EMU_STRIDED_ND(2, false);
+    return small ? EMU_STRIDED_ND(1, true) : EMU_STRIDED_ND(1, false);
 #undef EMU_STRIDED_ND
 #undef EMU_STRIDED
   }
@@ -833,25 +831,26 @@ static NormOperand<T> norm_operand(const T* X, int64_t ld, bool kcontig, int64_t
 }
 
 template <typename T>
-void launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
+cudaError_t launch_norm(const T* A, int64_t ldA, bool a_kcontig, int64_t M, const unsigned long long* maxA,
                  unsigned long long* accA, const T* B, int64_t ldB, bool b_kcontig, int64_t N,
                  const unsigned long long* maxB, unsigned long long* accB, int64_t k, int cw, cudaStream_t st) {
+  if (const cudaError_t e = fault_step(FAULT_NORM); e != cudaSuccess) return e;
   const NormOperand<T> a = norm_operand(A, ldA, a_kcontig, accA ? M : 0, k, cw, maxA, accA);
   const NormOperand<T> b = norm_operand(B, ldB, b_kcontig, accB ? N : 0, k, cw, maxB, accB);
-  if (a.blocks + b.blocks == 0) return;
-  launch_after(norm_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b);
+  if (a.blocks + b.blocks == 0) return cudaSuccess;
+  return launch_after(norm_kernel<T>, static_cast<unsigned>(a.blocks + b.blocks), 256, st, a, b);
 }
-template void launch_norm<double>(const double*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
+template cudaError_t launch_norm<double>(const double*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
                                   const double*, int64_t, bool, int64_t, const unsigned long long*,
                                   unsigned long long*, int64_t, int, cudaStream_t);
-template void launch_norm<float>(const float*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
+template cudaError_t launch_norm<float>(const float*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
                                  const float*, int64_t, bool, int64_t, const unsigned long long*, unsigned long long*,
                                  int64_t, int, cudaStream_t);
 
-template void launch_split_II<double>(const double*, int64_t, bool, int64_t, int64_t, int, int, int,
+template cudaError_t launch_split_II<double>(const double*, int64_t, bool, int64_t, int64_t, int, int, int,
                                       const ModTables&, const unsigned long long*, int8_t*, int32_t*,
                                       cudaStream_t, const unsigned long long*, bool);
-template void launch_split_II<float>(const float*, int64_t, bool, int64_t, int64_t, int, int, int,
+template cudaError_t launch_split_II<float>(const float*, int64_t, bool, int64_t, int64_t, int, int, int,
                                      const ModTables&, const unsigned long long*, int8_t*, int32_t*,
                                      cudaStream_t, const unsigned long long*, bool);
 

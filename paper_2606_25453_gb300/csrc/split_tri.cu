@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const 
 }
 
 template <typename T, int P>
-void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, const unsigned long long* maxbits,
+cudaError_t launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, const unsigned long long* maxbits,
               uint16_t* planes, int32_t* E, int32_t* sums, int num_sms, cudaStream_t st) {
   const int64_t kpad = (k + 63) / 64 * 64, ngroups = (kpad + 127) / 128;
   const bool vec = vec16_ok(X, ld);
@@ -119,8 +119,8 @@ void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, con
   int64_t nseg = (ngroups + per - 1) / per;
   if (kcontig) {
     const int64_t blocks = (rows * nseg + 7) / 8;
-    launch_after(split_tri_kcontig<T, P>, static_cast<unsigned>(blocks), 256, st, X, ld, rows, k, kpad, per, nseg, maxbits,
-                                                                           planes, E, sums, vec);
+    return launch_after(split_tri_kcontig<T, P>, static_cast<unsigned>(blocks), 256, st, X, ld, rows, k, kpad, per, nseg,
+                        maxbits, planes, E, sums, vec);
   } else {
     while (nseg > 65535) {
       per *= 2;
@@ -132,10 +132,8 @@ void launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, con
     // 1024 94.4 -> 92.4; with enough blocks the shorter rows only cost.
     const bool small = units * nseg < 2 * static_cast<int64_t>(num_sms);
     const dim3 grid(static_cast<unsigned>(small ? (rows + 7) / 8 : units), static_cast<unsigned>(nseg));
-    if (small)
-      launch_after(split_tri_kstrided<T, P, 8>, grid, 256, st, X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
-    else
-      launch_after(split_tri_kstrided<T, P, 32>, grid, 256, st, X, ld, rows, k, kpad, per, maxbits, planes, E, sums, vec);
+    return launch_after(small ? split_tri_kstrided<T, P, 8> : split_tri_kstrided<T, P, 32>, grid, 256, st, X, ld, rows, k,
+                        kpad, per, maxbits, planes, E, sums, vec);
   }
 }
 
@@ -153,25 +151,25 @@ void preload_p() {
 void preload_split_tri() { preload_p<1>(); }
 
 template <typename T>
-void launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
+cudaError_t launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,
                       const unsigned long long* maxbits, uint16_t* planes, int32_t* E, int32_t* sums, int num_sms,
                       cudaStream_t st) {
-  if (rows == 0 || k == 0) return;
+  if (rows == 0 || k == 0) return cudaSuccess;
+  if (const cudaError_t e = fault_step(FAULT_SPLIT); e != cudaSuccess) return e;
   switch (p) {
-#define EMU_CASE(PP)                                                                        \
-  case PP:                                                                                  \
-    launch_p<T, PP>(X, ld, kcontig, rows, k, maxbits, planes, E, sums, num_sms, st);        \
-    break;
+#define EMU_CASE(PP) \
+  case PP:           \
+    return launch_p<T, PP>(X, ld, kcontig, rows, k, maxbits, planes, E, sums, num_sms, st);
     EMU_CASE(1) EMU_CASE(2) EMU_CASE(3) EMU_CASE(4) EMU_CASE(5) EMU_CASE(6)
     EMU_CASE(7) EMU_CASE(8) EMU_CASE(9) EMU_CASE(10) EMU_CASE(11) EMU_CASE(12)
 #undef EMU_CASE
     default:
-      break;
+      return cudaErrorInvalidValue;
   }
 }
-template void launch_split_tri<double>(const double*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
+template cudaError_t launch_split_tri<double>(const double*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
                                        uint16_t*, int32_t*, int32_t*, int, cudaStream_t);
-template void launch_split_tri<float>(const float*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
+template cudaError_t launch_split_tri<float>(const float*, int64_t, bool, int64_t, int64_t, int, const unsigned long long*,
                                       uint16_t*, int32_t*, int32_t*, int, cudaStream_t);
 
 }  // namespace emu

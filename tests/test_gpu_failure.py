@@ -2,7 +2,8 @@
 made to run out reports EMU_ERR_TIMEOUT through the status word and leaves
 the context usable; host-side fault injection: EMU_FAULT=alloc turns
 workspace allocation into EMU_ERR_ALLOC while a caller-owned workspace still
-works, and EMU_FAULT=launch makes every fused GEMM launch fail on the host
+works, EMU_FAULT=launch makes every fused GEMM launch fail on the host, and
+EMU_FAULT=zero, scan, norm or split every launch of that step before it
 (EMU_ERR_CUDA, C untouched, context intact)."""
 import os
 import subprocess
@@ -100,3 +101,79 @@ def test_launch_fault_injection():
     assert "unspecified launch failure" in r.stdout
     assert "Z code 4" in r.stdout
     assert "status 0 ctx 64.0" in r.stdout
+
+
+CHILD_STEP = r"""
+import sys, torch
+sys.path.insert(0, %r)
+import paper_2606_25453_gb300 as emu
+h = emu.Handle(0)
+A = torch.ones((64, 64), dtype=torch.float64, device="cuda")
+At = A.t()
+
+def case(name, fn, C):
+    try:
+        fn(C)
+        code = 0
+    except emu.EmuError as e:
+        code = e.code
+    torch.cuda.synchronize()
+    print(name, "code", code, "untouched", bool((C == 7.0).all()), flush=True)
+
+def full(dtype=torch.float64, **kw):
+    return torch.full((64, 64), 7.0, dtype=dtype, **(kw or {"device": "cuda"}))
+
+for scheme, p in (("I", 4), ("I", 12), ("I_F8", 8), ("II", 10), ("II_NORM", 10)):
+    case("d_%%s_%%d" %% (scheme, p), lambda C: emu.dgemm(A, A, C, scheme=scheme, p=p, handle=h), full())
+    case("dcol_%%s_%%d" %% (scheme, p), lambda C: emu.dgemm(At, At, C.t(), scheme=scheme, p=p, handle=h), full())
+    Z = A.to(torch.complex128)
+    case("z_%%s_%%d" %% (scheme, p), lambda C: emu.zgemm(Z, Z, C, nm=p, p=p, scheme=scheme, handle=h), full(torch.complex128))
+    F = A.float()
+    case("s_%%s_%%d" %% (scheme, p), lambda C: emu.sgemm(F, F, C, scheme=scheme, p=p, handle=h), full(torch.float32))
+    H = A.cpu().pin_memory()
+    case("host_%%s_%%d" %% (scheme, p), lambda C: emu.dgemm_host(H, H, C, scheme=scheme, p=p, handle=h),
+         full(pin_memory=True))
+S = torch.cuda.current_stream().cuda_stream
+case("noalloc_I", lambda C: emu.check(emu.emu_dgemm_noalloc(0, 64, 64, 64, 1.0, A.data_ptr(), 64, A.data_ptr(), 64, 0.0,
+                                                            C.data_ptr(), 64, 4, None, S)), full())
+for scheme in ("I", "II"):
+    case("auto_" + scheme, lambda C: emu.dgemm_auto(A, A, 1e-10, handle=h, scheme=scheme, C=C), full())
+E = torch.zeros(64, dtype=torch.int32, device="cuda")
+X = torch.empty(1 << 16, dtype=torch.int8, device="cuda")
+for name, fn in (("I", lambda: emu.emu_split_I(h.h, 0, 0, 64, 64, A.data_ptr(), 64, 4, X.data_ptr(), E.data_ptr(), S)),
+                 ("F8", lambda: emu.emu_split_F8(h.h, 0, 0, 64, 64, A.data_ptr(), 64, 4, X.data_ptr(), E.data_ptr(), S)),
+                 ("II", lambda: emu.emu_split_II(h.h, 0, 0, 64, 64, 64, A.data_ptr(), 64, 4, X.data_ptr(), E.data_ptr(), S))):
+    print("split_" + name, "code", fn(), flush=True)
+print("status", h.status(), "ctx", float((A @ A)[0, 0]))
+"""
+
+
+@pytest.mark.parametrize("engine", ["", "mma"])
+@pytest.mark.parametrize("step", ["zero", "scan", "norm", "split"])
+def test_step_fault_injection(step, engine):
+    # a step whose launch fails must end the call with EMU_ERR_CUDA: the
+    # kernels after it would run on what an earlier call left in the workspace
+    env = dict(os.environ, EMU_FAULT=step)
+    if engine:
+        env.update(EMU_I_ENGINE=engine, EMU_II_ENGINE=engine, EMU_F8_ENGINE=engine)
+    r = subprocess.run([sys.executable, "-c", CHILD_STEP % ROOT], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    lines = [x.split() for x in r.stdout.splitlines()]
+    assert ["status", "0", "ctx", "64.0"] in lines, r.stdout
+    seen = 0
+    for x in lines:
+        if x[1] != "code":
+            continue
+        # who runs the step at all: norm scaling alone has sums of squares; the
+        # chunks of a product in host memory and the lone splits start with a
+        # memset, and the selector's own kernel zeroes for Scheme I
+        has = {"norm": "NORM" in x[0] or x[0] == "auto_II",
+               "zero": not (x[0].startswith(("split", "host")) or x[0] == "auto_I") or "NORM" in x[0],
+               "scan": True, "split": True}[step]
+        if x[0].startswith("host_II") and engine == "mma":
+            has = has or step == "zero"  # the INT8 engine takes the whole product
+        assert x[2] == ("4" if has else "0"), (step, x)
+        if has and not x[0].startswith("split"):
+            assert x[4] == "True", (step, x)
+        seen += has
+    assert seen >= 5
