@@ -145,7 +145,8 @@ emu_status_t emu_get_status(emu_handle_t h, emu_stream_t stream);
  * status word and returns, leaving the context usable.  emu_get_status then
  * reports EMU_ERR_TIMEOUT.  (The library's own waits give up after ~1 s.)
  * Host-side fault injection: with the environment variable EMU_FAULT=alloc
- * every library-owned workspace allocation fails with EMU_ERR_ALLOC; with
+ * every library-owned workspace allocation fails with EMU_ERR_ALLOC
+ * (EMU_FAULT=alloc:N: every one of more than N bytes); with
  * EMU_FAULT=launch the fused GEMM launch of every emu_dgemm / emu_sgemm /
  * emu_zgemm / emu_cgemm call fails with EMU_ERR_CUDA ("unspecified launch
  * failure") after the scan and split were enqueued, and C is not written;
@@ -165,7 +166,9 @@ const char *emu_last_cuda_error(void);
  * layouts: three residue sets per operand for the Scheme II 3M method, the
  * real embedding plus the slices of the 2K-deep product for Scheme I 4M).
  * For Scheme I this is what the bf16 engine uses; a smaller workspace that
- * still holds the INT8 slices makes the call run on the INT8 kernel. */
+ * still holds the INT8 slices makes the call run on the INT8 kernel, and so
+ * does a device without room for the library's own (which is then tried again
+ * after some tens of calls). */
 emu_status_t emu_workspace_size(emu_scheme_t scheme, int64_t m, int64_t n, int64_t k, int p_or_nm,
                                 int is_complex, size_t *bytes_host);
 
@@ -178,7 +181,10 @@ emu_status_t emu_workspace_size(emu_scheme_t scheme, int64_t m, int64_t n, int64
  * enough for the call (after an uncaptured call of the same shape, or with
  * a caller-owned workspace); a call that would have to grow the
  * library-owned workspace while its stream is capturing returns
- * EMU_ERR_ALLOC and enqueues nothing.  emu_dgemm_host, emu_dgemm_auto(_II)
+ * EMU_ERR_ALLOC and enqueues nothing.  Library-owned workspace that a capture
+ * used stays allocated until emu_destroy, also when later calls grow past it
+ * or this function replaces it, so that graphs can be replayed as long as the
+ * handle lives.  emu_dgemm_host, emu_dgemm_auto(_II)
  * and emu_get_status synchronise and cannot be captured. */
 emu_status_t emu_set_workspace(emu_handle_t h, void *workspace_dev, size_t bytes);
 

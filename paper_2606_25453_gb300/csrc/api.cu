@@ -356,7 +356,8 @@ static emu_status_t tmap_err() {
 
 namespace emu {
 // EMU_FAULT: host-side fault injection (read once).  alloc: every
-// library-owned workspace allocation fails; launch: the fused GEMM launch of
+// library-owned workspace allocation fails, alloc:N every one of more than N
+// bytes; launch: the fused GEMM launch of
 // every product, zero, scan, norm or split: every launch of that step before
 // it.  A launch fails as a launch would (cudaErrorLaunchFailure); nothing runs
 // on the device that could fault.
@@ -368,43 +369,52 @@ static int fault_mode() {
     int x = 0;
     for (int i = FAULT_ALLOC; e && i <= FAULT_SPLIT; ++i)
       if (std::strcmp(e, names[i]) == 0) x = i;
+    if (e && std::strncmp(e, "alloc:", 6) == 0) x = FAULT_ALLOC;
     v = x;
   }
   return v;
 }
-static bool fault_alloc() { return fault_mode() == FAULT_ALLOC; }
+static bool fault_alloc(size_t bytes) {
+  static const size_t most = [] {
+    const char* e = std::getenv("EMU_FAULT");
+    return e && std::strncmp(e, "alloc:", 6) == 0 ? static_cast<size_t>(std::strtoull(e + 6, nullptr, 10)) : 0;
+  }();
+  return fault_mode() == FAULT_ALLOC && bytes > most;
+}
 cudaError_t fault_step(FaultStep step) { return fault_mode() == step ? cudaErrorLaunchFailure : cudaSuccess; }
 static cudaError_t fault_launch() { return fault_step(FAULT_GEMM); }
 
-emu_status_t handle_workspace(emu_handle_s* h, size_t bytes, cudaStream_t st, uint8_t** out) {
-  if (bytes == 0) bytes = 256;
-  if (!h->ws_user && bytes > h->ws_bytes && fault_alloc()) return EMU_ERR_ALLOC;
+namespace {
+struct StreamMem {
+  cudaStream_t st;
+  bool capturing() const {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+  }
+  void* alloc(size_t n) const {
+    void* p = nullptr;
+    if (fault_alloc(n)) return nullptr;
+    if (cudaMallocAsync(&p, n, st) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+  void release(void* p) const { cudaFreeAsync(p, st); }
+};
+struct SyncMem {  // after a device synchronisation
+  void release(void* p) const { cudaFree(p); }
+};
+}  // namespace
+
+emu_status_t handle_workspace(emu_handle_s* h, size_t bytes, cudaStream_t st, uint8_t** out, bool optional) {
   if (h->ws_user) {
-    if (bytes > h->ws_bytes) return EMU_ERR_ALLOC;
-    *out = static_cast<uint8_t*>(h->ws);
+    if (bytes > h->ws_user_bytes) return EMU_ERR_ALLOC;
+    *out = static_cast<uint8_t*>(h->ws_user);
     return EMU_OK;
   }
-  if (bytes > h->ws_bytes) {
-    // no growth inside a stream capture: the memory would belong to the
-    // graph, and the handle would keep using it after the capture
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-      cudaGetLastError();
-      return EMU_ERR_ALLOC;
-    }
-    if (h->ws) cudaFreeAsync(h->ws, st);
-    h->ws = nullptr;
-    h->ws_bytes = 0;
-    size_t want = bytes + bytes / 8;
-    if (cudaMallocAsync(&h->ws, want, st) != cudaSuccess) {
-      h->ws = nullptr;
-      cudaGetLastError();
-      return EMU_ERR_ALLOC;
-    }
-    h->ws_bytes = want;
-  }
-  *out = static_cast<uint8_t*>(h->ws);
-  return EMU_OK;
+  StreamMem mem{st};
+  return ws_reserve(h->ws, bytes, optional, mem, out) ? EMU_OK : EMU_ERR_ALLOC;
 }
 }  // namespace emu
 
@@ -442,7 +452,8 @@ emu_status_t emu_destroy(emu_handle_t h) {
   cudaSetDevice(h->device);
   cudaDeviceSynchronize();
   handle_release_extras(h);
-  if (h->ws && !h->ws_user) cudaFree(h->ws);
+  SyncMem mem;
+  ws_close(h->ws, mem);
   if (h->status) cudaFree(h->status);
   delete h;
   return EMU_OK;
@@ -497,13 +508,13 @@ int emu_scale_bits_II(int nm, int64_t k, int is_complex) { return host_scale_bit
 emu_status_t emu_set_workspace(emu_handle_t h, void* ws, size_t bytes) {
   if (!h) return EMU_ERR_INVALID_ARG;
   cudaSetDevice(h->device);
-  if (h->ws && !h->ws_user) {
+  if (h->ws.p) {
     cudaDeviceSynchronize();
-    cudaFree(h->ws);
+    SyncMem mem;
+    if (!ws_drop(h->ws, mem)) return EMU_ERR_ALLOC;
   }
-  h->ws = ws;
-  h->ws_bytes = ws ? bytes : 0;
-  h->ws_user = ws != nullptr;
+  h->ws_user = ws;
+  h->ws_user_bytes = ws ? bytes : 0;
   if (ws && (reinterpret_cast<uintptr_t>(ws) & 255u)) return EMU_ERR_INVALID_ARG;
   return EMU_OK;
 }
@@ -803,7 +814,7 @@ emu_status_t run_scheme_I(emu_handle_s* h, const View& v, int64_t k, int p, doub
   if (tri > 0) {
     const size_t need = plan_tri(tri, v.N, k, p).bytes;
     uint8_t* tws = ws_override;
-    if (tws ? need <= ws_limit : handle_workspace(h, need, st, &tws) == EMU_OK)
+    if (tws ? need <= ws_limit : handle_workspace(h, need, st, &tws, true) == EMU_OK)
       return run_tri<T>(h, v, k, p, alpha, beta, C, ldc, out_mode, st, tws, tri, 0);
   }
   Plan pl = plan_I(v.M, v.N, k, p);

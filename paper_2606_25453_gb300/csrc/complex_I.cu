@@ -142,7 +142,7 @@ emu_status_t run_complex_I(emu_handle_s* h, emu_layout_t layout, int64_t M, int6
   // the whole of what emu_workspace_size says, or (a caller's smaller
   // workspace, a capture, full memory) the INT8 kernel's share
   size_t total = workspace_complex_I(M, N, K, p, f8);
-  emu_status_t s = handle_workspace(h, total, st, &ws);
+  emu_status_t s = handle_workspace(h, total, st, &ws, !f8);
   if (s != EMU_OK && !f8) {
     total = total - workspace_I(M, 2 * N, 2 * K, p, false) + plan_I(M, 2 * N, 2 * K, p).bytes;
     s = handle_workspace(h, total, st, &ws);

@@ -6,14 +6,15 @@
 #include <cuda_runtime.h>
 
 #include "../../include/emugemm.h"
+#include "workspace.h"
 
 struct emu_handle_s {
   int device = 0;
   int num_sms = 0;
   int* status = nullptr;  // device status word (bit flags, see emu_device.cuh)
-  void* ws = nullptr;     // workspace
-  size_t ws_bytes = 0;
-  bool ws_user = false;   // caller-owned workspace
+  emu::Workspace ws;      // library-owned workspace
+  void* ws_user = nullptr;  // caller-owned workspace, used in its place
+  size_t ws_user_bytes = 0;
   void* grouped = nullptr;   // grouped-GEMM plan cache (grouped.cu)
   void* selector = nullptr;  // selector state (select.cu)
   void* trace = nullptr;     // per-phase timing state (trace.cu), null when off
@@ -67,7 +68,7 @@ void normalize(emu_layout_t layout, int64_t m, int64_t n, const void* A, int64_t
                int64_t ldb, View* v);
 bool check_lds(emu_layout_t layout, int64_t m, int64_t n, int64_t k, int64_t lda, int64_t ldb, int64_t ldc);
 
-emu_status_t handle_workspace(emu_handle_s* h, size_t bytes, cudaStream_t st, uint8_t** out);
+emu_status_t handle_workspace(emu_handle_s* h, size_t bytes, cudaStream_t st, uint8_t** out, bool optional = false);
 
 // Argument checks shared by the emulated GEMM entry points; sets the
 // handle's device (api.cu).

@@ -170,7 +170,7 @@ emu_status_t host_gemm(emu_handle_s* h, HostIO* io, const View& v, int64_t k, do
         copy_rows(C_host, ldc, dC, N, 0, M, N, cudaMemcpyDeviceToHost, cs) != cudaSuccess)
       return EMU_ERR_CUDA;
   } else if (uint8_t* tws = nullptr; scheme == EMU_SCHEME_I && tri_rows(R, N, k, p) == R &&
-             handle_workspace(h, plan_tri(R, N, k, p).bytes, st, &tws) == EMU_OK) {
+             handle_workspace(h, plan_tri(R, N, k, p).bytes, st, &tws, true) == EMU_OK) {
     // Scheme I on the bf16 tensor cores: B's scan and split once, then each
     // chunk of A on a workspace laid out for R rows
     View vb{R, N, dA, std::max<int64_t>(k, 1), true, dB, N, false};

@@ -148,9 +148,6 @@ extern "C" emu_status_t emu_dgemm_noalloc(emu_layout_t layout, int64_t m, int64_
   cudaGetDevice(&hs.device);
   hs.num_sms = num_sms;
   hs.status = status_dev;
-  hs.ws = nullptr;
-  hs.ws_bytes = 0;
-  hs.ws_user = true;
   return run_scheme_I<double>(&hs, v, k, p, alpha, beta, C, ldc, OUT_F64, nullptr,
                               static_cast<cudaStream_t>(stream), scratch, false, kScratchBytes);
 }
