@@ -12,7 +12,13 @@ namespace emu {
 // First statement of a kernel that launch_after() starts, before it touches
 // global memory: the grid may be placed before the memory of the kernel ahead of
 // it on the stream is settled, and waits here until that kernel has completed
-// and its writes are visible.  Nothing in other launches.  No kernel lets the
+// and its writes are visible.  Nothing in other launches.  What a kernel
+// before it in the same call wrote is read with plain or .cg loads, never through
+// the read-only path (__ldg, const __restrict__): that path is for data nobody
+// writes while the grid exists, and here the grid can exist before the writer
+// has ended.  The caller's A and B may take it: the first kernel of a call
+// starts a new kernel only once it has itself waited for the caller's work.
+// No kernel lets the
 // next be placed earlier than its own end (griddepcontrol.launch_dependents):
 // blocks placed while others drain crowd the SMs that finish first, which cost
 // the residue split of n = 1000 7 us of 28.

@@ -216,7 +216,7 @@ __device__ __forceinline__ void load_pairs(const uint8_t* p, int64_t plane, int 
   uint32_t w[2 * MAXP];
 #pragma unroll
   for (int l = 0; l < 2 * MAXP; ++l)
-    w[l] = l < nm ? __ldg(reinterpret_cast<const uint32_t*>(p + static_cast<int64_t>(l) * plane)) : 0u;
+    w[l] = l < nm ? __ldcg(reinterpret_cast<const uint32_t*>(p + static_cast<int64_t>(l) * plane)) : 0u;
 #pragma unroll
   for (int i = 0; i < MAXP; ++i) {
     t01[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5140u);

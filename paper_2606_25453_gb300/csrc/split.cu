@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ NormO
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cw = op.cw;
   const int64_t r = op.kcontig ? bx * 8 + warp : bx * 32 + lane;
   // a zero vector adds nothing; a non-finite one was flagged by the scan
-  const uint64_t mb = r < op.rows ? op.maxbits[r] : 0ull;
+  const uint64_t mb = r < op.rows ? __ldcg(op.maxbits + r) : 0ull;
   const bool live = mb != 0 && mb < 0x7FF0000000000000ull;
   const int Emax = live ? frexp_exp_bits(mb) : 0;
   unsigned __int128 sum = 0;
@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ NormO
 __device__ __forceinline__ int exp_from_norm(const unsigned long long* acc, const unsigned long long* maxbits,
                                              int64_t r, int64_t rows) {
   if (r >= rows) return 0;
-  const unsigned long long lo = acc[2 * r], hi = acc[2 * r + 1];
-  const uint64_t mb = maxbits[r];
+  const unsigned long long lo = __ldcg(acc + 2 * r), hi = __ldcg(acc + 2 * r + 1);
+  const uint64_t mb = __ldcg(maxbits + r);
   if ((lo | hi) == 0 || mb >= 0x7FF0000000000000ull) return 0;
   const int L = hi ? 128 - __clzll(static_cast<long long>(hi)) : 64 - __clzll(static_cast<long long>(lo));
   const int d = L - 64;
@@ -333,7 +333,7 @@ __device__ __forceinline__ int exp_from_norm(const unsigned long long* acc, cons
 template <typename T, int P, bool F8>
 __global__ void split_I_kcontig(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                 int64_t rows_pad, int64_t nchunks,
-                                const unsigned long long* __restrict__ maxbits,
+                                const unsigned long long* maxbits,
                                 int8_t* __restrict__ hat, int32_t* __restrict__ E_out, bool vec) {
   const int lane = threadIdx.x & 31;
   const int64_t ngroups = (nchunks + 3) / 4;
@@ -365,7 +365,7 @@ __global__ void split_I_kcontig(const T* __restrict__ X, int64_t ld, int64_t row
 template <typename T, int P, bool F8>
 __global__ void __launch_bounds__(256) split_I_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                         int64_t rows_pad, int64_t nchunks,
-                                                        const unsigned long long* __restrict__ maxbits,
+                                                        const unsigned long long* maxbits,
                                                         int8_t* __restrict__ hat, int32_t* __restrict__ E_out,
                                                         bool vec) {
   __shared__ uint64_t tile[32][133];
@@ -598,7 +598,7 @@ __device__ __forceinline__ void residues4(const ModTables& mt, int nm, int shift
 template <typename T, int CW, bool BF, int ND>
 __global__ void split_II_kcontig(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k, int64_t rows_pad,
                                  int64_t kpad, int nm, int b, const __grid_constant__ ModTables mt,
-                                 const unsigned long long* __restrict__ maxbits, const unsigned long long* __restrict__ acc,
+                                 const unsigned long long* maxbits, const unsigned long long* acc,
                                  int8_t* __restrict__ res, int32_t* __restrict__ E_out, bool vec) {
   grid_begin();
   const int lane = threadIdx.x & 31;
@@ -629,8 +629,8 @@ template <typename T, int CW, bool BF, int ND, bool SMALL>
 __global__ void __launch_bounds__(256) split_II_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                          int64_t rows_pad, int64_t kpad, int nm, int b,
                                                          const __grid_constant__ ModTables mt,
-                                                         const unsigned long long* __restrict__ maxbits,
-                                                         const unsigned long long* __restrict__ acc, int8_t* __restrict__ res,
+                                                         const unsigned long long* maxbits,
+                                                         const unsigned long long* acc, int8_t* __restrict__ res,
                                                          int32_t* __restrict__ E_out, bool vec) {
   grid_begin();
   constexpr int TR = SMALL ? 8 : CW == 2 ? 16 : 32;  // vectors per tile (two tiles for complex)

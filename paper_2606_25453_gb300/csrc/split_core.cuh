@@ -29,7 +29,7 @@ __device__ __forceinline__ void slice_digits(uint64_t bits, int E, uint32_t* out
 __device__ __forceinline__ int exp_from_maxbits(const unsigned long long* maxbits, int64_t r,
                                                 int64_t rows) {
   if (r >= rows) return 0;
-  uint64_t mb = maxbits[r];
+  uint64_t mb = __ldcg(maxbits + r);
   if (mb >= 0x7FF0000000000000ull) return 0;  // non-finite: flagged by the scan
   return frexp_exp_bits(mb);
 }

@@ -19,7 +19,7 @@ namespace {
 template <typename T, int P>
 __global__ void __launch_bounds__(256) split_tri_kcontig(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                          int64_t kpad, int per, int64_t nseg,
-                                                         const unsigned long long* __restrict__ maxbits,
+                                                         const unsigned long long* maxbits,
                                                          uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
                                                          int32_t* __restrict__ sums, bool vec) {
   grid_begin();
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) split_tri_kcontig(const T* __restrict__ X
 template <typename T, int P, int TR>
 __global__ void __launch_bounds__(256, P <= 8 ? 4 : 2) split_tri_kstrided(const T* __restrict__ X, int64_t ld, int64_t rows, int64_t k,
                                                           int64_t kpad, int per,
-                                                          const unsigned long long* __restrict__ maxbits,
+                                                          const unsigned long long* maxbits,
                                                           uint16_t* __restrict__ planes, int32_t* __restrict__ E_out,
                                                           int32_t* __restrict__ sums, bool vec) {
   grid_begin();

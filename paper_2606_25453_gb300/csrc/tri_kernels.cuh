@@ -219,7 +219,7 @@ __device__ __forceinline__ void combine_patch(const KParamsTriComb& kp, int bloc
     int4 v[O::planes];
 #pragma unroll
     for (int u = 0; u < O::planes; ++u)
-      v[u] = live ? __ldg(reinterpret_cast<const int4*>(src + static_cast<int64_t>(u) * kp.nkc * plane))
+      v[u] = live ? __ldcg(reinterpret_cast<const int4*>(src + static_cast<int64_t>(u) * kp.nkc * plane))
                   : make_int4(0, 0, 0, 0);
     if (kc == 0) {  // the row and column terms while the planes are on their way
       if (threadIdx.x < kCombRows) {
