@@ -190,10 +190,6 @@ struct GemmTriArgs {
   int* status;
   int num_sms;
 };
-// Load the kernels of every p (the runtime otherwise loads a kernel at its
-// first launch, about 20 us each).
-void preload_tri();
-void preload_split_tri();
 cudaError_t launch_gemm_I_tc(int p, int out_mode, const GemmTriArgs& a, cudaStream_t st, int part);
 template <typename T>
 [[nodiscard]] cudaError_t launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,

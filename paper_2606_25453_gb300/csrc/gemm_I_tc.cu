@@ -92,23 +92,7 @@ cudaError_t launch_combine(const KParamsTriComb& kp, bool one, cudaStream_t st) 
              : launch_after(combine_I_kernel<P, false>, grid, 256, st, kp);
 }
 
-template <int P>
-void preload_p() {
-  cudaFuncAttributes a;
-  cudaFuncGetAttributes(&a, combine_I_kernel<P, false>);
-  cudaFuncGetAttributes(&a, combine_I_kernel<P, true>);
-  if constexpr (P < kTriMaxP) preload_p<P + 1>();
-}
-
 }  // namespace
-
-void preload_tri() {
-  cudaFuncAttributes a;
-  cudaFuncGetAttributes(&a, gemm_I_tc_kernel);
-  preload_p<1>();
-  preload_split_tri();
-  cudaGetLastError();
-}
 
 int tri_tile_m() { return kBM; }
 int tri_tile_n() { return kBN; }

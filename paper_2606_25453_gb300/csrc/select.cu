@@ -605,7 +605,6 @@ emu_status_t emu_sel_load(emu_handle_t h, const float* params) {
   if (cudaMemcpy(s->params, params, sizeof(float) * kNParam, cudaMemcpyHostToDevice) != cudaSuccess)
     return EMU_ERR_CUDA;
   s->loaded = true;
-  preload_tri();  // any p may be chosen: no kernel is loaded inside a call
   return EMU_OK;
 }
 

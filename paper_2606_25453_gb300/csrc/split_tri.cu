@@ -137,18 +137,7 @@ cudaError_t launch_p(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t
   }
 }
 
-template <int P>
-void preload_p() {
-  cudaFuncAttributes a;
-  cudaFuncGetAttributes(&a, split_tri_kcontig<double, P>);
-  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P, 8>);
-  cudaFuncGetAttributes(&a, split_tri_kstrided<double, P, 32>);
-  if constexpr (P < kTriMaxP) preload_p<P + 1>();
-}
-
 }  // namespace
-
-void preload_split_tri() { preload_p<1>(); }
 
 template <typename T>
 cudaError_t launch_split_tri(const T* X, int64_t ld, bool kcontig, int64_t rows, int64_t k, int p,

@@ -187,6 +187,40 @@ def test_training_II_beats_fixed_nm(h):
     assert code == 0 and nm in sel.NM_CLASSES
 
 
+CHILD_INSTALL = r"""
+import ctypes, sys, time
+import numpy as np
+sys.path.insert(0, %r)
+import torch
+import paper_2606_25453_gb300 as emu
+h = emu.Handle(0)
+w = np.zeros(8968, dtype=np.float32).ctypes.data_as(ctypes.POINTER(ctypes.c_float))
+t = []
+for load in (emu.emu_sel_load_II, emu.emu_sel_load):
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    emu.check(load(h.h, w))
+    t.append(time.perf_counter() - t0)
+print(t[1] - t[0])
+"""
+
+
+def test_installing_a_network_does_no_other_work():
+    """Installing the Scheme I network costs what installing the Scheme II
+    one does (one small copy): kernels are loaded by the calls that launch
+    them, not by emu_sel_load (all of them took 2 ms)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    extra = []
+    for _ in range(3):  # a kernel is loaded once per process
+        r = subprocess.run([sys.executable, "-c", CHILD_INSTALL % root], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr
+        extra.append(float(r.stdout))
+    assert min(extra) < 1e-3, extra
+
+
 def test_committed_selector_end_to_end_gain_at_1e8():
     """The committed Scheme I network, timed end to end through
     emu_dgemm_auto -- feature scan, MLP, probe and every escalation inside
