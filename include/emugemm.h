@@ -416,20 +416,26 @@ typedef struct {
 } emu_gemm_desc_t;
 
 /* `count` independent Scheme I products with p slices (row-major, the
- * descriptors are host memory).  Each product falls into a shape bucket (p
- * and log2 classes of sqrt(m n) and of k) and runs in that bucket's tuned
- * configuration: output tiles of 64 x 32, 32 x 32 or 32 x 64 and the
- * triangle's slice pairs B-slice-major or A-slice-major (64 x 32,
+ * descriptors are host memory), as one CUDA graph that is captured once and
+ * replayed while the descriptors stay identical.  Up to eight slices the batch
+ * runs on the bf16 tensor cores: one grouped exponent scan, one grouped split,
+ * one persistent GEMM launch over the (product, unit, tile) work list and one
+ * combine launch.  More slices, a batch that would need more than 32 GiB of
+ * workspace or whose workspace cannot be had, and EMU_I_ENGINE=mma run on the
+ * INT8 mma.sync kernels, with the same results.  There each product falls into
+ * a shape bucket (p and log2 classes of sqrt(m n) and of k) and runs in that
+ * bucket's tuned configuration: output tiles of 64 x 32, 32 x 32 or 32 x 64
+ * and the triangle's slice pairs B-slice-major or A-slice-major (64 x 32,
  * B-slice-major where the handle holds no tuning).  The products are
  * ordered by GEMM work per operand element and cut into up to three stages
  * (at 15 % and 50 % of the batch's GEMM work; one stage below 8 products).
  * Per stage: one grouped exponent scan, one grouped split, then one
  * persistent grouped GEMM launch per configuration in use over its
  * (problem, tile) work list, balanced longest-first over the CTAs.  Each
- * stage's GEMM launches run on parallel branches of one CUDA graph beside
- * the next stages' scan and split; the graph is captured once and replayed
- * while the descriptors and tunings stay identical.  The paper has no
- * batched interface; the tile model follows Table I. */
+ * stage's GEMM launches run on parallel branches of the graph beside
+ * the next stages' scan and split; that graph is captured again when the
+ * tunings change.  The paper has no batched interface; the tile model
+ * follows Table I. */
 emu_status_t emu_dgemm_grouped(emu_handle_t h, int count, const emu_gemm_desc_t *descs_host, int p,
                                emu_stream_t stream);
 
@@ -437,8 +443,10 @@ emu_status_t emu_dgemm_grouped(emu_handle_t h, int count, const emu_gemm_desc_t 
 emu_status_t emu_dgemm_grouped_loop(emu_handle_t h, int count, const emu_gemm_desc_t *descs_host,
                                     int p, emu_stream_t stream);
 
-/* Autotune the configuration per shape bucket on this problem list (data
- * as given).  A configuration is a tile shape (64 x 32, 32 x 32 or 32 x 64
+/* Autotune the configuration per shape bucket of the INT8 mma.sync kernels on
+ * this problem list (data as given).  A batch that emu_dgemm_grouped runs on
+ * the bf16 tensor cores uses no configuration: it neither gains nor loses by
+ * a tuning.  A configuration is a tile shape (64 x 32, 32 x 32 or 32 x 64
  * outputs per CTA) and a slice-pair order of the triangle of Eq. (2)
  * (B-slice-major or A-slice-major): indices 0-2 are the three shapes in
  * B-slice-major order, 3-5 the same shapes A-slice-major.  Tuned twice,

@@ -416,9 +416,9 @@ GroupState* state_of(emu_handle_s* h) {
 
 bool same_plan(const GroupPlan* pl, const emu_gemm_desc_t* b, int count, int p, const std::vector<int>& pcfg,
                int stages, bool tri) {
-  if (!pl || pl->p != p || (pl->want_tri != tri) || pl->max_stages != stages || static_cast<int>(pl->descs.size()) != count ||
-      pl->pcfg != pcfg)
-    return false;
+  if (!pl || pl->p != p || pl->want_tri != tri || static_cast<int>(pl->descs.size()) != count) return false;
+  // tile configurations and stages are the mma.sync kernels'
+  if (!pl->tri && (pl->max_stages != stages || pl->pcfg != pcfg)) return false;
   return std::memcmp(pl->descs.data(), b, sizeof(emu_gemm_desc_t) * count) == 0;
 }
 

@@ -67,3 +67,67 @@ def test_more_than_eight_slices_mixed_configurations(orc, tmp_path, p):
     shapes = [tuple(int(x) for x in rng.integers((20, 20, 60), (500, 500, 900))) for _ in range(12)]
     check(orc, h, shapes, p, 70)
     h.close()
+
+
+@pytest.mark.parametrize("p", [9])
+def test_one_stage_of_the_mma_kernels(orc, tmp_path, p):
+    # three stages by default (the test above), here one
+    path = tmp_path / "one.json"
+    lines = ['  "p%d_s%d_k%d": %d' % (p, sc, kc, (2 * sc + kc) % 6) for sc in range(5) for kc in range(5)]
+    path.write_text("{\n" + ",\n".join(lines + ['  "p%d_stages": 1' % p]) + "\n}\n")
+    h = emu.Handle(0)
+    emu.check(emu.emu_load_tuning(h.h, str(path).encode()))
+    rng = np.random.Generator(np.random.PCG64(4))
+    shapes = [tuple(int(x) for x in rng.integers((20, 20, 60), (500, 500, 900))) for _ in range(12)]
+    check(orc, h, shapes, p, 170)
+    h.close()
+
+
+def test_tuned_batch_of_nine_slices_is_bit_exact(orc, tmp_path):
+    # nine slices run on the mma.sync kernels that the tuner times
+    p = 9
+    mats = [synth.gemm_pair(m, n, k, 1.0, 270 + i) for i, (m, n, k) in enumerate([(60, 200, 300), (250, 40, 100)] * 5)]
+    As, Bs = [torch.from_numpy(A).cuda() for A, _ in mats], [torch.from_numpy(B).cuda() for _, B in mats]
+    Cs = [torch.full((A.shape[0], B.shape[1]), float("nan"), dtype=torch.float64, device="cuda") for A, B in mats]
+    d = emu.grouped_descs(As, Bs, Cs)
+    h = emu.Handle(0)
+    path = str(tmp_path / "tune.json")
+    assert emu.tune_grouped(d, p, path=path, handle=h) > 0
+    h2 = emu.Handle(0)
+    emu.check(emu.emu_load_tuning(h2.h, path.encode()))
+    for hd in (h, h2):
+        for C in Cs:
+            C.fill_(float("nan"))
+        emu.dgemm_grouped(d, p, handle=hd)
+        torch.cuda.synchronize()
+        assert hd.status() == 0
+        for (A, B), C in zip(mats, Cs):
+            assert np.array_equal(C.cpu().numpy(), orc.emu_I(A, B, p))
+    h.close()
+    h2.close()
+
+
+def test_tuning_leaves_a_bf16_plan_alone(tmp_path):
+    """A tuning concerns the mma.sync kernels: loading one must not make the
+    next call of a batch on the bf16 engine synchronise the device and build
+    its plan again."""
+    A, B = synth.gemm_pair(300, 200, 500, 1.0, 6)
+    As, Bs = [torch.from_numpy(A).cuda()] * 4, [torch.from_numpy(B).cuda()] * 4
+    Cs = [torch.empty((300, 200), dtype=torch.float64, device="cuda") for _ in As]
+    d = emu.grouped_descs(As, Bs, Cs)
+    h = emu.Handle(0)
+    emu.dgemm_grouped(d, 6, handle=h)
+    ref = Cs[0].clone()
+    torch.cuda.synchronize()
+    path = tmp_path / "t.json"
+    path.write_text("{\n" + ",\n".join('  "p6_s%d_k%d": 3' % (i, j) for i in range(5) for j in range(5)) +
+                    ',\n  "p6_stages": 1\n}\n')
+    emu.check(emu.emu_load_tuning(h.h, str(path).encode()))
+    done = torch.cuda.Event()
+    torch.cuda._sleep(200_000_000)  # about 0.1 s of a busy stream
+    emu.dgemm_grouped(d, 6, handle=h)
+    done.record()
+    assert not done.query()  # a rebuild would have waited for the device
+    torch.cuda.synchronize()
+    assert torch.equal(Cs[0], ref)
+    h.close()
