@@ -54,12 +54,21 @@ struct KParamsIITC {
   int* status;
 };
 
-// A multiple of m_l added to (or removed from) an exact int32 sum, keeping
-// its residue: x = hi 2^16 + lo -> hi (2^16 mod m) + lo, |result| < 2^22.1
-// (p16: the symmetric residue of 2^16 mod m, |p16| <= 128).
+// Segments (|sum| <= 2^24 each) between folds of the int32 sums, the largest
+// sum that is folded then, and what a fold leaves of it.
+constexpr int kFold = 64;
+constexpr int64_t kSumMax = (int64_t{kFold} << 24) + (int64_t{1} << 22);
+constexpr int64_t kFoldMax = ((kSumMax >> 16) + 1) * 128 + 0xFFFF;
+
+// A multiple of m_l added to (or removed from) an exact int32 sum |x| <=
+// kSumMax, keeping its residue: x = hi 2^16 + lo -> hi (2^16 mod m) + lo,
+// |result| <= kFoldMax < 2^21.1 (p16: the symmetric residue of 2^16 mod m,
+// |p16| <= 128).
+static_assert(kSumMax < INT32_MAX && kFoldMax < (int64_t{1} << 22) && kFoldMax < 2580000,
+              "folded sums stay in int32, and within what mod4 takes");
 __device__ __forceinline__ int fold16(int x, int p16) { return (x >> 16) * p16 + (x & 0xFFFF); }
 
-// Residues in [0, m) of four sums |x| <= 2^21.3 (fold16's output), one byte
+// Residues in [0, m) of four sums |x| <= 2^21.3 (2.58e6; fold16's output is smaller), one byte
 // each, in FP32 arithmetic without conversions or corrections: with x / m =
 // n + j / m, y = x / m + 1 / (2m) - 1/2 lies 1 / (2m) >= 0.0019 inside
 // (n - 1/2, n + 1/2), and its computed value errs by less than 2^-10 (inv by
@@ -118,7 +127,6 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1)
     // drain: exact integer sums of this thread's columns over the segments;
     // only the final sum is reduced mod m
     constexpr int kC = bf16g::kDrainCols;
-    constexpr int kFold = 64;  // segments (|sum| < 2^24 each) per fold of the int32 sums
     const int c0 = (c.warp >> 2) * kC, row = (c.warp & 3) * 32 + c.lane;
     const uint32_t addr = bf16g::drain_addr(c);
     uint32_t seg = 0;
@@ -150,7 +158,7 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1)
             for (int x = 0; x < 16; ++x) run[16 * q + x] += __float2int_rn(__uint_as_float(v[x]));
           }
         }
-        // fold every 64 segments, so that the int32 sums never overflow, whatever K is
+        // fold every kFold segments, so that the int32 sums never overflow, whatever K is
         if (s % kFold == kFold - 1) {
 #pragma unroll
           for (int x = 0; x < kC; ++x) run[x] = fold16(run[x], p16);
