@@ -147,16 +147,6 @@ __device__ __forceinline__ void mma_e4m3(float* d, const uint32_t* a, const uint
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// E4M3 byte of an integer v with |v| <= 16 (exact): sign, exponent
-// floor(log2 |v|) + 7, three mantissa bits.
-__device__ __forceinline__ uint32_t e4m3_of_int(int v) {
-  uint32_t a = static_cast<uint32_t>(v < 0 ? -v : v);
-  if (a == 0) return 0u;
-  int e = 31 - __clz(static_cast<int>(a));
-  uint32_t mant = ((a << 3) >> e) & 7u;
-  return (v < 0 ? 0x80u : 0u) | (static_cast<uint32_t>(e + 7) << 3) | mant;
-}
-
 // Byte offset inside a [rows][32 B] block written by TMA with 32-byte
 // swizzling: the 16-byte half `chunk` of row `row` is stored at
 // chunk ^ ((row >> 2) & 1).

@@ -267,9 +267,6 @@ cudaError_t launch_p(const GemmIArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-int gemm_I_tile_m() { return kBM; }
-int gemm_I_tile_n() { return kBN; }
-
 cudaError_t launch_gemm_I(int p, int out_mode, const GemmIArgs& a, cudaStream_t st, bool f8) {
 #define EMU_P(PP)                                                                       \
   case PP:                                                                              \

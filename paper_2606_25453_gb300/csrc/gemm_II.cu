@@ -282,8 +282,6 @@ cudaError_t launch_mode(const GemmIIArgs& a, const ModTables& mt, const CrtTable
 
 }  // namespace
 
-int gemm_II_kchunk() { return kKS * 32; }
-
 cudaError_t launch_gemm_II(int out_mode, const GemmIIArgs& a, const ModTables& mt,
                            const CrtTables& ct, cudaStream_t st) {
   switch (out_mode) {

@@ -408,9 +408,6 @@ cudaError_t launch_tc(const GemmIArgs& a, cudaStream_t st, bool partials) {
 
 }  // namespace
 
-int gemm_f8tc_tile_m() { return kBM; }
-int gemm_f8tc_tile_n() { return kBN; }
-
 cudaError_t launch_gemm_f8tc(int p, int out_mode, const GemmIArgs& a, cudaStream_t st) {
 #define EMU_TC(PP)                                                \
   case PP:                                                        \
