@@ -77,6 +77,23 @@ def test_extreme_digits(orc, a):
         run(orc, A, B, p)
 
 
+# digit sums at -256 over whole 256-deep segments with one -255 in each, on
+# both sides: every segment's FP32 sum ends at 2^24 - 511, an odd integer
+# beside the end of the exact range (constant operands give even sums only)
+@pytest.mark.parametrize("p", [3, 4, 6])
+def test_odd_sums_beside_2_24(orc, p):
+    k = 1024
+    rng = np.random.Generator(np.random.PCG64(p))
+    low = -(2.0 ** (8 * p - 1)) + 1  # leading digit -128, bytes 0 .. 0 1: digits -128, .., -128, -127
+    A, B = np.full((140, k), low), np.full((k, 270), low)
+    for seg in range(0, k, 256):
+        at = seg + int(rng.integers(256))
+        A[:, at] += 2.0 ** (8 * (p - 2))  # second byte 1: digit sum -255
+        B[at, :] += 2.0 ** (8 * (p - 2))
+    assert 255 * 65536 + 255 * 255 == 2 ** 24 - 511
+    run(orc, A, B, p)
+
+
 def test_one_plane_per_group_and_row_strides(orc):
     # enough tiles that each group of digit sums shares one output plane
     A, B = synth.gemm_pair(1300, 2200, 130, 0.5, 77)
