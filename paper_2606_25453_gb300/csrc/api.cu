@@ -763,14 +763,17 @@ emu_status_t run_tri(emu_handle_s* h, const View& v, int64_t k, int p, double al
     a.L = tri_layout(rows, v.N, k, p);  // the workspace's layout, for fewer rows in the last pass
     a.L.tiles_m = (m + tri_tile_m() - 1) / tri_tile_m();
     const uint64_t row_bytes = 2 * static_cast<uint64_t>(a.L.kpad);
+    // boxes no higher than the product (in steps of the 8-row swizzle atoms
+    // and of the 32 columns that the MMAs compute)
+    const auto box_a = static_cast<uint32_t>(std::min<int64_t>((m + 7) / 8 * 8, tri_tile_m()));
+    const auto box_b = static_cast<uint32_t>(std::min<int64_t>((v.N + 31) / 32 * 32, tri_tile_n()));
     CUtensorMap ta, tb;
-    if (!make_tmap_i8(&ta, planesA, row_bytes, static_cast<uint64_t>(m) * np, static_cast<uint32_t>(tri_tile_m()),
-                      128) ||
-        !make_tmap_i8(&tb, planesB, row_bytes, static_cast<uint64_t>(v.N) * np,
-                      static_cast<uint32_t>(tri_tile_n()), 128))
+    if (!make_tmap_i8(&ta, planesA, row_bytes, static_cast<uint64_t>(m) * np, box_a, 128) ||
+        !make_tmap_i8(&tb, planesB, row_bytes, static_cast<uint64_t>(v.N) * np, box_b, 128))
       return tmap_err();
     a.descA = &ta;
     a.descB = &tb;
+    a.box_bytes = static_cast<int>((box_a + box_b) * 128);
     a.M = static_cast<int>(m);
     a.N = static_cast<int>(v.N);
     a.K = k;

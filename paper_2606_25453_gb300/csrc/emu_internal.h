@@ -177,6 +177,7 @@ struct GemmTriArgs {
   TriLayout L;
   const CUtensorMap* descA;
   const CUtensorMap* descB;
+  int box_bytes;  // of one 64-deep chunk: the rows of both maps' boxes x 128 bytes
   int M, N;
   int64_t K;
   int32_t* Cs;

@@ -25,12 +25,13 @@ namespace emu {
 namespace {
 
 struct KParamsTri {
-  CUtensorMap tA;  // planes as bytes: 128-byte x 128-row boxes, 128-byte swizzle
-  CUtensorMap tB;  // 128-byte x 256-row boxes
+  CUtensorMap tA;  // planes as bytes: 128-byte x 128-row boxes (fewer if M is less), 128-byte swizzle
+  CUtensorMap tB;  // 128-byte x 256-row boxes (fewer if N is less)
   TriPlan tp;
   int nst, kcs, nkc;  // 64-deep chunks of a plane; chunks per K range; K ranges
   int tiles_m, tiles_n;  // 128-row and 256-column tiles
   int M, N;  // rows of A's planes and of B's
+  int box_bytes;
   int32_t* Cs;  // output planes, tile by tile (tri_elem)
   int* status;
 };
@@ -62,7 +63,7 @@ struct TriWork {
   }
   __device__ __forceinline__ const CUtensorMap* tA(const bf16g::Item&) const { return &kp.tA; }
   __device__ __forceinline__ const CUtensorMap* tB(const bf16g::Item&) const { return &kp.tB; }
-  __device__ __forceinline__ int bytes(const bf16g::Item&) const { return bf16g::Cfg<false>::kChunkBytes; }
+  __device__ __forceinline__ int bytes(const bf16g::Item&) const { return kp.box_bytes; }
   // where this item's sums go
   __device__ __forceinline__ int32_t* tile_of(const bf16g::Item& t) const {
     const int64_t plane = static_cast<int64_t>(kp.tp.unit[t.unit].out) * kp.nkc + t.aux;
@@ -148,6 +149,7 @@ cudaError_t launch_gemm_I_tc(int p, int out_mode, const GemmTriArgs& a, cudaStre
     kp.tiles_n = tiles_n;
     kp.M = a.M;
     kp.N = a.N;
+    kp.box_bytes = a.box_bytes;
     kp.Cs = a.Cs;
     kp.status = a.status;
     const int64_t nitems = static_cast<int64_t>(tp.nunits) * nkc * tiles_m * tiles_n;

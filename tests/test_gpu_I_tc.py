@@ -148,3 +148,13 @@ def test_engine_switch_gives_the_same_bits(orc, tmp_path):
     assert r.returncode == 0, r.stderr
     assert np.array_equal(np.load(out), orc.emu_I(A, B, 8))
     run(orc, A, B, 8)
+
+
+# products narrower than a tile: boxes and combine blocks follow M in steps of
+# 8 and 32 rows, N in steps of 32 columns
+@pytest.mark.parametrize("m,n", [(1, 300), (300, 1), (8, 32), (9, 33), (121, 31), (136, 64), (33, 250), (127, 255)])
+def test_narrow_products(orc, m, n):
+    A, B = synth.gemm_pair(m, n, 200, 1.0, 10 * m + n)
+    C0 = synth.test_matrix(m, n, 1.0, m + n)
+    for p in (2, 8):
+        run(orc, A, B, p, alpha=-0.5, beta=2.0, C0=C0)
