@@ -87,8 +87,7 @@ __global__ void __launch_bounds__(256) combine_I_kernel(const __grid_constant__ 
 // ---------------------------------------------------------------- plan
 template <int P>
 cudaError_t launch_combine(const KParamsTriComb& kp, bool one, cudaStream_t st) {
-  const unsigned grid =
-      static_cast<unsigned>(kp.tiles_m * kp.tiles_n * (kBN / kCombCols) * (kBM / kCombRows));
+  const unsigned grid = static_cast<unsigned>(kp.tiles_m * kp.tiles_n * kp.pr * kp.pc);
   return one ? launch_after(combine_I_kernel<P, true>, grid, 256, st, kp)
              : launch_after(combine_I_kernel<P, false>, grid, 256, st, kp);
 }
@@ -164,6 +163,8 @@ cudaError_t launch_gemm_I_tc(int p, int out_mode, const GemmTriArgs& a, cudaStre
   kc.tiles_n = tiles_n;
   kc.M = a.M;
   kc.N = a.N;
+  kc.pr = patch_rows(a.M);
+  kc.pc = patch_cols(a.N);
   kc.sumA = a.sumA;
   kc.sumB = a.sumB;
   tri_const(p, a.K, &kc.const_lo, &kc.const_hi);

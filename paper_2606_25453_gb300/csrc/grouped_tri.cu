@@ -191,6 +191,8 @@ __global__ void __launch_bounds__(256, P == 8 && !ONE ? 2 : 0) grouped_combine_k
   kp.tiles_n = pr.tiles_n;
   kp.M = pr.M;
   kp.N = pr.N;
+  kp.pr = patch_rows(pr.M);
+  kp.pc = patch_cols(pr.N);
   kp.sumA = pr.sumA;
   kp.sumB = pr.sumB;
   kp.const_lo = pr.const_lo;
@@ -226,7 +228,6 @@ Share share_of(const emu_gemm_desc_t& d, int p, bool one) {
 
 // A batch's workspace beyond this keeps the mma.sync kernels (a fifth of it).
 constexpr size_t kGroupTriBytes = size_t{32} << 30;
-constexpr int kPatches = (kBM / kCombRows) * (kBN / kCombCols);
 
 bool batch_one(int count, const emu_gemm_desc_t* d, int p) {
   int64_t tiles = 0;
@@ -278,7 +279,7 @@ emu_status_t group_tri_build(emu_handle_s* h, int count, const emu_gemm_desc_t* 
     const int64_t nrun = ((L.kpad + 127) / 128 + kSplitRun - 1) / kSplitRun;
     sA[i + 1] = sA[i] + static_cast<int>((d[i].m + 7) / 8 * nrun);
     sB[i + 1] = sB[i] + static_cast<int>((d[i].n + 31) / 32 * nrun);
-    sC[i + 1] = sC[i] + static_cast<int>(L.tiles_m * L.tiles_n * kPatches);
+    sC[i + 1] = sC[i] + static_cast<int>(L.tiles_m * L.tiles_n * patch_rows(d[i].m) * patch_cols(d[i].n));
     for (int u = 0; u < tp.nunits; ++u) {
       const int64_t cols = std::min<int64_t>((d[i].n + 31) / 32 * 32, kBN);
       runs.push_back({tp.unit[u].count * L.kcs * (kBM + cols), i, u});
