@@ -16,8 +16,9 @@
  *     digits and sums of two of them are exact bf16 values, their FP32 sums
  *     stay exact integers, and the triangle needs one product per pair i < j
  *     and per digit (24 instead of 36 at p = 8).  The INT8 mma.sync kernel
- *     gives the same result and serves p > 8 below 2^33 multiply-adds,
- *     workspaces that only hold its slices, and EMU_I_ENGINE=mma.
+ *     gives the same result and serves p > 8 below 2^33 multiply-adds, long
+ *     and narrow products of short K (where its few bytes count more than the
+ *     products), workspaces that only hold its slices, and EMU_I_ENGINE=mma.
  *
  *   Scheme II (Sec. II-C-2, Eqs. 4-8; fused kernel of Sec. IV-A)
  *     A and B are scaled to integers, reduced modulo N pairwise-coprime
@@ -420,7 +421,8 @@ typedef struct {
  * replayed while the descriptors stay identical.  Up to eight slices the batch
  * runs on the bf16 tensor cores: one grouped exponent scan, one grouped split,
  * one persistent GEMM launch over the (product, unit, tile) work list and one
- * combine launch.  More slices, a batch that would need more than 32 GiB of
+ * combine launch.  More slices, batches of many small products with K below
+ * about 64, a batch that would need more than 32 GiB of
  * workspace or whose workspace cannot be had, and EMU_I_ENGINE=mma run on the
  * INT8 mma.sync kernels, with the same results.  There each product falls into
  * a shape bucket (p and log2 classes of sqrt(m n) and of k) and runs in that

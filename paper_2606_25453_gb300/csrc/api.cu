@@ -611,16 +611,39 @@ constexpr int64_t kTriMaxK = int64_t{1} << 20;
 constexpr int kTriSmallP = 8;
 constexpr int64_t kTriLargeWork = int64_t{1} << 33;
 
-bool tri_takes(int64_t m, int64_t n, int64_t k, int p) {
+bool tri_can(int64_t m, int64_t n, int64_t k, int p) {
   if (!i_engine_tc() || k < 1 || k > kTriMaxK) return false;
-  if (p > kTriSmallP && static_cast<double>(m) * static_cast<double>(n) * static_cast<double>(k) < kTriLargeWork)
-    return false;
   // plane rows are TMA coordinates (int32)
   return (m > n ? m : n) <= INT32_MAX / tri_num_planes(p) / 2;
 }
 
+// Long and narrow products of short K: what counts is not the products but
+// the bf16 planes (46 bytes per operand element at p = 8, the INT8 slices 8)
+// and the int32 planes of 32 columns at least, written and read again.  From
+// 20 items per SM on (smaller products are bound by their launches) INT8
+// mma.sync against bf16 planes, us, 262144 rows:
+//   p = 8: 8 columns, K = 32 383 / 659, 64 512 / 663, 128 771 / 807, 256 1383
+//          / 1340; 32 columns, K = 64 580 / 702, 128 829 / 843; 64 columns,
+//          K = 32 709 / 872, 64 958 / 872; 128 columns, K = 32 1218 / 1255
+//   p = 4: 8 columns, K = 64 292 / 380, 128 367 / 414; 32 columns, K = 64 369 /
+//          399, 128 452 / 430; 64 columns, K = 32 491 / 496
+//   p = 3: 8 columns, K = 64 258 / 282, 128 312 / 312; 16 columns, K = 64 309 / 285
+//   p = 2: 8 columns, K = 32 219 / 231, 64 233 / 231
+// and short and wide: p = 8, 8 x 262144, K = 32 464 / 542, 64 722 / 563; 32 x
+// 262144, K = 32 542 / 585; p = 6, 8 x 262144, K = 32 370 / 429; p = 4 292 / 312.
+static bool tri_pays(int64_t m, int64_t n, int64_t k, int p) {
+  if (p > kTriSmallP && static_cast<double>(m) * static_cast<double>(n) * static_cast<double>(k) < kTriLargeWork)
+    return false;
+  if (p < 3 || (m + tri_tile_m() - 1) / tri_tile_m() * ((n + tri_tile_n() - 1) / tri_tile_n()) * tri_num_units(p) <
+                   20 * 152)
+    return true;
+  const int64_t k32 = (k + 31) / 32 * 32;
+  if (n <= 64 && k32 * std::max<int64_t>(n, 16) <= 2048 && (p > 3 || n <= 8)) return false;
+  return !(p >= 6 && m <= 8 && k <= 32);
+}
+
 int64_t tri_rows(int64_t m, int64_t n, int64_t k, int p) {
-  if (!tri_takes(m, n, k, p)) return 0;
+  if (!tri_can(m, n, k, p) || !tri_pays(m, n, k, p)) return 0;
   auto pass = [&](int64_t rows) {
     const TriLayout L = tri_layout(rows, n, k, p);
     return static_cast<int64_t>(L.Cs_bytes) + 2 * static_cast<int64_t>(tri_num_planes(p)) * rows * L.kpad;

@@ -40,8 +40,8 @@ struct PlanTri {
   size_t off_EA, off_FB, off_planesA, off_planesB, off_Cs, bytes;
 };
 PlanTri plan_tri(int64_t rows, int64_t n, int64_t k, int p);
-// Whether a product may take the bf16 tensor cores (engine, K, p), workspace aside.
-bool tri_takes(int64_t m, int64_t n, int64_t k, int p);
+// Whether a product can take the bf16 tensor cores (engine, K, sizes), workspace aside.
+bool tri_can(int64_t m, int64_t n, int64_t k, int p);
 // Workspace of a real Scheme I product on either engine.
 size_t workspace_I(int64_t m, int64_t n, int64_t k, int p, bool f8);
 // Rows of A per pass, 0 if the product does not take this path (see api.cu).

@@ -173,6 +173,7 @@ void tri_const(int p, int64_t K, uint64_t* lo, uint64_t* hi);
 int tri_tile_m();
 int tri_tile_n();
 int tri_num_planes(int p);
+int tri_num_units(int p);  // int32 output planes with one unit per group
 struct GemmTriArgs {
   TriLayout L;
   const CUtensorMap* descA;

@@ -101,6 +101,8 @@ int tri_num_planes(int p) {
   return counts.n[p];
 }
 
+int tri_num_units(int p) { return plan_of(p, false).nunits; }
+
 void tri_const(int p, int64_t K, uint64_t* lo, uint64_t* hi) {
   // 2^14 K sum_{i,j>=1, i+j<p} 256^(p-1-i-j): s - 1 pairs with i + j = s
   unsigned __int128 w = 0;

@@ -237,11 +237,40 @@ bool batch_one(int count, const emu_gemm_desc_t* d, int p) {
 
 }  // namespace
 
+// Batches of many small products of short K: each of their tiles is an item
+// with its own chain of table loads, TMA and drain whatever it holds, and
+// their int32 planes cost more than their products.  INT8 mma.sync against
+// bf16 planes, us, `count` products of n x n x K:
+//   p = 8, 3000: n = 32, K = 32 533 / 844, 64 603 / 862, 256 1309 / 1560; n = 64,
+//     K = 32 880 / 1389, 64 1094 / 1422, 256 2625 / 2490; n = 128, K = 32 2287 /
+//     3015, 64 3003 / 3090; 512: n = 256, K = 32 1345 / 1506, 64 1807 / 1518
+//   p = 6, 3000: n = 32, K = 64 508 / 640, 256 1060 / 1075; n = 128, K = 32 1838 /
+//     2294, 64 2284 / 2330; 512: n = 16, K = 64 101 / 86; 64: n = 64, K = 32 47 / 43
+//   p = 4, 3000: n = 64, K = 32 657 / 719, 64 744 / 737; n = 16, K = 32 397 / 335
+// K is the mean over the outputs; the fill is the mean outputs per 128 x 256
+// tile; the lines in items per SM are where the fixed cost of a launch ends.
+static bool group_tri_pays(int count, const emu_gemm_desc_t* d, int p) {
+  double outs = 0.0, ks = 0.0;
+  int64_t tiles = 0;
+  for (int i = 0; i < count; ++i) {
+    const double o = static_cast<double>(d[i].m) * static_cast<double>(d[i].n);
+    outs += o;
+    ks += o * static_cast<double>((d[i].k + 31) / 32 * 32);
+    tiles += ((d[i].m + kBM - 1) / kBM) * ((d[i].n + kBN - 1) / kBN);
+  }
+  if (tiles == 0 || outs == 0.0) return true;
+  const double k = ks / outs, fill = outs / static_cast<double>(tiles);
+  const int64_t items = tiles * plan_of(p, false).nunits;
+  if (k > 64.0) return true;
+  return fill < 500.0 ? items < 200 * kSms : p < 5 || items < 30 * kSms || k * fill > 1048576.0;
+}
+
 bool group_tri_takes(int count, const emu_gemm_desc_t* d, int p) {
   size_t bytes = 0;
+  if (!group_tri_pays(count, d, p)) return false;
   const bool one = batch_one(count, d, p);
   for (int i = 0; i < count; ++i) {
-    if (!tri_takes(d[i].m, d[i].n, d[i].k, p)) return false;
+    if (!tri_can(d[i].m, d[i].n, d[i].k, p)) return false;
     const Share s = share_of(d[i], p, one);
     bytes += s.zero + s.rest;
     if (s.L.nkc > 255 || bytes > kGroupTriBytes) return false;

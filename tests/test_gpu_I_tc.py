@@ -158,3 +158,32 @@ def test_narrow_products(orc, m, n):
     C0 = synth.test_matrix(m, n, 1.0, m + n)
     for p in (2, 8):
         run(orc, A, B, p, alpha=-0.5, beta=2.0, C0=C0)
+
+
+# both sides of every line between the bf16 engine and the INT8 kernel for
+# long, narrow products of short K (and short, wide ones): rows for 20 items
+# per SM, columns times K, the single columns of three slices
+@pytest.mark.parametrize("m,n,k,p,layout,bf16", [
+    (26000, 8, 32, 8, "row", False), (25000, 8, 32, 8, "row", True), (26000, 8, 128, 8, "row", False),
+    (26000, 8, 129, 8, "row", True), (26000, 64, 32, 8, "row", False), (26000, 65, 32, 8, "row", True),
+    (26000, 33, 63, 8, "row", True), (26000, 32, 63, 7, "row", True), (31000, 32, 63, 7, "row", False), (8, 26000, 40, 8, "col", False),
+    (7, 52000, 32, 8, "row", False), (9, 52000, 32, 8, "row", True), (7, 52000, 33, 8, "row", True),
+    (97300, 8, 64, 3, "row", False), (97300, 9, 64, 3, "row", True), (97300, 3, 64, 2, "row", True)])
+def test_engine_lines_of_narrow_products(orc, m, n, k, p, layout, bf16):
+    A, B = synth.gemm_pair(m, n, k, 1.0, m + n + k)
+    h = emu.Handle(0)
+    Ad, Bd = (dev(A), dev(B)) if layout == "row" else (dev(A.T).t(), dev(B.T).t())
+    C = torch.empty((m, n), dtype=torch.float64, device="cuda") if layout == "row" else \
+        torch.empty((n, m), dtype=torch.float64, device="cuda").t()
+    h.trace(True)
+    h.trace_read()
+    emu.dgemm(Ad, Bd, C, scheme="I", p=p, handle=h)
+    t = h.trace_read()
+    h.trace(False)
+    assert h.status() == 0
+    assert (t["ms_other"] > 0.0) == bf16  # the combine kernel is the bf16 engine's
+    h.close()
+    rows = np.unique(np.linspace(0, m - 1, 700).astype(int))
+    cols = np.unique(np.linspace(0, n - 1, 700).astype(int))
+    want = orc.emu_I(np.ascontiguousarray(A[rows]), np.ascontiguousarray(B[:, cols]), p)
+    assert np.array_equal(C.cpu().numpy()[np.ix_(rows, cols)], want)

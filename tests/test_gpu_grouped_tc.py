@@ -131,3 +131,27 @@ def test_tuning_leaves_a_bf16_plan_alone(tmp_path):
     torch.cuda.synchronize()
     assert torch.equal(Cs[0], ref)
     h.close()
+
+
+# both sides of the lines between the engines for batches of many small
+# products of short K: items per SM, mean K, fill
+@pytest.mark.parametrize("count,n,k,p,bf16", [
+    (320, 32, 32, 8, False), (300, 32, 32, 8, True), (320, 32, 65, 8, True), (160, 200, 64, 8, True),
+    (160, 150, 40, 8, False), (320, 32, 32, 4, True), (2100, 16, 32, 8, False), (2000, 16, 32, 8, True)])
+def test_engine_lines_of_small_products(orc, count, n, k, p, bf16):
+    rng = np.random.Generator(np.random.PCG64(count + n))
+    A = torch.from_numpy(rng.standard_normal((count, n, k))).cuda()
+    B = torch.from_numpy(rng.standard_normal((count, k, n))).cuda()
+    C = torch.full((count, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    h = emu.Handle(0)
+    h.trace(True)
+    h.trace_read()
+    emu.dgemm_grouped(emu.grouped_descs(list(A), list(B), list(C)), p, handle=h)
+    t = h.trace_read()
+    h.trace(False)
+    assert h.status() == 0
+    h.close()
+    # scan, split, GEMM, combine; else three stages of scan, split and GEMMs
+    assert (t["kernel_launches"] == 4) == bf16, t
+    for i in (0, 1, count // 2, count - 1):
+        assert np.array_equal(C[i].cpu().numpy(), orc.emu_I(A[i].cpu().numpy(), B[i].cpu().numpy(), p)), i
