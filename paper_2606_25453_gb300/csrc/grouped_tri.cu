@@ -40,7 +40,9 @@ constexpr int kSplitRun = 8;  // groups of 128 elements along K per split block
 // costs is each block's chain of dependent loads (product, table entry,
 // exponent, elements), hence several groups per block: the batch above took
 // 4.59 ms with one group per block and a binary search for the product, 4.01
-// with this and the search by whole warps.
+// with this and the search by whole warps.  Blocks per SM: what the compiler
+// reaches by itself, and at p = 6 three instead of two (80 registers for 97; that
+// batch 3.95 ms against 4.26).
 template <int P>
 __global__ void __launch_bounds__(256, P <= 4 ? 4 : P <= 6 ? 3 : 2) grouped_split_tri_kernel(const GTriProb* __restrict__ probs, int count,
                                                                    const int* __restrict__ startA,
@@ -179,6 +181,10 @@ __global__ void __launch_bounds__(bf16g::kThreads, 1) gemm_I_grouped_tc_kernel(c
   tri_gemm(GTriWork{kp}, kp.status);
 }
 
+// Two blocks per SM at p = 8 with one plane per group, where the compiler would
+// take 152 registers for one (512 products, M, N <= 1024, K <= 2048: 5.63 ms
+// against 6.19); below it reaches two by itself, and with one plane per pair
+// (small batches) 128 registers spill.
 template <int P, bool ONE>
 __global__ void __launch_bounds__(256, P == 8 && !ONE ? 2 : 0) grouped_combine_kernel(const GTriProb* __restrict__ probs, int count,
                                                               const int* __restrict__ startC) {
