@@ -603,11 +603,14 @@ constexpr int64_t kTriPassBytes = int64_t{8} << 30;
 constexpr int64_t kTriMaxK = int64_t{1} << 20;
 
 // More than eight slices (FP64 accuracy needs eight; the rest serves wide
-// exponent ranges) take this path only from 2^33 multiply-adds.  It would be
-// the faster one below as well (n = 1344, p = 12: 0.41 ms against 2.61), but
-// then the largest p costs no more than a chosen one plus the choice (about
-// 45 us a call), and emu_dgemm_auto has to gain over the fixed largest p at
-// n = 1024 .. 1536: it does by 2.1x with this rule, by 1.02-1.07 without.
+// exponent ranges) take this path only from 2^33 multiply-adds.  This line is
+// not where it stops paying: it is faster below as well (n = 1344, p = 12: 0.41
+// ms against 2.61).  But then the largest p costs little more than a chosen one
+// plus the choice, whose waits for the device are 30 to 50 us of a call of 220
+// to 350, and emu_dgemm_auto is to gain 1.05x over the fixed largest p at n =
+// 1024 .. 1536: it does by 1.47x with this line, by 1.02-1.03x without (1.04-1.06
+// with the probe's sums enqueued before the product instead of behind it).  It
+// can go when the automatic call costs some 20 us less.
 constexpr int kTriSmallP = 8;
 constexpr int64_t kTriLargeWork = int64_t{1} << 33;
 
