@@ -541,7 +541,7 @@ def run_ours(args, rank, world, local_rank):
                 "config": config(args, world),
                 "int8_tops": (int8_ops * args.steps * world / (ms * 1e-3) / 1e12) if not ii_tc else None,
                 "int8_frac_of_peak": ((int8_ops * args.steps / (ms * 1e-3) / 1e12 / int8_peak)
-                                      if int8_peak and args.scheme != "I_F8" and not ii_tc else None),
+                                      if int8_peak and args.scheme != "I_F8" and not ii_tc and not i_tc else None),
                 "roofline": {"bound": "tensor",
                              "kernel": kname,
                              "achieved": achieved,
@@ -597,7 +597,8 @@ def suite_markdown(paths):
     o.append("1 warm-up + 3 timed calls per point, 1 at n = 16384 and for ZGEMM; accuracy = -log2 of")
     o.append("max |C - C_ref| / (|A||B|) on 8 x 64 sampled entries against the library's double-double probe")
     o.append("kernel, emu_probe_dd).")
-    o.append("Slice-product rates count executed products x 2: Scheme I p(p+1)MNK (8-bit), Scheme II 2 N_m MNK and 3M")
+    o.append("Slice-product rates count the method's products x 2: Scheme I p(p+1)MNK (8-bit; the bf16 engine forms fewer,")
+    o.append("products of digits and of digit sums, so its rate can exceed any INT8 peak), Scheme II 2 N_m MNK and 3M")
     o.append("6 N_m MNK (residue products; bf16 on the default tcgen05 engine, INT8 on the mma.sync engine).")
     o.append("Measured INT8 peak of this GPU: 150-156 TOP/s (cuBLASLt INT8 GEMM; register-only mma.sync s8 loop")
     o.append("150.9).  bf16 peak: %.1f TFLOP/s (MEASURED_PEAKS.json); FP8 tensor peak: %.0f TFLOP/s (that x 2, the"
@@ -662,11 +663,12 @@ def suite_markdown(paths):
             o.append(f"| emu_cgemm | {d['scheme']} ({'3M' if d['scheme']=='II' else '4M'}) | {d['p_or_nm']} | {d['tflops_8mnk']:.2f} | {bits(d['err'])} |")
     o.append("\n## Naive (INT32 partials to HBM + separate shift-reduce) vs fused, n = 4096, k <= K_c\n")
     o.append("`emu_partials_I` / `emu_partials_F8` + `emu_shift_reduce_I` against `emu_dgemm` (results")
-    o.append("bit-identical).\n")
+    o.append("bit-identical).  The 8-bit partials come from the INT8 mma.sync kernel, `emu_dgemm` runs 8-bit slices on")
+    o.append("the bf16 engine: that row compares the two, the E4M3 row one kernel with and without its epilogue.\n")
     o.append("| slices | p | naive ms | fused ms | fused speedup | INT32 partials bytes |\n|---|---|---|---|---|---|")
     for d in rows:
         if d["path"] == "ablation_naive_vs_fused":
-            o.append(f"| {'E4M3 (tcgen05)' if d['slices'] == 'e4m3' else 'INT8 (mma.sync)'} | {d['p']} | {d['ms_naive']:.2f} | "
+            o.append(f"| {'E4M3 (tcgen05)' if d['slices'] == 'e4m3' else '8-bit'} | {d['p']} | {d['ms_naive']:.2f} | "
                      f"{d['ms_fused']:.2f} | {d['speedup_fused']:.2f} | {d['int32_partials_bytes']} |")
     # Fig. 7 analogue: precision, throughput and workspace of every real DGEMM
     # path at n = 8192, phi = 0.5 (workspace from the library's size query,
@@ -685,7 +687,7 @@ def suite_markdown(paths):
             if d.get("n") != 8192 or d.get("phi") != 0.5:
                 continue
             if d["path"] == "emu_dgemm_I":
-                pts.append(("Scheme I, INT8 (mma.sync)", "p = %d" % d["p"], d, ws_gb(emu.EMU_SCHEME_I, d["p"])))
+                pts.append(("Scheme I, 8-bit slices (bf16 tcgen05)", "p = %d" % d["p"], d, ws_gb(emu.EMU_SCHEME_I, d["p"])))
             elif d["path"] == "emu_dgemm_I_F8":
                 pts.append(("Scheme I, E4M3 (tcgen05)", "p = %d" % d["p"], d, ws_gb(emu.EMU_SCHEME_I_F8, d["p"])))
             elif d["path"] == "emu_dgemm_II":
@@ -701,10 +703,12 @@ def suite_markdown(paths):
     o.append("\n## Grouped: 512 uneven products, one CUDA graph vs per-product loop\n")
     for d in rows:
         if d["path"] == "emu_dgemm_grouped":
-            o.append(f"p = {d['p']}: graph (tuned) {d['ms_graph_tuned']:.2f} ms, untuned (64 x 32, B-slice-major) "
-                     f"{d['ms_graph_default_tile']:.2f} ms, loop {d['ms_loop']:.2f} ms: "
-                     f"{d['speedup_graph_vs_loop']:.2f}x; {d['tflops_graph']:.2f} emulated TFLOP/s, "
-                     f"{d['int8_tops_graph']:.1f} INT8 TOP/s.")
+            graph = (f"graph {d['ms_graph']:.2f} ms on the bf16 engine" if d["engine"] == "bf16" else
+                     f"graph (tuned) {d['ms_graph']:.2f} ms, untuned (64 x 32, B-slice-major) "
+                     f"{d['ms_graph_default_tile']:.2f} ms on the INT8 kernels")
+            o.append(f"p = {d['p']}: {graph}, loop {d['ms_loop']:.2f} ms: "
+                     f"{d['speedup_graph_vs_loop']:.2f}x; {d['tflops_graph']:.2f} emulated TFLOP/s" +
+                     (f", {d['int8_tops_graph']:.1f} INT8 TOP/s." if "int8_tops_graph" in d else "."))
             if d.get("tuned"):
                 hist = {}
                 for v in d["tuned"].values():
@@ -721,8 +725,9 @@ GROUPED_CFGS = ("64x32 B-major", "32x32 B-major", "32x64 B-major",
 
 def grouped_points(emu, h, dev, emit, timed):
     """512 uneven products (M, N log-uniform in [32, 1024], K in [64, 2048]):
-    the grouped CUDA graph untuned and after the autotuner, against the
-    per-product loop, at p = 6 and p = 10."""
+    the grouped CUDA graph against the per-product loop at p = 6 (bf16 engine,
+    which uses no tuning) and p = 10 (INT8 mma.sync kernels, untuned and after
+    the autotuner)."""
     import tempfile
 
     import torch
@@ -736,27 +741,28 @@ def grouped_points(emu, h, dev, emit, timed):
     d = emu.grouped_descs(As, Bs, Cs)
     flops = sum(2 * m * nn * k for m, nn, k in shapes)
     for p in (6, 10):
-        ms_default = timed(lambda: emu.dgemm_grouped(d, p, handle=h), reps=5)
-        with tempfile.TemporaryDirectory() as td:
-            path = os.path.join(td, "tune.json")
-            ncfg = emu.tune_grouped(d, p, path=path, handle=h)
-            with open(path) as fh:
-                tuned = json.load(fh)
-        ms_tuned = timed(lambda: emu.dgemm_grouped(d, p, handle=h), reps=5)
+        ms = timed(lambda: emu.dgemm_grouped(d, p, handle=h), reps=5)
+        row = {"path": "emu_dgemm_grouped", "count": 512, "p": p, "engine": "bf16" if p <= 8 else "int8"}
+        if p > 8:
+            with tempfile.TemporaryDirectory() as td:
+                path = os.path.join(td, "tune.json")
+                row["configs_timed"] = emu.tune_grouped(d, p, path=path, handle=h)
+                with open(path) as fh:
+                    tuned = json.load(fh)
+            row["ms_graph_default_tile"], ms = ms, timed(lambda: emu.dgemm_grouped(d, p, handle=h), reps=5)
+            row["tuned"] = {k: GROUPED_CFGS[v] for k, v in sorted(tuned.items())
+                            if k.startswith("p%d_s" % p) and not k.endswith("_stages")}
+            row["stages"] = tuned.get("p%d_stages" % p)
+            row["int8_tops_graph"] = (p * (p + 1) // 2) * flops / ms / 1e9
         ms_loop = timed(lambda: emu.dgemm_grouped(d, p, handle=h, loop=True), reps=2)
-        emit({"path": "emu_dgemm_grouped", "count": 512, "p": p, "ms_graph_default_tile": ms_default,
-              "ms_graph_tuned": ms_tuned, "configs_timed": ncfg, "ms_loop": ms_loop,
-              "tuned": {k: GROUPED_CFGS[v] for k, v in sorted(tuned.items())
-                        if k.startswith("p%d_s" % p) and not k.endswith("_stages")},
-              "stages": tuned.get("p%d_stages" % p),
-              "tflops_graph": flops / ms_tuned / 1e9, "tflops_loop": flops / ms_loop / 1e9,
-              "int8_tops_graph": (p * (p + 1) // 2) * flops / ms_tuned / 1e9,
-              "speedup_graph_vs_loop": ms_loop / ms_tuned})
+        row.update({"ms_graph": ms, "ms_loop": ms_loop, "tflops_graph": flops / ms / 1e9,
+                    "tflops_loop": flops / ms_loop / 1e9, "speedup_graph_vs_loop": ms_loop / ms})
+        emit(row)
 
 
 def grouped_run(args):
-    """The 512-product grouped batch (the grouped_points shapes) at p = args.p,
-    untuned: args.warmup + args.steps graph launches, CUDA-event time of the
+    """The 512-product grouped batch (the grouped_points shapes) at p = args.p
+    (up to eight on the bf16 engine, beyond on the INT8 kernels, untuned): args.warmup + args.steps graph launches, CUDA-event time of the
     timed ones."""
     import torch
     import __graft_entry__
@@ -786,7 +792,8 @@ def grouped_run(args):
     ms = e0.elapsed_time(e1) / max(args.steps, 1)
     flops = sum(2 * m * nn * k for m, nn, k in shapes)
     print(json.dumps({"path": "emu_dgemm_grouped", "count": 512, "p": args.p, "ms": ms,
-                      "tflops": flops / ms / 1e9, "int8_tops": args.p * (args.p + 1) // 2 * flops / ms / 1e9}))
+                      "engine": "bf16" if args.p <= 8 else "int8", "tflops": flops / ms / 1e9,
+                      "int8_tops": args.p * (args.p + 1) // 2 * flops / ms / 1e9 if args.p > 8 else None}))
     h.close()
 
 
@@ -890,7 +897,7 @@ def selector_markdown(path):
          "committed weights -- feature",
          "scan, MLP, the 64-entry double-double probe and every escalation and recomputation inside the",
          "timed region -- against `emu_dgemm` at the fixed p (N) that passes every training product (Scheme I",
-         "INT8 p = 12; Scheme II with norm scaling N = 20).  Pass: max |C - AB| / (|A||B|) <= tol on 256",
+         "p = 12; Scheme II with norm scaling N = 20).  Pass: max |C - AB| / (|A||B|) <= tol on 256",
          "other sampled entries against the GPU double-double probe.\n",
          "| scheme | tol | products | fixed | mean chosen | auto pass | fixed pass | auto total ms | fixed total ms"
          " | speed-up |",
@@ -899,6 +906,15 @@ def selector_markdown(path):
         o.append("| %s | %.0e | %d | %d | %.2f | %.0f %% | %.0f %% | %.1f | %.1f | %.2fx |" % (
             d["scheme"], d["tol"], d["products"], d["fixed"], d["mean_used"], 100 * d["pass_auto"],
             100 * d["pass_fixed"], d["ms_auto_total"], d["ms_fixed_total"], d["speedup_vs_fixed"]))
+    # more than eight slices run on the INT8 kernel below 2^33 multiply-adds (n = 2048), at several times the cost
+    o.append("\nScheme I by the engine of the fixed arm (p > 8: the INT8 kernel below n = 2048, the bf16 engine from"
+             " there;\na chosen p <= 8 runs on the bf16 engine everywhere):\n")
+    o.append("| tol | n < 2048: auto / fixed ms | n >= 2048: auto / fixed ms | speed-up, n >= 2048 |\n|---|---|---|---|")
+    for tol in sorted({d["tol"] for d in pts if d["scheme"] == "I"}, reverse=True):
+        t = [[sum(d[k] for d in pts if d["scheme"] == "I" and d["tol"] == tol and (d["n"] >= 2048) == big)
+              for k in ("ms_auto", "ms_fixed")] for big in (False, True)]
+        if t[1][0]:
+            o.append("| %.0e | %.2f / %.2f | %.2f / %.2f | %.2fx |" % (tol, *t[0], *t[1], t[1][1] / t[1][0]))
     o.append("\nPer product (time in ms; chosen = the p or N of the returned result):\n")
     o.append("| scheme | n | phi | tol | chosen | ms auto | ms fixed | err auto | err fixed |")
     o.append("|---|---|---|---|---|---|---|---|---|")

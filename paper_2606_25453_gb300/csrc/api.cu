@@ -357,10 +357,9 @@ static emu_status_t tmap_err() {
 namespace emu {
 // EMU_FAULT: host-side fault injection (read once).  alloc: every
 // library-owned workspace allocation fails, alloc:N every one of more than N
-// bytes; launch: the fused GEMM launch of
-// every product, zero, scan, norm or split: every launch of that step before
-// it.  A launch fails as a launch would (cudaErrorLaunchFailure); nothing runs
-// on the device that could fault.
+// bytes; launch: the fused GEMM launch of every product, zero, scan, norm or
+// split: every launch of that step before it.  A launch fails as a launch would
+// (cudaErrorLaunchFailure); nothing runs on the device that could fault.
 static int fault_mode() {
   static int v = -1;
   if (v < 0) {

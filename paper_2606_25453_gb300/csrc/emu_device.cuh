@@ -16,12 +16,12 @@ namespace emu {
 // before it in the same call wrote is read with plain or .cg loads, never through
 // the read-only path (__ldg, const __restrict__): that path is for data nobody
 // writes while the grid exists, and here the grid can exist before the writer
-// has ended.  The caller's A and B may take it: the first kernel of a call
-// starts a new kernel only once it has itself waited for the caller's work.
-// No kernel lets the
-// next be placed earlier than its own end (griddepcontrol.launch_dependents):
-// blocks placed while others drain crowd the SMs that finish first, which cost
-// the residue split of n = 1000 7 us of 28.
+// has ended.  The caller's A and B may take it in every kernel but a call's
+// first, which here only zeroes: when the next is placed that one has ended, so
+// it has waited for all the caller's work.
+// No kernel lets the next be placed earlier than its own end
+// (griddepcontrol.launch_dependents): blocks placed while others drain crowd
+// the SMs that finish first, which cost the residue split of n = 1000 7 us of 28.
 __device__ __forceinline__ void grid_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------- status word

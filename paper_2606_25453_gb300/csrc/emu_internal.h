@@ -12,8 +12,9 @@ namespace emu {
 // Launch a kernel that begins with grid_begin() so that its launch and the end
 // of the kernel before it overlap: a small product is six or seven short
 // kernels, and what passed between them was a third of its time.  256^3, p = 7:
-// 32.8 -> 21.9 us per call; 2905 x 1777 x 803, 14 moduli, norm scaling: 278 ->
-// 260; 3001 x 2047 x 2500 complex64: 755 -> 742.
+// 32.8 -> 22 to 25 us per call (two modes of the host's launch rate); 2905 x
+// 1777 x 803, 14 moduli, norm scaling: 278 -> 260; 3001 x 2047 x 2500 complex64:
+// 755 -> 742.
 template <class... P, class... A>
 inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
