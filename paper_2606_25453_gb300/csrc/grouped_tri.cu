@@ -250,6 +250,7 @@ bool batch_one(int count, const emu_gemm_desc_t* d, int p) {
 //   p = 8, 3000: n = 32, K = 32 533 / 844, 64 603 / 862, 256 1309 / 1560; n = 64,
 //     K = 32 880 / 1389, 64 1094 / 1422, 256 2625 / 2490; n = 128, K = 32 2287 /
 //     3015, 64 3003 / 3090; 512: n = 256, K = 32 1345 / 1506, 64 1807 / 1518
+//   p = 8, n = 16, K = 32, 512 106 / 113, 3000 504 / 684
 //   p = 6, 3000: n = 32, K = 64 508 / 640, 256 1060 / 1075; n = 128, K = 32 1838 /
 //     2294, 64 2284 / 2330; 512: n = 16, K = 64 101 / 86; 64: n = 64, K = 32 47 / 43
 //   p = 4, 3000: n = 64, K = 32 657 / 719, 64 744 / 737; n = 16, K = 32 397 / 335
@@ -268,7 +269,8 @@ static bool group_tri_pays(int count, const emu_gemm_desc_t* d, int p) {
   const double k = ks / outs, fill = outs / static_cast<double>(tiles);
   const int64_t items = tiles * plan_of(p, false).nunits;
   if (k > 64.0) return true;
-  return fill < 500.0 ? items < 200 * kSms : p < 5 || items < 30 * kSms || k * fill > 1048576.0;
+  if (fill < 500.0) return items < (p < 7 ? 200 : 100) * kSms;
+  return p < 5 || items < 30 * kSms || k * fill > 1048576.0;
 }
 
 bool group_tri_takes(int count, const emu_gemm_desc_t* d, int p) {

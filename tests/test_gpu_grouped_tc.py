@@ -137,7 +137,8 @@ def test_tuning_leaves_a_bf16_plan_alone(tmp_path):
 # products of short K: items per SM, mean K, fill
 @pytest.mark.parametrize("count,n,k,p,bf16", [
     (320, 32, 32, 8, False), (300, 32, 32, 8, True), (320, 32, 65, 8, True), (160, 200, 64, 8, True),
-    (160, 150, 40, 8, False), (320, 32, 32, 4, True), (2100, 16, 32, 8, False), (2000, 16, 32, 8, True)])
+    (160, 150, 40, 8, False), (320, 32, 32, 4, True), (1100, 16, 32, 8, False), (1000, 16, 32, 8, True),
+    (2800, 16, 32, 6, False), (2700, 16, 32, 6, True)])
 def test_engine_lines_of_small_products(orc, count, n, k, p, bf16):
     rng = np.random.Generator(np.random.PCG64(count + n))
     A = torch.from_numpy(rng.standard_normal((count, n, k))).cuda()
